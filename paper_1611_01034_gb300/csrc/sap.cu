@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 #include "tm_stencil.cuh"
 
 namespace tmamg {
@@ -204,10 +205,28 @@ template void launch_sap_colour<float>(const float*, const float*, const float*,
 //   S = D_ee - D_eo D_oo^-1 D_oe  over the even sites,
 // with right-hand side r_e - D_eo D_oo^-1 r_o; afterwards
 //   e_o = D_oo^-1 (r_o - D_oe e_e).
-// One CTA owns one block and one right-hand side; thread j owns the j-th even
-// and the j-th odd site (same t, z, y; x = 2 j_x + parity offset), so no lane
-// idles in either half-step.  D_oo^-1 comes precomputed per odd site
-// (launch_clover_inverse).
+// D_oo^-1 comes precomputed per odd site (launch_clover_inverse).
+//
+// One CTA owns one block and one lane type R of right-hand sides (two at once
+// as packed FP32, or one); thread j owns the j-th even and the j-th odd site
+// (same t, z, y; x = 2 j_x + parity offset), so no lane idles in either
+// half-step.  The kernel waits on operator loads (L1 and L2) and issue, not on
+// DRAM: two right-hand sides per thread share every operator load, conversion
+// and link row and halve the instructions (823 M -> 497 M warp instructions
+// per 6-rhs launch at 48 x 24^3).  Their 255 registers leave two CTAs per SM;
+// a bound of 168 registers (three CTAs) spills and its shared memory takes the
+// L1 from the operator: 1.96 ms against 1.11 ms per launch (one right-hand
+// side per thread: 1.24 ms; lattice-ordered operator before: 1.50 ms).
+//
+// The kernel walks 2 n_MR + 3 half-steps, odd and even alternating, so that the
+// hop gather, D_oo^-1 and the site-diagonal term each appear once in the code
+// (the instruction cache holds the loop); H = the sum of the intra-block hops,
+// D_eo, D_oe = -H/2:
+//   step 0 (odd):            od = D_oo^-1 r_o; x_o += od
+//   step 1 (even):           rho = r_e + H od / 2
+//   step 2k (odd, k >= 1):   od = D_oo^-1 H rho
+//   step 2k+1 (even):        q = D_ee rho - H od / 4; MR update of e_e, rho
+//   step 2 n_MR + 2 (odd):   x_o += D_oo^-1 H e_e / 2; x_e += e_e
 // ===========================================================================
 namespace {
 
@@ -215,96 +234,60 @@ namespace {
 __device__ __forceinline__ int half_index(const int lc[4], const int blk[4]) {
   return ((lc[0] * blk[1] + lc[1]) * blk[2] + lc[2]) * (blk[3] / 2) + (lc[3] >> 1);
 }
-
-// acc += hops (Dirichlet, without the -1/2) from the neighbours of a site inside
-// the block, whose values of the other parity are in shared memory src [12][HB]
-template <typename T, int S>
-__device__ __forceinline__ void oe_block_hops(const cx<T>* __restrict__ src, int HB, const int lc[4],
-                                              const int blk[4], const void* __restrict__ gauge, const Lat& g, int s,
-                                              const int c[4], cx<T> (&acc)[12]) {
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = cx<T>{0, 0};
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    if (lc[mu] < blk[mu] - 1) {
-      int ln[4] = {lc[0], lc[1], lc[2], lc[3]};
-      ln[mu] += 1;
-      const int j = half_index(ln, blk);
-      cx<T> p[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) p[k] = src[k * HB + j];
-      switch (mu) {
-        case 0: hop_fwd_p<T, 0, S>(p, gauge, g.V, s, T(1), acc); break;
-        case 1: hop_fwd_p<T, 1, S>(p, gauge, g.V, s, T(1), acc); break;
-        case 2: hop_fwd_p<T, 2, S>(p, gauge, g.V, s, T(1), acc); break;
-        default: hop_fwd_p<T, 3, S>(p, gauge, g.V, s, T(1), acc); break;
-      }
-    }
-    if (lc[mu] > 0) {
-      int ln[4] = {lc[0], lc[1], lc[2], lc[3]};
-      ln[mu] -= 1;
-      const int j = half_index(ln, blk);
-      cx<T> p[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) p[k] = src[k * HB + j];
-      const int sb = nb_bwd(g, s, c, mu);
-      switch (mu) {
-        case 0: hop_bwd_p<T, 0, S>(p, gauge, g.V, sb, T(1), acc); break;
-        case 1: hop_bwd_p<T, 1, S>(p, gauge, g.V, sb, T(1), acc); break;
-        case 2: hop_bwd_p<T, 2, S>(p, gauge, g.V, sb, T(1), acc); break;
-        default: hop_bwd_p<T, 3, S>(p, gauge, g.V, sb, T(1), acc); break;
-      }
-    }
-  }
+// linear index of a block from its block coordinates
+__device__ __forceinline__ int block_linear(const SapGeom& sg, const int bc[4]) {
+  return ((bc[0] * sg.nb[1] + bc[1]) * sg.nb[2] + bc[2]) * sg.nb[3] + bc[3];
 }
 
-// y = D_oo^-1 p at odd site s: two general 6x6 complex blocks, 36 float4 /
-// double2-pair chunks per odd site, compact odd index s >> 1
-template <typename T, int S>
-__device__ __forceinline__ void apply_dinv(const void* __restrict__ dinv, long Vh, int s, const cx<T> (&p)[12],
-                                           cx<T> (&y)[12]) {
-  const long so = s >> 1;
+template <typename T, int NC, int S>
+__device__ __forceinline__ void ld_op(const void* __restrict__ base, long off, long V, long s, cx<T> (&z)[NC]) {
+  if constexpr (S == ST_NATIVE)
+    ld_cx<T, NC>(static_cast<const T*>(base) + off, V, s, z);
+  else
+    ld_cx16<T, S, NC>(static_cast<const unsigned short*>(base) + off, V, s, z);
+}
+
+// sums of 3 values over the CTA; red holds 3 values per warp, read by the next call only after a barrier
+template <class R>
+__device__ __forceinline__ void lanes_allreduce3(R (&v)[3], R* red) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int k = 0; k < 3; ++k) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      cx<T> m[6];
-      const long off = (long)(h * 6 + i) * 12 * Vh;  // row i of block h: 6 complex
-      if constexpr (S == ST_NATIVE)
-        ld_cx<T, 6>(static_cast<const T*>(dinv) + off, Vh, so, m);
+    for (int o = 16; o > 0; o >>= 1) {
+      if constexpr (LaneOf<R>::n == 2)
+        v[k] = v[k] + f2{__shfl_xor_sync(0xffffffffu, v[k].v, o)};
       else
-        ld_cx16<T, S, 6>(static_cast<const unsigned short*>(dinv) + off, Vh, so, m);
-      cx<T> acc = m[0] * p[6 * h];
-#pragma unroll
-      for (int j = 1; j < 6; ++j) cfma(acc, m[j], p[6 * h + j]);
-      y[6 * h + i] = acc;
+        v[k] = v[k] + __shfl_xor_sync(0xffffffffu, v[k], o);
     }
+  }
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) red[(threadIdx.x >> 5) * 3 + k] = v[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    R s = red[k];
+    for (int w = 1; w < (int)blockDim.x >> 5; ++w) s = s + red[w * 3 + k];
+    v[k] = s;
   }
 }
 
-// r = b - D x at site s (full operator, neighbours from global memory; b may be null)
-template <typename T, int S = ST_NATIVE>
-__device__ __forceinline__ void sap_residual_site(const T* __restrict__ x, const T* __restrict__ b,
-                                                  const void* __restrict__ gauge, const void* __restrict__ clover,
-                                                  const Lat& g, int s, const int c[4], T bc, T mu, cx<T> (&r)[12]) {
-  cx<T> acc[12], p[12];
-  all_hops_global<T, S>(x, gauge, g, s, c, bc, acc);
-  ld_cx<T, 12>(x, g.V, s, p);
-  site_diag<T, S>(clover, g.V, s, mu, p, r);
-#pragma unroll
-  for (int i = 0; i < 12; ++i) r[i] = T(0.5) * acc[i] - r[i];
-  if (b) {
-    ld_cx<T, 12>(b, g.V, s, p);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) r[i] = r[i] + p[i];
-  }
+// <q, r> / <q, q> from the three sums, 0 where <q, q> is not positive
+__device__ __forceinline__ float mr_ratio(float n, float d) { return d > 0.f ? n / d : 0.f; }
+__device__ __forceinline__ double mr_ratio(double n, double d) { return d > 0.0 ? n / d : 0.0; }
+__device__ __forceinline__ f2 mr_ratio(f2 n, f2 d) {
+  const float2 a = f2_unpack(n), b = f2_unpack(d);
+  return f2_pack(mr_ratio(a.x, b.x), mr_ratio(a.y, b.y));
 }
 
 }  // namespace
 
 template <typename T>
 struct SapOeArgs {
-  const void* gauge;  // links, clover and D_oo^-1 as T, or in 16 bits (kernel parameter S)
+  // links, clover and D_oo^-1 as T in lattice order, or in 16 bits in block
+  // order (kernel parameter S): site index block * BS + parity * HB + half_index
+  const void* gauge;
   const void* clover;
   const void* dinv;
   const T* b;
@@ -318,31 +301,29 @@ struct SapOeArgs {
   T rho;  // odd sites carry mu + rho (D_oo^-1 is built with it)
 };
 
-// The kernel walks 2 n_MR + 3 half-steps, odd and even alternating, so that the
-// hop gather, D_oo^-1 and the site-diagonal term each appear once in the code
-// (the instruction cache holds the loop):
-//   step 0 (odd):            u_o = D_oo^-1 r_o
-//   step 1 (even):           rho = r_e - D_eo u_o
-//   step 2k (odd, k >= 1):   t_o = D_oo^-1 D_oe rho
-//   step 2k+1 (even):        q = D_ee rho - D_eo t_o; MR update of e_e, rho
-//   step 2 n_MR + 2 (odd):   e_o = D_oo^-1 (r_o - D_oe e_e); x += e
-// (D_eo, D_oe = -1/2 times the intra-block hops.)
-template <typename T, int S>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2) k_sap_oe(SapOeArgs<T> a) {
+template <class R, int S>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
+    k_sap_oe(SapOeArgs<typename LaneOf<R>::T> a) {
+  using T = typename LaneOf<R>::T;
+  constexpr bool BLOCKED = S != ST_NATIVE;  // operator in block order
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SapGeom& sg = a.sg;
   const Lat& g = sg.g;
   const int HB = sg.bsites / 2;
-  cx<T>* ev = reinterpret_cast<cx<T>*>(smem_raw);  // [12][HB] even-site values (rho, then e_e)
-  cx<T>* od = ev + 12 * HB;                         // [12][HB] odd-site values (u_o, t_o)
-  cx<T>* ro = od + 12 * HB;                         // [12][HB] r_o
-  T* red = reinterpret_cast<T*>(ro + 12 * HB);      // [32 * 3]
-  const int rhs = blockIdx.x % a.nrhs;
-  const long off = (long)rhs * NR_SPINOR * g.V;
-  T* x = a.x + off;
+  cx<R>* ev = reinterpret_cast<cx<R>*>(smem_raw);  // [12][HB] even-site values (rho, then e_e)
+  cx<R>* od = ev + 12 * HB;                         // [12][HB] odd-site values
+  cx<R>* ee = od + 12 * HB;                         // [12][HB] e_e
+  R* red = reinterpret_cast<R*>(ee + 12 * HB);      // 3 per warp
+  const int groups = a.nrhs / LaneOf<R>::n;  // right-hand sides fastest over the CTAs (operator reuse in L2)
+  const long fs = (long)NR_SPINOR * g.V;
+  const long r0 = (long)(blockIdx.x % groups) * LaneOf<R>::n * fs;
+  T* x0 = a.x + r0;
+  T* x1 = x0 + fs;  // second lane
+  const T* b0 = a.b ? a.b + r0 : nullptr;
+  const T* b1 = b0 + fs;
   const long Vh = g.V / 2;
 
-  int k = blockIdx.x / a.nrhs;
+  int k = blockIdx.x / groups;
   const int nbxh = sg.nb[3] / 2;
   int bc4[4];
   const int bxh = k % nbxh;
@@ -352,6 +333,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2) k_sap_oe(SapOeArg
   bc4[1] = k % sg.nb[1];
   bc4[0] = k / sg.nb[1];
   bc4[3] = 2 * bxh + ((bc4[0] + bc4[1] + bc4[2] + a.colour) & 1);
+  const int bl = block_linear(sg, bc4);
 
   const int j = threadIdx.x;
   const bool act = j < HB;
@@ -379,138 +361,325 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2) k_sap_oe(SapOeArg
     for (int d = 0; d < 4; ++d) c[d] = bc4[d] * sg.blk[d] + lc[d];
     return ((c[0] * g.L[1] + c[1]) * g.L[2] + c[2]) * g.L[3] + c[3];
   };
-  const T half = T(0.5);
+  // operator index of the j-th site of the given parity
+  auto own_op = [&](int parity, int s) { return BLOCKED ? bl * sg.bsites + parity * HB + j : s; };
+  auto link = [&](int mu, long so, Link<T>& U) {
+    cx<T> z[6];
+    ld_op<T, 6, S>(a.gauge, (long)mu * NR_LINK * g.V, g.V, so, z);
+    link_from_rows(z, U);
+  };
+  // y += (A + i m gamma5) p
+  auto diag = [&](long so, T m, const cx<R> (&p)[12], cx<R> (&y)[12]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      T mm[36];
+      ld_re_s<T, S, 36>(BLOCKED ? static_cast<const void*>(static_cast<const unsigned short*>(a.clover) + (long)h * 36 * g.V)
+                                : static_cast<const void*>(static_cast<const T*>(a.clover) + (long)h * 36 * g.V),
+                        g.V, so, mm);
+      herm6_lanes<R, T>(mm, h == 0 ? -m : m, p + 6 * h, y + 6 * h);
+    }
+  };
 
-  // r = b - D x on the odd (pass 0, -> shared r_o) and the even site (pass 1, -> rho)
-  cx<T> rho[12];
+  // r = b - D x on the odd (pass 0, -> od) and the even site (pass 1, -> ev)
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     if (act) {
+      const int par = pass ^ 1;
       int lc[4], c[4];
-      const int s = site_of(pass ^ 1, lc, c);
-      sap_residual_site<T, S>(x, a.b ? a.b + off : nullptr, a.gauge, a.clover, g, s, c, a.bc,
-                              pass == 0 ? a.mu + a.rho : a.mu, rho);
-      if (pass == 0) {
+      const int s = site_of(par, lc, c);
+      const int so = own_op(par, s);
+      cx<R> acc[12];
 #pragma unroll
-        for (int i = 0; i < 12; ++i) ro[i * HB + j] = rho[i];
+      for (int i = 0; i < 12; ++i) acc[i] = czero<R>();
+      auto hops = [&](auto MUC) {
+        constexpr int MU = decltype(MUC)::value;
+        {
+          cx<R> p[12];
+          ld_lanes<R, 12, T>(x0, x1, g.V, nb_fwd(g, s, c, MU), p);
+          Link<T> U;
+          link(MU, so, U);
+          if (MU == 0 && c[0] == g.L[0] - 1) {
+#pragma unroll
+            for (int i = 0; i < 12; ++i) p[i] = cx<R>{bcast<R>(a.bc) * p[i].r, bcast<R>(a.bc) * p[i].i};
+          }
+          hop_lanes<R, T, MU, true>([&](int i) { return p[i]; }, U, acc);
+        }
+        {
+          cx<R> p[12];
+          const int sb = nb_bwd(g, s, c, MU);
+          ld_lanes<R, 12, T>(x0, x1, g.V, sb, p);
+          int ob = sb;
+          if (BLOCKED) {  // the link belongs to the neighbour, in this block or the one before it
+            int ln[4] = {lc[0], lc[1], lc[2], lc[3]}, bn[4] = {bc4[0], bc4[1], bc4[2], bc4[3]};
+            if (lc[MU] > 0) {
+              ln[MU] = lc[MU] - 1;
+            } else {
+              ln[MU] = sg.blk[MU] - 1;
+              bn[MU] = bn[MU] > 0 ? bn[MU] - 1 : sg.nb[MU] - 1;
+            }
+            ob = block_linear(sg, bn) * sg.bsites + (par ^ 1) * HB + half_index(ln, sg.blk);
+          }
+          Link<T> U;
+          link(MU, ob, U);
+          if (MU == 0 && c[0] == 0) {
+#pragma unroll
+            for (int i = 0; i < 12; ++i) p[i] = cx<R>{bcast<R>(a.bc) * p[i].r, bcast<R>(a.bc) * p[i].i};
+          }
+          hop_lanes<R, T, MU, false>([&](int i) { return p[i]; }, U, acc);
+        }
+      };
+      hops(std::integral_constant<int, 0>{});
+      hops(std::integral_constant<int, 1>{});
+      hops(std::integral_constant<int, 2>{});
+      hops(std::integral_constant<int, 3>{});
+      // acc = -H x / 2 + A x, then b - acc
+#pragma unroll
+      for (int i = 0; i < 12; ++i) acc[i] = cx<R>{bcast<R>(T(-0.5)) * acc[i].r, bcast<R>(T(-0.5)) * acc[i].i};
+      cx<R> p[12];
+      ld_lanes<R, 12, T>(x0, x1, g.V, s, p);
+      diag(so, par ? a.mu + a.rho : a.mu, p, acc);
+      if (b0) {
+        ld_lanes<R, 12, T>(b0, b1, g.V, s, p);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) acc[i] = p[i] - acc[i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) acc[i] = czero<R>() - acc[i];
       }
+      cx<R>* to = par ? od : ev;
+#pragma unroll
+      for (int i = 0; i < 12; ++i) st_shared(to + i * HB + j, acc[i]);
     }
   }
-  cx<T> e[12];
-#pragma unroll
-  for (int i = 0; i < 12; ++i) e[i] = cx<T>{0, 0};
+
   const int nsteps = 2 * a.n_mr + 3;
 #pragma unroll 1
   for (int st = 0; st < nsteps; ++st) {
     const int parity = (st & 1) ^ 1;  // even steps work on odd sites
     __syncthreads();
-    cx<T> acc[12];
+    cx<R> acc[12];
     int lc[4], c[4];
     const int s = site_of(parity, lc, c);
-    if (act && st > 0) oe_block_hops<T, S>(parity ? ev : od, HB, lc, sg.blk, a.gauge, g, s, c, acc);
-    if (parity) {
-      // odd site: y = D_oo^-1 in
-      if (act) {
-        cx<T> in[12], y[12];
-        const bool last = st == nsteps - 1;
+    const int so = own_op(parity, s);
+    if (act && st > 0) {
+      const cx<R>* src = parity ? ev : od;
 #pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          if (st == 0)
-            in[i] = ro[i * HB + j];
-          else if (last)
-            in[i] = ro[i * HB + j] + half * acc[i];
-          else
-            in[i] = -half * acc[i];
+      for (int i = 0; i < 12; ++i) acc[i] = czero<R>();
+      auto hops = [&](auto MUC) {
+        constexpr int MU = decltype(MUC)::value;
+        if (lc[MU] < sg.blk[MU] - 1) {
+          int ln[4] = {lc[0], lc[1], lc[2], lc[3]};
+          ln[MU] += 1;
+          const cx<R>* sp = src + half_index(ln, sg.blk);
+          Link<T> U;
+          link(MU, so, U);
+          hop_lanes<R, T, MU, true>([&](int i) { return ld_shared(sp + i * HB); }, U, acc);
         }
-        apply_dinv<T, S>(a.dinv, Vh, s, in, y);
+        if (lc[MU] > 0) {
+          int ln[4] = {lc[0], lc[1], lc[2], lc[3]};
+          ln[MU] -= 1;
+          const int jn = half_index(ln, sg.blk);
+          const cx<R>* sp = src + jn;
+          Link<T> U;
+          link(MU, BLOCKED ? bl * sg.bsites + (parity ^ 1) * HB + jn : nb_bwd(g, s, c, MU), U);
+          hop_lanes<R, T, MU, false>([&](int i) { return ld_shared(sp + i * HB); }, U, acc);
+        }
+      };
+      hops(std::integral_constant<int, 0>{});
+      hops(std::integral_constant<int, 1>{});
+      hops(std::integral_constant<int, 2>{});
+      hops(std::integral_constant<int, 3>{});
+    }
+    if (parity) {
+      // odd site: D_oo^-1 of r_o (step 0) or of the hops
+      if (act) {
+        const bool last = st == nsteps - 1;
+        if (st == 0) {
+#pragma unroll
+          for (int i = 0; i < 12; ++i) acc[i] = ld_shared(od + i * HB + j);
+        }
+        cx<R> y[12];
+        const long di = BLOCKED ? bl * HB + j : s >> 1;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 6; ++i) {
+            cx<T> m[6];
+            ld_op<T, 6, S>(a.dinv, (long)(h * 6 + i) * 12 * Vh, Vh, di, m);  // row i of block h
+            y[6 * h + i] = lcmul(m[0], acc[6 * h]);
+#pragma unroll
+            for (int q = 1; q < 6; ++q) lcfma(y[6 * h + i], m[q], acc[6 * h + q]);
+          }
         if (!last) {
 #pragma unroll
-          for (int i = 0; i < 12; ++i) od[i * HB + j] = y[i];
-        } else {
-          // x_o += e_o, x_e += e_e
-          cx<T> p[12];
-          ld_cx<T, 12>(x, g.V, s, p);
+          for (int i = 0; i < 12; ++i) st_shared(od + i * HB + j, y[i]);
+        }
+        if (st == 0 || last) {
+          // every residual of the block has been formed from the old x (barrier above)
+          const R w = bcast<R>(st == 0 ? T(1) : T(0.5));
+          cx<R> p[12];
+          ld_lanes_rw<R, 12, T>(x0, x1, g.V, s, p);
 #pragma unroll
-          for (int i = 0; i < 12; ++i) p[i] = p[i] + y[i];
-          st_cx<T, 12>(x, g.V, s, p);
+          for (int i = 0; i < 12; ++i) p[i] = cx<R>{lfma(w, y[i].r, p[i].r), lfma(w, y[i].i, p[i].i)};
+          st_lanes<R, 12, T>(x0, x1, g.V, s, p);
+        }
+        if (last) {
           int lc2[4], c2[4];
           const int s2 = site_of(0, lc2, c2);
-          ld_cx<T, 12>(x, g.V, s2, p);
+          cx<R> p[12];
+          ld_lanes_rw<R, 12, T>(x0, x1, g.V, s2, p);
 #pragma unroll
-          for (int i = 0; i < 12; ++i) p[i] = p[i] + e[i];
-          st_cx<T, 12>(x, g.V, s2, p);
+          for (int i = 0; i < 12; ++i) p[i] = p[i] + ld_shared(ev + i * HB + j);
+          st_lanes<R, 12, T>(x0, x1, g.V, s2, p);
         }
       }
     } else {
-      const int kk = (st - 1) / 2;  // MR steps done before this one
+      const bool store_e = (st - 1) / 2 == a.n_mr;  // the next odd step gathers e_e
+      cx<R> rho[12];
+      if (act) {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) rho[i] = ld_shared(ev + i * HB + j);
+      }
       if (st == 1) {
         if (act) {
+          const R hf = bcast<R>(T(0.5));
 #pragma unroll
-          for (int i = 0; i < 12; ++i) rho[i] = rho[i] + half * acc[i];
+          for (int i = 0; i < 12; ++i) {
+            rho[i] = cx<R>{lfma(hf, acc[i].r, rho[i].r), lfma(hf, acc[i].i, rho[i].i)};
+            st_shared(ee + i * HB + j, czero<R>());
+            st_shared(ev + i * HB + j, store_e ? czero<R>() : rho[i]);
+          }
         }
       } else {
-        cx<T> q[12];
-        T dots[3] = {0, 0, 0};
+        R dots[3] = {bcast<R>(T(0)), bcast<R>(T(0)), bcast<R>(T(0))};
         if (act) {
-          site_diag<T, S>(a.clover, g.V, s, a.mu, rho, q);
+          const R mq = bcast<R>(T(-0.25));
+#pragma unroll
+          for (int i = 0; i < 12; ++i) acc[i] = cx<R>{mq * acc[i].r, mq * acc[i].i};
+          diag(so, a.mu, rho, acc);  // acc = q
+          R d1 = bcast<R>(T(0));
 #pragma unroll
           for (int i = 0; i < 12; ++i) {
-            q[i] = q[i] + half * acc[i];
-            dots[0] = fma(q[i].r, rho[i].r, fma(q[i].i, rho[i].i, dots[0]));   // Re <q, rho>
-            dots[1] = fma(q[i].r, rho[i].i, fma(-q[i].i, rho[i].r, dots[1]));  // Im <q, rho>
-            dots[2] = fma(q[i].r, q[i].r, fma(q[i].i, q[i].i, dots[2]));       // <q, q>
+            dots[0] = lfma(acc[i].r, rho[i].r, lfma(acc[i].i, rho[i].i, dots[0]));  // Re <q, rho>
+            dots[1] = lfma(acc[i].r, rho[i].i, dots[1]);                           // Im <q, rho> = the difference
+            d1 = lfma(acc[i].i, rho[i].r, d1);
+            dots[2] = lfma(acc[i].r, acc[i].r, lfma(acc[i].i, acc[i].i, dots[2]));  // <q, q>
           }
+          dots[1] = dots[1] - d1;
         }
-        block_allreduce<T, 3>(dots, red);
-        const cx<T> alpha = dots[2] > T(0) ? cx<T>{dots[0] / dots[2], dots[1] / dots[2]} : cx<T>{0, 0};
+        lanes_allreduce3<R>(dots, red);
         if (act) {
+          const R ar = mr_ratio(dots[0], dots[2]), ai = mr_ratio(dots[1], dots[2]);
+          const R nr = bcast<R>(T(0)) - ar, ni = bcast<R>(T(0)) - ai;
 #pragma unroll
           for (int i = 0; i < 12; ++i) {
-            cfma(e[i], alpha, rho[i]);
-            cfma(rho[i], -alpha, q[i]);
+            cx<R> e = ld_shared(ee + i * HB + j);
+            e.r = lfma(ni, rho[i].i, lfma(ar, rho[i].r, e.r));
+            e.i = lfma(ai, rho[i].r, lfma(ar, rho[i].i, e.i));
+            if (!store_e) st_shared(ee + i * HB + j, e);
+            cx<R> q = rho[i];  // rho - alpha q
+            q.r = lfma(ai, acc[i].i, lfma(nr, acc[i].r, q.r));
+            q.i = lfma(ni, acc[i].r, lfma(nr, acc[i].i, q.i));
+            st_shared(ev + i * HB + j, store_e ? e : q);
           }
         }
-      }
-      // the next odd step gathers rho, or e_e after the last MR step (step 2 n_MR + 1)
-      if (act) {
-        const bool store_e = kk == a.n_mr;
-#pragma unroll
-        for (int i = 0; i < 12; ++i) ev[i * HB + j] = store_e ? e[i] : rho[i];
       }
     }
   }
 }
 
-template <typename T, int S>
-void sap_oe_s(const SapOeArgs<T>& a, int nblocks, int threads, size_t smem, cudaStream_t st) {
+template <class R, int S>
+void sap_oe_s(SapOeArgs<typename LaneOf<R>::T> a, int nblocks, cudaStream_t st) {
+  const int HB = a.sg.bsites / 2;
+  const int threads = (HB + 31) / 32 * 32;
+  const size_t smem = 36 * (size_t)HB * sizeof(cx<R>) + (threads / 32) * 3 * sizeof(R);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_sap_oe<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_sap_oe<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
-  k_sap_oe<T, S><<<dim3(nblocks), threads, smem, st>>>(a);
+  k_sap_oe<R, S><<<dim3(nblocks * (a.nrhs / LaneOf<R>::n)), threads, smem, st>>>(a);
 }
 
 template <typename T>
 void launch_sap_oe_colour(const void* gauge, const void* clover, const void* dinv, const T* b, T* x,
                           const SapGeom& sg, double mu, double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st,
                           double rho, int s16) {
-  const int HB = sg.bsites / 2;
-  const int threads = (HB + 31) / 32 * 32;
-  const size_t smem = 3 * 12 * (size_t)HB * sizeof(cx<T>) + 32 * 3 * sizeof(T);
   const int nblk_colour = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2;
   SapOeArgs<T> a{gauge, clover, dinv, b, x, sg, (T)mu, (T)bc_t, n_mr, colour, nrhs, (T)rho};
   if constexpr (std::is_same<T, float>::value) {
-    if (s16 == ST_F16) return sap_oe_s<T, ST_F16>(a, nblk_colour * nrhs, threads, smem, st);
-    if (s16 == ST_BF16) return sap_oe_s<T, ST_BF16>(a, nblk_colour * nrhs, threads, smem, st);
+    // whole pairs two to a thread; an odd one out alone (a pair with an idle lane
+    // costs 1.8 times a single right-hand side).  While one CTA per right-hand
+    // side still fits the chip at once (3 CTAs on each of 152 SMs) pairs would
+    // only make the longest CTA longer: 8^4 with 2 right-hand sides, 3 sweeps,
+    // 331 us in pairs, 276 us alone.
+    const bool alone = (long)nblk_colour * nrhs <= 3 * 152;
+    a.nrhs = alone ? 0 : nrhs & ~1;
+    if (a.nrhs) {
+      if (s16 == ST_F16)
+        sap_oe_s<f2, ST_F16>(a, nblk_colour, st);
+      else if (s16 == ST_BF16)
+        sap_oe_s<f2, ST_BF16>(a, nblk_colour, st);
+      else
+        sap_oe_s<f2, ST_NATIVE>(a, nblk_colour, st);
+    }
+    const long off = (long)a.nrhs * NR_SPINOR * sg.g.V;
+    a.nrhs = nrhs - a.nrhs;
+    if (!a.nrhs) return;
+    a.x += off;
+    if (a.b) a.b += off;
+    if (s16 == ST_F16) return sap_oe_s<T, ST_F16>(a, nblk_colour, st);
+    if (s16 == ST_BF16) return sap_oe_s<T, ST_BF16>(a, nblk_colour, st);
   }
-  sap_oe_s<T, ST_NATIVE>(a, nblk_colour * nrhs, threads, smem, st);
+  sap_oe_s<T, ST_NATIVE>(a, nblk_colour, st);
 }
 
 template void launch_sap_oe_colour<double>(const void*, const void*, const void*, const double*, double*,
                                            const SapGeom&, double, double, int, int, int, cudaStream_t, double, int);
 template void launch_sap_oe_colour<float>(const void*, const void*, const void*, const float*, float*,
                                           const SapGeom&, double, double, int, int, int, cudaStream_t, double, int);
+
+// 16-bit copy in block order of a chunked FP32 field: `planes` chunk planes of n
+// sites, all V of them (PAR = 0) or the V / 2 odd ones by their index s >> 1
+template <int KIND>
+__global__ void k_to16_blocks(const float4* __restrict__ in, uint2* __restrict__ out, SapGeom sg, int n) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= n) return;
+  const int HB = sg.bsites / 2;
+  const bool half = n != sg.g.V;
+  int c[4], lc[4], bc[4];
+  site_coords(sg.g, half ? 2 * s : s, c);
+  if (half) c[3] = (c[3] & ~1) | (((c[0] + c[1] + c[2]) & 1) ^ 1);  // the odd site of the pair (X even)
+  for (int d = 0; d < 4; ++d) {
+    bc[d] = c[d] / sg.blk[d];
+    lc[d] = c[d] - bc[d] * sg.blk[d];
+  }
+  const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
+  const int to = block_linear(sg, bc) * (half ? HB : sg.bsites) + (half ? 0 : par * HB) + half_index(lc, sg.blk);
+  const long p = (long)blockIdx.y * n;
+  const float4 v = in[p + s];
+  unsigned u[2];
+  if constexpr (KIND == ST_F16) {
+    const __half2 a = __float22half2_rn(make_float2(v.x, v.y)), b = __float22half2_rn(make_float2(v.z, v.w));
+    memcpy(&u[0], &a, 4);
+    memcpy(&u[1], &b, 4);
+  } else {
+    const __nv_bfloat162 a = __float22bfloat162_rn(make_float2(v.x, v.y)), b = __float22bfloat162_rn(make_float2(v.z, v.w));
+    memcpy(&u[0], &a, 4);
+    memcpy(&u[1], &b, 4);
+  }
+  out[p + to] = make_uint2(u[0], u[1]);
+}
+
+void launch_to16_blocks(const float* in, void* out, const SapGeom& sg, int planes, bool odd_only, int kind,
+                        cudaStream_t st) {
+  const int n = odd_only ? sg.g.V / 2 : sg.g.V;
+  dim3 grid((n + 127) / 128, planes);
+  if (kind == ST_F16)
+    k_to16_blocks<ST_F16><<<grid, 128, 0, st>>>(reinterpret_cast<const float4*>(in), static_cast<uint2*>(out), sg, n);
+  else
+    k_to16_blocks<ST_BF16><<<grid, 128, 0, st>>>(reinterpret_cast<const float4*>(in), static_cast<uint2*>(out), sg, n);
+}
 
 // ===========================================================================
 // D_oo^-1 for the odd-even block solve: per odd site the inverses of the two

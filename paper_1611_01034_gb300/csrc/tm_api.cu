@@ -348,7 +348,7 @@ void build_sap_inverse(tm_handle* h) {
                                  h->st);
   CKL();
   if (h->dinv16) {
-    launch_to16(static_cast<const float*>(h->dinv_sap), h->dinv16, (long)h->g.V / 2 * 72, h->p.sap_prec, h->st);
+    launch_to16_blocks(static_cast<const float*>(h->dinv_sap), h->dinv16, h->sg, 36, true, h->p.sap_prec, h->st);
     CKL();
   }
 }
@@ -2529,9 +2529,9 @@ tm_status tm_load_gauge(tm_handle* h, const double* gauge) {
   }
   if (h->g16) {
     Prof pf(h, PK_OTHER, 1, 2);
-    launch_to16(h->g32, h->g16, (long)h->g.V * 4 * NR_LINK / 2, h->p.sap_prec, h->st);
+    launch_to16_blocks(h->g32, h->g16, h->sg, 4 * NR_LINK / 4, false, h->p.sap_prec, h->st);
     CKL();
-    launch_to16(h->c32, h->c16, (long)h->g.V * NR_CLOVER / 2, h->p.sap_prec, h->st);
+    launch_to16_blocks(h->c32, h->c16, h->sg, NR_CLOVER / 4, false, h->p.sap_prec, h->st);
     CKL();
   }
   if (h->gdf) {

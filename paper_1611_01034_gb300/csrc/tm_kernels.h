@@ -58,11 +58,16 @@ void launch_sap_colour(const T* gauge, const T* clover, const T* b, T* x, const 
 
 // the same with the block solves on the odd-even Schur complement (Sec. 3);
 // all block dims even; dinv from launch_clover_inverse
-// gauge, clover, dinv stored as T, or (T = float) in 16 bits when s16 = ST_F16 / ST_BF16
+// gauge, clover, dinv stored as T in lattice order, or (T = float) in 16 bits and block order
+// (launch_to16_blocks) when s16 = ST_F16 / ST_BF16
 template <typename T>
 void launch_sap_oe_colour(const void* gauge, const void* clover, const void* dinv, const T* b, T* x,
                           const SapGeom& sg, double mu, double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st,
                           double rho = 0.0, int s16 = 0);
+// 16-bit copy of `planes` chunk planes of an FP32 field, the sites of each SAP block side by
+// side (even ones first); odd_only: a field over the odd sites (index s >> 1)
+void launch_to16_blocks(const float* in, void* out, const SapGeom& sg, int planes, bool odd_only, int kind,
+                        cudaStream_t st);
 // dinv [12 rows x 6 complex chunks][V/2] = (A(x) + i mu gamma5)^-1 of the two
 // chiral blocks at every odd site (compact index s >> 1; X even); mu = the
 // odd sites' twisted mass

@@ -1,0 +1,48 @@
+"""SAP on batches of right-hand sides: pairs share a thread, an odd one out runs alone.
+
+Every right-hand side of a batch must get what it gets alone, in every storage of the operator, for
+blocks that fill their warps (4^4), leave lanes idle (2^4) and have unequal dims, with and without b;
+the last one of each batch is also held against the oracle on the smaller lattices.  Tolerances: the two
+forms order their FP32 sums differently (4 MR steps amplify 2^-24 to below 5e-6); against the oracle as
+for one right-hand side (FP32 5e-5, a 16-bit operator 2^-11 or 2^-8 per entry over the same chain).
+"""
+import numpy as np
+import pytest
+
+import inputs
+import paper_1611_01034_gb300 as tm
+from oracle.dirac import Operator
+from oracle.sap import SAP
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from tests.gpu_helpers import GPU, rel  # noqa: E402
+
+F32 = tm.TM_F32
+
+
+def _sweeps(g, b, x0, sweeps):
+    n = x0.shape[0]
+    fx = g.pack(0, F32, x0, n)
+    tm.tm_sap(g.h, F32, None if b is None else g.pack(0, F32, b, n), fx, sweeps, n)
+    return g.unpack(0, F32, fx, x0.shape, n)
+
+
+@pytest.mark.parametrize("L,blk,nrhs", [((8, 8, 8, 16), (2, 2, 2, 2), 3), ((8, 8, 8, 24), (4, 2, 4, 2), 7),
+                                        ((16, 16, 16, 16), (4, 4, 4, 4), 2), ((16, 16, 16, 16), (4, 4, 4, 4), 5),
+                                        ((8, 16, 16, 8), (4, 4, 4, 4), 15)])
+@pytest.mark.parametrize("prec,tol", [(tm.TM_F32, 5e-5), (tm.TM_F16, 5e-3), (tm.TM_BF16, 3e-2)])
+def test_odd_even_sap_batches(L, blk, nrhs, prec, tol):
+    U = inputs.gauge_field(L, 0.5, 17)
+    g = GPU(U, m0=-0.3, c_sw=1.3, mu=0.05, nv=2, agg=blk, sap_block=blk, cycle_prec=F32, max_rhs=nrhs, block_oe=1,
+            sap_prec=prec)
+    b, x0 = inputs.gaussian_spinor(L, 1, nrhs), inputs.gaussian_spinor(L, 2, nrhs)
+    got, got0 = _sweeps(g, b, x0, 2), _sweeps(g, None, x0, 1)
+    for r in range(nrhs):
+        assert rel(got[r], _sweeps(g, b[r:r + 1], x0[r:r + 1], 2)[0]) <= 5e-6
+        assert rel(got0[r], _sweeps(g, None, x0[r:r + 1], 1)[0]) <= 5e-6
+    if nrhs in (3, 7):
+        sap = SAP(Operator(U, -0.3, 1.3, 0.05), blk, n_mr=4, block_oe=True)
+        assert rel(got[-1], sap.smooth(b[-1], x0[-1], 2)) <= tol
+        assert rel(got0[0], sap.smooth(np.zeros_like(b[0]), x0[0], 1)) <= tol
