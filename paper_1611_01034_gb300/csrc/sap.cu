@@ -601,6 +601,407 @@ void sap_oe_s(SapOeArgs<typename LaneOf<R>::T> a, int nblocks, cudaStream_t st) 
   k_sap_oe<R, S><<<dim3(nblocks * (a.nrhs / LaneOf<R>::n)), threads, smem, st>>>(a);
 }
 
+// ===========================================================================
+// The same block solve for 4^4 blocks, a 16-bit operator and pairs of
+// right-hand sides.  k_sap_oe holds 74 KB of shared memory per CTA for such a
+// pair and needs 255 registers, so two CTAs share an SM.  Here the sums e_e and
+// e_o, which only their own thread reads, live in tensor memory (96 of 128
+// allocated columns), shared memory holds just the two fields that the hops
+// gather (48 KB), and with the block's shape known at compile time 168
+// registers suffice: three CTAs, 12 warps per SM (6-rhs launch at 48 x 24^3:
+// 1.11 -> 1.02 ms).  Measured and left out: the block's operator (78 KB) staged
+// in shared memory for two or three pairs of one larger CTA (1.25 and 1.61 ms:
+// its warps wait in the same phases), four CTAs per SM (128 registers, 1.63 ms).
+//
+// e_o needs no half-step of its own: with z_k = D_oo^-1 H rho_k, which every MR
+// step forms anyway, D_oo^-1 H e_e = sum_k alpha_k z_k, so the last odd half-step
+// of k_sap_oe becomes one more running sum:
+//   step 0 (odd):           od = D_oo^-1 r_o; e_o = 2 od
+//   step 1 (even):          rho = r_e + H od / 2
+//   step 2k (odd, k >= 1):  od = z = D_oo^-1 H rho
+//   step 2k+1 (even):       q = D_ee rho - H od / 4; e_e += alpha rho, e_o += alpha z,
+//                           rho -= alpha q
+//   then x_e += e_e, x_o += e_o / 2.
+// ===========================================================================
+namespace {
+
+constexpr int kB4 = 256, kH4 = 128;           // sites of a 4^4 block, of one parity
+constexpr unsigned kTmemCols = 128;  // e_e at column 0, e_o at 48
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) {
+  return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+// four complex pairs (16 words per thread) to and from tensor memory; the caller waits
+__device__ __forceinline__ void tmem_st4(unsigned ta, const cx<f2>* z) {
+  float2 v[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[2 * k] = f2_unpack(z[k].r);
+    v[2 * k + 1] = f2_unpack(z[k].i);
+  }
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(ta),
+      "f"(v[0].x), "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y),
+      "f"(v[4].x), "f"(v[4].y), "f"(v[5].x), "f"(v[5].y), "f"(v[6].x), "f"(v[6].y), "f"(v[7].x), "f"(v[7].y)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(unsigned ta, cx<f2>* z) {
+  float v[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+      : "r"(ta)
+      : "memory");
+#pragma unroll
+  for (int k = 0; k < 4; ++k) z[k] = cx<f2>{f2_pack(v[4 * k], v[4 * k + 1]), f2_pack(v[4 * k + 2], v[4 * k + 3])};
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// two complex numbers of a 16-bit chunk
+template <int S>
+__device__ __forceinline__ void unpack_chunk(uint2 v, cx<float>& a, cx<float>& b) {
+  const float2 p = unpack16x2<S>(v.x), q = unpack16x2<S>(v.y);
+  a = cx<float>{p.x, p.y};
+  b = cx<float>{q.x, q.y};
+}
+
+template <int S>
+__global__ void __launch_bounds__(kH4, 3) k_sap_oe4(SapOeArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned tmem_base;
+  __shared__ f2 red[4 * 3];
+  const SapGeom& sg = a.sg;
+  const Lat& g = sg.g;
+  const int pairs = a.nrhs / 2;
+  const int j = threadIdx.x, warp = j >> 5;
+  const long V = g.V, Vh = g.V / 2;
+
+  int bc4[4];
+  {
+    int k = blockIdx.x / pairs;  // pairs fastest over the CTAs (operator reuse in L2)
+    const int nbxh = sg.nb[3] / 2;
+    const int bxh = k % nbxh;
+    k /= nbxh;
+    bc4[2] = k % sg.nb[2];
+    k /= sg.nb[2];
+    bc4[1] = k % sg.nb[1];
+    bc4[0] = k / sg.nb[1];
+    bc4[3] = 2 * bxh + ((bc4[0] + bc4[1] + bc4[2] + a.colour) & 1);
+  }
+  const int bl = block_linear(sg, bc4);
+  const uint2* gauge = static_cast<const uint2*>(a.gauge);
+  const uint2* clover = static_cast<const uint2*>(a.clover);
+  const uint2* dinv = static_cast<const uint2*>(a.dinv);
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned ta = tmem_base + ((unsigned)warp << 21);  // a warp reaches its own 32 lanes
+  {
+    const int grp = blockIdx.x % pairs;
+    cx<f2>* ev = reinterpret_cast<cx<f2>*>(smem_raw);  // [12][128] rho
+    cx<f2>* od = ev + 12 * kH4;                         // [12][128] u_o and z
+    const long fs = (long)NR_SPINOR * V;
+    float* x0 = a.x + 2 * grp * fs;
+    float* x1 = x0 + fs;
+    const float* b0 = a.b ? a.b + 2 * grp * fs : nullptr;
+    const float* b1 = a.b ? b0 + fs : nullptr;
+    // j = ((t 4 + z) 4 + y) 2 + (x >> 1)
+    const int lt = j >> 5, lz = (j >> 3) & 3, ly = (j >> 1) & 3, xh = j & 1;
+    const int pr = (lt + lz + ly) & 1;  // x parity of the even site
+    const uint2* olink = gauge + (long)bl * kB4;
+    const uint2* oclov = clover + (long)bl * kB4;
+    const uint2* odinv = dinv + (long)bl * kH4 + j;
+    auto link = [&](int mu, int w, Link<float>& U) {  // site w of the block in block order
+      cx<float> z[6];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) unpack_chunk<S>(__ldg(olink + (mu * 3 + k) * V + w), z[2 * k], z[2 * k + 1]);
+      link_from_rows(z, U);
+    };
+    // y += (A + i m gamma5) p, the clover chunk k of the site from ld(k)
+    auto diag = [&](auto ld, float m, const cx<f2>(&p)[12], cx<f2>(&y)[12]) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float mm[36];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          cx<float> u, v;
+          unpack_chunk<S>(ld(9 * h + k), u, v);
+          mm[4 * k] = u.r;
+          mm[4 * k + 1] = u.i;
+          mm[4 * k + 2] = v.r;
+          mm[4 * k + 3] = v.i;
+        }
+        herm6_lanes<f2, float>(mm, h == 0 ? -m : m, p + 6 * h, y + 6 * h);
+      }
+    };
+    auto site = [&](int par, int (&c)[4]) {
+      c[0] = 4 * bc4[0] + lt;
+      c[1] = 4 * bc4[1] + lz;
+      c[2] = 4 * bc4[2] + ly;
+      c[3] = 4 * bc4[3] + 2 * xh + (pr ^ par);
+      return ((c[0] * g.L[1] + c[1]) * g.L[2] + c[2]) * g.L[3] + c[3];
+    };
+
+    // r = b - D x on the odd (pass 0, -> od) and the even site (pass 1, -> ev)
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      const int par = pass ^ 1;
+      int c[4];
+      const int s = site(par, c);
+      const int lx = 2 * xh + (pr ^ par), own = par * kH4 + j;
+      cx<f2> acc[12];
+#pragma unroll
+      for (int i = 0; i < 12; ++i) acc[i] = czero<f2>();
+      auto hops = [&](auto MUC) {
+        constexpr int MU = decltype(MUC)::value;
+        const int lm = MU == 0 ? lt : MU == 1 ? lz : MU == 2 ? ly : lx;
+        const int js = MU == 0 ? 32 : MU == 1 ? 8 : 2;
+        {
+          cx<f2> p[12];
+          ld_lanes<f2, 12, float>(x0, x1, V, nb_fwd(g, s, c, MU), p);
+          Link<float> U;
+          link(MU, own, U);
+          if (MU == 0 && c[0] == g.L[0] - 1) {
+#pragma unroll
+            for (int i = 0; i < 12; ++i) p[i] = cx<f2>{bcast<f2>(a.bc) * p[i].r, bcast<f2>(a.bc) * p[i].i};
+          }
+          hop_lanes<f2, float, MU, true>([&](int i) { return p[i]; }, U, acc);
+        }
+        {
+          cx<f2> p[12];
+          ld_lanes<f2, 12, float>(x0, x1, V, nb_bwd(g, s, c, MU), p);
+          cx<float> z[6];
+          if (lm > 0) {
+            const int jn = MU < 3 ? j - js : (j & ~1) + ((lx - 1) >> 1);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+              unpack_chunk<S>(__ldg(olink + (MU * 3 + k) * V + (par ^ 1) * kH4 + jn), z[2 * k], z[2 * k + 1]);
+          } else {  // the link belongs to the block before this one
+            int bn[4] = {bc4[0], bc4[1], bc4[2], bc4[3]};
+            bn[MU] = bn[MU] > 0 ? bn[MU] - 1 : sg.nb[MU] - 1;
+            const int jn = MU < 3 ? j + 3 * js : (j & ~1) + 1;
+            const uint2* src = gauge + (long)block_linear(sg, bn) * kB4 + (par ^ 1) * kH4 + jn;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) unpack_chunk<S>(__ldg(src + (MU * 3 + k) * V), z[2 * k], z[2 * k + 1]);
+          }
+          Link<float> U;
+          link_from_rows(z, U);
+          if (MU == 0 && c[0] == 0) {
+#pragma unroll
+            for (int i = 0; i < 12; ++i) p[i] = cx<f2>{bcast<f2>(a.bc) * p[i].r, bcast<f2>(a.bc) * p[i].i};
+          }
+          hop_lanes<f2, float, MU, false>([&](int i) { return p[i]; }, U, acc);
+        }
+      };
+      hops(std::integral_constant<int, 0>{});
+      hops(std::integral_constant<int, 1>{});
+      hops(std::integral_constant<int, 2>{});
+      hops(std::integral_constant<int, 3>{});
+#pragma unroll
+      for (int i = 0; i < 12; ++i) acc[i] = cx<f2>{bcast<f2>(-0.5f) * acc[i].r, bcast<f2>(-0.5f) * acc[i].i};
+      cx<f2> p[12];
+      ld_lanes<f2, 12, float>(x0, x1, V, s, p);
+      diag([&](int k) { return __ldg(oclov + k * V + own); }, par ? a.mu + a.rho : a.mu, p, acc);
+      cx<f2>* to = par ? od : ev;
+      if (b0) {
+        ld_lanes<f2, 12, float>(b0, b1, V, s, p);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) st_shared(to + i * kH4 + j, p[i] - acc[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) st_shared(to + i * kH4 + j, czero<f2>() - acc[i]);
+      }
+    }
+
+    const int nsteps = 2 * a.n_mr + 2;
+#pragma unroll 1
+    for (int st = 0; st < nsteps; ++st) {
+      const int parity = (st & 1) ^ 1;  // even steps work on odd sites
+      __syncthreads();
+      cx<f2> acc[12];
+      if (st > 0) {
+        const cx<f2>* src = parity ? ev : od;
+        const int own = parity * kH4 + j, oth = (parity ^ 1) * kH4;
+        const int lx = 2 * xh + (pr ^ parity);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) acc[i] = czero<f2>();
+        auto hops = [&](auto MUC) {
+          constexpr int MU = decltype(MUC)::value;
+          const int lm = MU == 0 ? lt : MU == 1 ? lz : MU == 2 ? ly : lx;
+          const int js = MU == 0 ? 32 : MU == 1 ? 8 : 2;
+          if (lm < 3) {
+            const cx<f2>* sp = src + (MU < 3 ? j + js : (j & ~1) + ((lx + 1) >> 1));
+            Link<float> U;
+            link(MU, own, U);
+            hop_lanes<f2, float, MU, true>([&](int i) { return ld_shared(sp + i * kH4); }, U, acc);
+          }
+          if (lm > 0) {
+            const int jn = MU < 3 ? j - js : (j & ~1) + ((lx - 1) >> 1);
+            const cx<f2>* sp = src + jn;
+            Link<float> U;
+            link(MU, oth + jn, U);
+            hop_lanes<f2, float, MU, false>([&](int i) { return ld_shared(sp + i * kH4); }, U, acc);
+          }
+        };
+        hops(std::integral_constant<int, 0>{});
+        hops(std::integral_constant<int, 1>{});
+        hops(std::integral_constant<int, 2>{});
+        hops(std::integral_constant<int, 3>{});
+      }
+      if (parity) {
+        if (st == 0) {
+#pragma unroll
+          for (int i = 0; i < 12; ++i) acc[i] = ld_shared(od + i * kH4 + j);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          cx<f2> y[6];
+#pragma unroll
+          for (int i = 0; i < 6; ++i) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {  // chunk (6 h + i) 3 + q: entries 2 q, 2 q + 1 of row i
+              cx<float> u, v;
+              unpack_chunk<S>(__ldg(odinv + ((6 * h + i) * 3 + q) * Vh), u, v);
+              if (q == 0)
+                y[i] = lcmul(u, acc[6 * h]);
+              else
+                lcfma(y[i], u, acc[6 * h + 2 * q]);
+              lcfma(y[i], v, acc[6 * h + 2 * q + 1]);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) st_shared(od + (6 * h + i) * kH4 + j, y[i]);
+        }
+        if (st == 0) {
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            cx<f2> e[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = czero<f2>();
+            tmem_st4(ta + 16 * q, e);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const cx<f2> u = ld_shared(od + (4 * q + i) * kH4 + j);
+              e[i] = u + u;
+            }
+            tmem_st4(ta + 48 + 16 * q, e);
+          }
+          tmem_wait_st();
+        }
+      } else {
+        cx<f2> rho[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) rho[i] = ld_shared(ev + i * kH4 + j);
+        if (st == 1) {
+          const f2 hf = bcast<f2>(0.5f);
+#pragma unroll
+          for (int i = 0; i < 12; ++i)
+            st_shared(ev + i * kH4 + j, cx<f2>{lfma(hf, acc[i].r, rho[i].r), lfma(hf, acc[i].i, rho[i].i)});
+        } else {
+          const f2 mq = bcast<f2>(-0.25f);
+#pragma unroll
+          for (int i = 0; i < 12; ++i) acc[i] = cx<f2>{mq * acc[i].r, mq * acc[i].i};
+          diag([&](int k) { return __ldg(oclov + k * V + j); }, a.mu, rho, acc);  // acc = q
+          f2 dots[3] = {bcast<f2>(0.f), bcast<f2>(0.f), bcast<f2>(0.f)}, d1 = bcast<f2>(0.f);
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            dots[0] = lfma(acc[i].r, rho[i].r, lfma(acc[i].i, rho[i].i, dots[0]));  // Re <q, rho>
+            dots[1] = lfma(acc[i].r, rho[i].i, dots[1]);                           // Im <q, rho> = the difference
+            d1 = lfma(acc[i].i, rho[i].r, d1);
+            dots[2] = lfma(acc[i].r, acc[i].r, lfma(acc[i].i, acc[i].i, dots[2]));  // <q, q>
+          }
+          dots[1] = dots[1] - d1;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dots[k] = dots[k] + f2{__shfl_xor_sync(0xffffffffu, dots[k].v, o)};
+          }
+          if ((j & 31) == 0) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) red[(j >> 5) * 3 + k] = dots[k];
+          }
+          __syncthreads();
+#pragma unroll
+          for (int k = 0; k < 3; ++k) dots[k] = (red[k] + red[3 + k]) + (red[6 + k] + red[9 + k]);
+          const f2 ar = mr_ratio(dots[0], dots[2]), ai = mr_ratio(dots[1], dots[2]);
+          const f2 nr = bcast<f2>(0.f) - ar, ni = bcast<f2>(0.f) - ai;
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+            cx<f2> q = rho[i];  // rho - alpha q
+            q.r = lfma(ai, acc[i].i, lfma(nr, acc[i].r, q.r));
+            q.i = lfma(ni, acc[i].r, lfma(nr, acc[i].i, q.i));
+            st_shared(ev + i * kH4 + j, q);
+          }
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            cx<f2> e[4];
+            tmem_ld4(ta + 16 * q, e);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const cx<f2> r = rho[4 * q + i];
+              e[i].r = lfma(ni, r.i, lfma(ar, r.r, e[i].r));
+              e[i].i = lfma(ai, r.r, lfma(ar, r.i, e[i].i));
+            }
+            tmem_st4(ta + 16 * q, e);
+            tmem_ld4(ta + 48 + 16 * q, e);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const cx<f2> z = ld_shared(od + (4 * q + i) * kH4 + j);
+              e[i].r = lfma(ni, z.i, lfma(ar, z.r, e[i].r));
+              e[i].i = lfma(ai, z.r, lfma(ar, z.i, e[i].i));
+            }
+            tmem_st4(ta + 48 + 16 * q, e);
+          }
+          tmem_wait_st();
+        }
+      }
+    }
+    // x_e += e_e, x_o += e_o / 2
+#pragma unroll
+    for (int par = 0; par < 2; ++par) {
+      int c[4];
+      const int s = site(par, c);
+      const f2 w = bcast<f2>(par ? 0.5f : 1.f);
+      cx<f2> p[12];
+      ld_lanes<f2, 12, float>(x0, x1, V, s, p);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        cx<f2> e[4];
+        tmem_ld4(ta + 48 * par + 16 * q, e);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[4 * q + i] = cx<f2>{lfma(w, e[i].r, p[4 * q + i].r), lfma(w, e[i].i, p[4 * q + i].i)};
+      }
+      st_lanes<f2, 12, float>(x0, x1, V, s, p);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+}
+
+template <int S>
+void sap_oe4_s(const SapOeArgs<float>& a, int nblocks, cudaStream_t st) {
+  constexpr size_t smem = 24 * kH4 * sizeof(cx<f2>);
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaFuncSetAttribute(k_sap_oe4<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    attr_set = true;
+  }
+  k_sap_oe4<S><<<dim3(nblocks * (a.nrhs / 2)), kH4, smem, st>>>(a);
+}
+
+}  // namespace
+
 template <typename T>
 void launch_sap_oe_colour(const void* gauge, const void* clover, const void* dinv, const T* b, T* x,
                           const SapGeom& sg, double mu, double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st,
@@ -616,7 +1017,13 @@ void launch_sap_oe_colour(const void* gauge, const void* clover, const void* din
     const bool alone = (long)nblk_colour * nrhs <= 3 * 152;
     a.nrhs = alone ? 0 : nrhs & ~1;
     if (a.nrhs) {
-      if (s16 == ST_F16)
+      bool b4 = s16 != ST_NATIVE;  // k_sap_oe4 has the block shape and 16-bit storage built in
+      for (int d = 0; d < 4; ++d) b4 = b4 && sg.blk[d] == 4;
+      if (b4 && s16 == ST_F16)
+        sap_oe4_s<ST_F16>(a, nblk_colour, st);
+      else if (b4)
+        sap_oe4_s<ST_BF16>(a, nblk_colour, st);
+      else if (s16 == ST_F16)
         sap_oe_s<f2, ST_F16>(a, nblk_colour, st);
       else if (s16 == ST_BF16)
         sap_oe_s<f2, ST_BF16>(a, nblk_colour, st);
