@@ -18,50 +18,76 @@
 #include <type_traits>
 
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 #include "tm_pair.cuh"
 
 namespace tmamg {
 
 namespace {
 
-// exact difference / sum of two FP32 complex numbers as a pair
-__device__ __forceinline__ cdf exact_sum(cx<float> a, cx<float> b) { return cdf{two_sum(a.r, b.r), two_sum(a.i, b.i)}; }
-// the same for pair inputs (a pair sum)
-__device__ __forceinline__ dfl pair_add(dfl a, dfl b) {
-  const dfl s = two_sum(a.h, b.h);
-  return dfl{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
-}
-__device__ __forceinline__ cdf exact_sum(cdf a, cdf b) { return cdf{pair_add(a.r, b.r), pair_add(a.i, b.i)}; }
-__device__ __forceinline__ cx<float> negc(cx<float> z) { return cx<float>{-z.r, -z.i}; }
-__device__ __forceinline__ cdf negc(cdf z) { return cdf{neg(z.r), neg(z.i)}; }
-// acc += a * b for an input component b that is an exact FP32 number or a pair
-__device__ __forceinline__ void fma_px(dfl& acc, dfl a, float b) { fma_pf(acc, a, b); }
-__device__ __forceinline__ void fma_px(dfl& acc, dfl a, dfl b) { fma_pp(acc, a, b); }
-__device__ __forceinline__ void cfma_px(cdf& acc, cdf u, cx<float> x) { cfma_pf(acc, u, x); }
-__device__ __forceinline__ void cfma_px(cdf& acc, cdf u, cdf x) { cfma_pp(acc, u, x); }
-__device__ __forceinline__ void cfmac_px(cdf& acc, cdf u, cx<float> x) { cfmac_pf(acc, u, x); }
-__device__ __forceinline__ void cfmac_px(cdf& acc, cdf u, cdf x) { cfmac_pp(acc, u, x); }
+// A complex pair number with its real and imaginary parts as the lanes of packed
+// FP32 arithmetic: h = (re.h, im.h), l = (re.l, im.l).
+struct pk2 {
+  f2 h, l;
+};
 
-// link entry e = 3 a + b of direction mu at site s: float4 (re.h, im.h, re.l, im.l)
-__device__ __forceinline__ cdf ld_link_entry(const float4* __restrict__ gdf, long V, int mu, int e, long s) {
-  const float4 v = __ldg(gdf + ((long)mu * 9 + e) * V + s);
-  return cdf{dfl{v.x, v.z}, dfl{v.y, v.w}};
+__device__ __forceinline__ pk2 two_sum2(f2 a, f2 b) {
+  const f2 s = a + b;
+  const f2 bb = s - a;
+  return {s, (a - (s - bb)) + (b - bb)};
 }
-
-// multiply by the phase i^q, q runtime (exact; branch-free selects)
-__device__ __forceinline__ cdf mulp_sel(cdf z, int q);
-__device__ __forceinline__ cx<float> mulph_sel(cx<float> z, int q) {
+__device__ __forceinline__ void add_to(pk2& acc, pk2 a) {
+  const pk2 s = two_sum2(acc.h, a.h);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l + a.l);
+}
+// a pair of scalars broadcast to both lanes: h, -h and -l
+struct bc2 {
+  f2 h, nh, nl;
+};
+__device__ __forceinline__ bc2 bc_pair(float h, float l) {
+  return {f2_pack(h, h), f2_pack(-h, -h), f2_pack(-l, -l)};
+}
+// acc += a x for x exact in FP32, and for x a pair (l l, 2^-48 relative, is dropped);
+// ne = minus the rounding error of a.h x.h and the cross terms
+__device__ __forceinline__ void fma_px(pk2& acc, bc2 a, f2 x) {
+  const f2 p = a.h * x;
+  f2 ne = lfma(a.nh, x, p);
+  ne = lfma(a.nl, x, ne);
+  const pk2 s = two_sum2(acc.h, p);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l - ne);
+}
+__device__ __forceinline__ void fma_px(pk2& acc, bc2 a, pk2 x) {
+  const f2 p = a.h * x.h;
+  f2 ne = lfma(a.nh, x.h, p);
+  ne = lfma(a.nh, x.l, ne);
+  ne = lfma(a.nl, x.h, ne);
+  const pk2 s = two_sum2(acc.h, p);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l - ne);
+}
+// i x
+__device__ __forceinline__ f2 times_i(f2 x) {
+  const float2 v = f2_unpack(x);
+  return f2_pack(-v.y, v.x);
+}
+__device__ __forceinline__ pk2 times_i(pk2 x) { return {times_i(x.h), times_i(x.l)}; }
+// i^q x, q at run time (exact; branch-free selects)
+__device__ __forceinline__ f2 times_ph(f2 x, int q) {
+  const float2 v = f2_unpack(x);
   const bool sw = q & 1;
   const float sr = (q == 1 || q == 2) ? -1.f : 1.f, si = q >= 2 ? -1.f : 1.f;
-  return cx<float>{sr * (sw ? z.i : z.r), si * (sw ? z.r : z.i)};
+  return f2_pack(sr * (sw ? v.y : v.x), si * (sw ? v.x : v.y));
 }
-__device__ __forceinline__ cdf mulph_sel(cdf z, int q) { return mulp_sel(z, q); }
-__device__ __forceinline__ cdf mulp_sel(cdf z, int q) {
-  const bool sw = q & 1;
-  const float sr = (q == 1 || q == 2) ? -1.f : 1.f, si = q >= 2 ? -1.f : 1.f;
-  const dfl a = sw ? z.i : z.r, b = sw ? z.r : z.i;
-  return cdf{dfl{sr * a.h, sr * a.l}, dfl{si * b.h, si * b.l}};
+__device__ __forceinline__ pk2 times_ph(pk2 x, int q) { return {times_ph(x.h, q), times_ph(x.l, q)}; }
+// x + y as a pair (exact for FP32 x, y)
+__device__ __forceinline__ pk2 pair_sum(f2 x, f2 y) { return two_sum2(x, y); }
+__device__ __forceinline__ pk2 pair_sum(pk2 x, pk2 y) {
+  const pk2 s = two_sum2(x.h, y.h);
+  return {s.h, s.l + (x.l + y.l)};
 }
+
 __device__ __forceinline__ int gphase_rt(int mu, int r) {
   return mu == 0 ? 2 : mu == 1 ? (r == 0 ? 3 : 1) : mu == 2 ? (r == 0 ? 2 : 0) : 3;
 }
@@ -71,57 +97,53 @@ __device__ __forceinline__ int gphase_rt(int mu, int r) {
 // (U^dagger of U_mu(x - mu), psi(x - mu), projector 1 + gamma); link site sl.
 // One copy of the code serves all eight hops, so the kernel's loop over them
 // stays in the instruction cache.
-template <typename PT>  // input spinor components: exact FP32 (cx<float>) or pairs (cdf)
+template <typename PT>  // input spinor components: exact FP32 (f2) or pairs (pk2)
 __device__ __forceinline__ void hop_df_rt(const PT (&p)[12], const float4* __restrict__ gdf, long V, long sl, int mu,
-                                          bool fwd, float sign, cdf (&acc)[12]) {
+                                          bool fwd, float sign, pk2 (&acc)[12]) {
   const bool sw = mu >= 2;  // A_mu's row r holds its entry in column r (T, Z) or 1 - r (Y, X)
-  cdf h[2][3];
+  const f2 sg = f2_pack(sign, sign);
+  pk2 h[2][3];
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+  for (int r = 0; r < 2; ++r) {
+    // (1 - gamma): h = up - A dn; (1 + gamma): h = up + A dn  (exact as pairs for FP32 input)
+    const int q = (gphase_rt(mu, r) + (fwd ? 2 : 0)) & 3;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const PT dn = (sw != (r == 1)) ? p[9 + k] : p[6 + k];  // spin 2 + perm(r)
-      const PT lo = mulph_sel(dn, gphase_rt(mu, r));
-      const PT up = p[3 * r + k];
-      // (1 - gamma): h = up - A dn; (1 + gamma): h = up + A dn  (exact as pairs for FP32 input)
-      cdf t = exact_sum(up, fwd ? negc(lo) : lo);
-      t = cdf{dfl{sign * t.r.h, sign * t.r.l}, dfl{sign * t.i.h, sign * t.i.l}};
-      h[r][k] = t;
+      const pk2 t = pair_sum(p[3 * r + k], times_ph(dn, q));
+      h[r][k] = pk2{sg * t.h, sg * t.l};
     }
-  cdf w[2][3];
+  }
+  pk2 w[2][3];
+  const float4* lk = gdf + (long)mu * 9 * V + sl;  // entry e at lk + e V: (re.h, im.h, re.l, im.l)
+  const float cj = fwd ? 1.f : -1.f;               // backward hops take conj(U[b][a])
 #pragma unroll
   for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) w[r][a] = cdf{{0.f, 0.f}, {0.f, 0.f}};
-  const float cj = fwd ? 1.f : -1.f;  // backward hops take conj(U[b][a])
+    for (int a = 0; a < 3; ++a) w[r][a] = pk2{f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+  for (int b = 0; b < 3; ++b) {
+    const pk2 hi[2] = {times_i(h[0][b]), times_i(h[1][b])};
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      cdf u = ld_link_entry(gdf, V, mu, fwd ? 3 * a + b : 3 * b + a, sl);
-      u.i = dfl{cj * u.i.h, cj * u.i.l};
+    for (int a = 0; a < 3; ++a) {
+      const float4 u = __ldg(lk + (long)(fwd ? 3 * a + b : 3 * b + a) * V);
+      const bc2 ur = bc_pair(u.x, u.z), ui = bc_pair(cj * u.y, cj * u.w);
 #pragma unroll
-      for (int r = 0; r < 2; ++r) cfma_pp(w[r][a], u, h[r][b]);
+      for (int r = 0; r < 2; ++r) {
+        fma_px(w[r][a], ur, h[r][b]);
+        fma_px(w[r][a], ui, hi[r]);
+      }
     }
-  cdf lw[2][3];
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      add_to(acc[3 * r + k].r, w[r][k].r);
-      add_to(acc[3 * r + k].i, w[r][k].i);
-      // lower components: -+ A^dagger w, (A^dagger w)[perm r] = conj(phase r) w[r]
-      cdf l = mulp_sel(w[r][k], conjph(gphase_rt(mu, r)));
-      if (fwd) l = cdf{neg(l.r), neg(l.i)};
-      lw[r][k] = l;
-    }
+  }
+  // lower components: -+ A^dagger w, (A^dagger w)[perm r] = conj(phase r) w[r]
+  const int q0 = (4 - gphase_rt(mu, 0) + (fwd ? 2 : 0)) & 3, q1 = (4 - gphase_rt(mu, 1) + (fwd ? 2 : 0)) & 3;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const cdf l2 = sw ? lw[1][k] : lw[0][k], l3 = sw ? lw[0][k] : lw[1][k];
-    add_to(acc[6 + k].r, l2.r);
-    add_to(acc[6 + k].i, l2.i);
-    add_to(acc[9 + k].r, l3.r);
-    add_to(acc[9 + k].i, l3.i);
+    add_to(acc[k], w[0][k]);
+    add_to(acc[3 + k], w[1][k]);
+    const pk2 l0 = times_ph(w[0][k], q0), l1 = times_ph(w[1][k], q1);
+    add_to(acc[6 + k], sw ? l1 : l0);
+    add_to(acc[9 + k], sw ? l0 : l1);
   }
 }
 
@@ -137,38 +159,57 @@ struct DfArgs {
   int nrhs;
 };
 
-// clover chunk j of site s: float4 (r[2j].h, r[2j+1].h, r[2j].l, r[2j+1].l)
-__device__ __forceinline__ void ld_clover_pair(const float4* __restrict__ c4, long V, int j, long s, dfl& a, dfl& b) {
-  const float4 v = __ldg(c4 + (long)j * V + s);
-  a = dfl{v.x, v.z};
-  b = dfl{v.y, v.w};
-}
-
-// input spinor of site s as exact FP32 components or as pairs split from FP64
-__device__ __forceinline__ void ld_in(const float* in, long V, long s, cx<float> (&p)[12]) { ld_cx<float, 12>(in, V, s, p); }
-__device__ __forceinline__ void ld_in(const double* in, long V, long s, cdf (&p)[12]) {
-  const double2* q = reinterpret_cast<const double2*>(in);
+// chunks k0 .. k0 + N / 2 - 1 of a site: exact FP32 components, or pairs split from FP64
+template <int N>
+__device__ __forceinline__ void ld_in(const float* in, long V, long s, int k0, f2 (&p)[N]) {
+  const float4* q = reinterpret_cast<const float4*>(in) + (long)k0 * V + s;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const double2 v0 = __ldg(q + 2 * (k * V + s)), v1 = __ldg(q + 2 * (k * V + s) + 1);
-    p[2 * k] = cx2pair(v0.x, v0.y);
-    p[2 * k + 1] = cx2pair(v1.x, v1.y);
+  for (int k = 0; k < N / 2; ++k) {
+    const float4 v = __ldg(q + k * V);
+    p[2 * k] = f2_pack(v.x, v.y);
+    p[2 * k + 1] = f2_pack(v.z, v.w);
   }
 }
+__device__ __forceinline__ pk2 pk_of(double re, double im) {
+  const dfl a = d2pair(re), b = d2pair(im);
+  return {f2_pack(a.h, b.h), f2_pack(a.l, b.l)};
+}
+template <int N>
+__device__ __forceinline__ void ld_in(const double* in, long V, long s, int k0, pk2 (&p)[N]) {
+  const double2* q = reinterpret_cast<const double2*>(in) + 2 * ((long)k0 * V + s);
+#pragma unroll
+  for (int k = 0; k < N / 2; ++k) {
+    const double2 v0 = __ldg(q + 2 * k * V), v1 = __ldg(q + 2 * k * V + 1);
+    p[2 * k] = pk_of(v0.x, v0.y);
+    p[2 * k + 1] = pk_of(v1.x, v1.y);
+  }
+}
+__device__ __forceinline__ double2 pk2d(pk2 a) {
+  const float2 h = f2_unpack(a.h), l = f2_unpack(a.l);
+  return make_double2(pair2d(dfl{h.x, l.x}), pair2d(dfl{h.y, l.y}));
+}
 
+// Bound by FP32 issue and instruction fetch, not by memory (0.67 TB/s).  The
+// real and imaginary parts of a pair go through every step of the double-length
+// arithmetic alike, so they are the two lanes of packed FP32: half the
+// instructions and half the code of the scalar form (2.05 G -> 1.36 G warp
+// instructions for 6 right-hand sides at 48 x 24^3).  The two chiralities of the
+// clover term run through one copy of their code as well.  Three CTAs per SM
+// (168 registers): 2.84 -> 1.95 ms there; four 2.10 ms, two 2.50 ms.
 template <typename IN>
-__global__ void __launch_bounds__(128) k_dslash_df(DfArgs a) {
-  using PT = typename std::conditional<std::is_same<IN, float>::value, cx<float>, cdf>::type;
+__global__ void __launch_bounds__(128, 3) k_dslash_df(DfArgs a) {
+  using PT = typename std::conditional<std::is_same<IN, float>::value, f2, pk2>::type;
   const int rhs = a.nrhs == 1 ? 0 : (int)(blockIdx.x % a.nrhs);
   const int s = (a.nrhs == 1 ? blockIdx.x : blockIdx.x / a.nrhs) * blockDim.x + threadIdx.x;
   if (s >= a.g.V) return;
-  const long off = (long)rhs * NR_SPINOR * a.g.V;
+  const long V = a.g.V;
+  const long off = (long)rhs * NR_SPINOR * V;
   const IN* in = static_cast<const IN*>(a.in) + off;
   int c[4];
   site_coords(a.g, s, c);
-  cdf acc[12];
+  pk2 acc[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = cdf{{0.f, 0.f}, {0.f, 0.f}};
+  for (int k = 0; k < 12; ++k) acc[k] = pk2{f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
   // the eight hops through one copy of the hop code (direction and orientation at run time)
 #pragma unroll 1
   for (int hop = 0; hop < 8; ++hop) {
@@ -180,59 +221,55 @@ __global__ void __launch_bounds__(128) k_dslash_df(DfArgs a) {
     const int sn = fwd ? (cm + 1 < Lm ? s + stm : s - (Lm - 1) * stm) : (cm > 0 ? s - stm : s + (Lm - 1) * stm);
     const float sign = (mu == 0 && cm == (fwd ? Lm - 1 : 0)) ? a.bc : 1.f;
     PT p[12];
-    ld_in(in, a.g.V, sn, p);
-    hop_df_rt(p, a.gdf, a.g.V, fwd ? s : sn, mu, fwd, sign, acc);
+    ld_in(in, V, sn, 0, p);
+    hop_df_rt(p, a.gdf, V, fwd ? s : sn, mu, fwd, sign, acc);
   }
-  PT p[12];
-  ld_in(in, a.g.V, s, p);
-  // y = A p + i mu gamma5 p - acc / 2
-#pragma unroll
+  // y = A p + i mu gamma5 p - acc / 2, one chirality (gamma5 = -1, then +1) per turn
+  const dfl mus = ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu_odd : a.mu;
+  const f2 mhalf = f2_pack(-0.5f, -0.5f);
+#pragma unroll 1
   for (int h = 0; h < 2; ++h) {
-    cdf y[6];
+    PT p[6], ip[6];
+    ld_in(in, V, s, 3 * h, p);
+    pk2 y[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-      y[i].r = dfl{-0.5f * acc[6 * h + i].r.h, -0.5f * acc[6 * h + i].r.l};
-      y[i].i = dfl{-0.5f * acc[6 * h + i].i.h, -0.5f * acc[6 * h + i].i.l};
+      ip[i] = times_i(p[i]);
+      y[i] = pk2{mhalf * acc[i].h, mhalf * acc[i].l};
     }
-    // diagonal reals (chunks 18 h + 0..2 hold reals 36 h + 0..5)
+    // clover chunk k of a chirality: float4 (r[2k].h, r[2k+1].h, r[2k].l, r[2k+1].l)
+    const float4* c4 = a.cdf4 + (long)18 * h * V + s;
+    // diagonal reals (chunks 0..2)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      dfl d0, d1;
-      ld_clover_pair(a.cdf4, a.g.V, 18 * h + j, s, d0, d1);
-      fma_px(y[2 * j].r, d0, p[6 * h + 2 * j].r);
-      fma_px(y[2 * j].i, d0, p[6 * h + 2 * j].i);
-      fma_px(y[2 * j + 1].r, d1, p[6 * h + 2 * j + 1].r);
-      fma_px(y[2 * j + 1].i, d1, p[6 * h + 2 * j + 1].i);
+    for (int k = 0; k < 3; ++k) {
+      const float4 d = __ldg(c4 + k * V);
+      fma_px(y[2 * k], bc_pair(d.x, d.z), p[2 * k]);
+      fma_px(y[2 * k + 1], bc_pair(d.y, d.w), p[2 * k + 1]);
     }
-    // upper triangle (0,1),(0,2),...,(4,5): complex entry q at reals 6 + 2q, 7 + 2q = chunk 3 + q
+    // upper triangle (0,1),(0,2),...,(4,5): complex entry q = chunk 3 + q
     int q = 0;
 #pragma unroll
     for (int i = 0; i < 6; ++i)
 #pragma unroll
       for (int j = i + 1; j < 6; ++j) {
-        cdf u;
-        ld_clover_pair(a.cdf4, a.g.V, 18 * h + 3 + q, s, u.r, u.i);
+        const float4 u = __ldg(c4 + (3 + q) * V);
         ++q;
-        cfma_px(y[i], u, p[6 * h + j]);
-        cfmac_px(y[j], u, p[6 * h + i]);
+        const bc2 ur = bc_pair(u.x, u.z), ui = bc_pair(u.y, u.w), un = bc_pair(-u.y, -u.w);
+        fma_px(y[i], ur, p[j]);
+        fma_px(y[i], ui, ip[j]);
+        fma_px(y[j], ur, p[i]);
+        fma_px(y[j], un, ip[i]);
       }
-    // i mu gamma5 p, gamma5 = -1 on spins 0, 1 (h = 0), +1 on spins 2, 3
-    const dfl mus = ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu_odd : a.mu;
-    const dfl m = h == 0 ? neg(mus) : mus;
+    const bc2 m = bc_pair(h == 0 ? -mus.h : mus.h, h == 0 ? -mus.l : mus.l);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      fma_px(y[i].r, neg(m), p[6 * h + i].i);
-      fma_px(y[i].i, m, p[6 * h + i].r);
-    }
+    for (int i = 0; i < 6; ++i) fma_px(y[i], m, ip[i]);
     // FP64 output: h + l (or sub - (h + l))
     double2* o = reinterpret_cast<double2*>(a.out + off);
     const double2* sb = a.sub ? reinterpret_cast<const double2*>(a.sub + off) : nullptr;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const int chunk = 3 * h + k;  // complex numbers 6 h + 2 k, 6 h + 2 k + 1
-      const long i0 = 2 * ((long)chunk * a.g.V + s);
-      double2 v0 = make_double2(pair2d(y[2 * k].r), pair2d(y[2 * k].i));
-      double2 v1 = make_double2(pair2d(y[2 * k + 1].r), pair2d(y[2 * k + 1].i));
+      const long i0 = 2 * ((long)(3 * h + k) * V + s);  // complex numbers 6 h + 2 k, 6 h + 2 k + 1
+      double2 v0 = pk2d(y[2 * k]), v1 = pk2d(y[2 * k + 1]);
       if (sb) {
         const double2 b0 = sb[i0], b1 = sb[i0 + 1];
         v0 = make_double2(b0.x - v0.x, b0.y - v0.y);
@@ -241,6 +278,8 @@ __global__ void __launch_bounds__(128) k_dslash_df(DfArgs a) {
       o[i0] = v0;
       o[i0 + 1] = v1;
     }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) acc[i] = acc[6 + i];  // the other chirality next
   }
 }
 
