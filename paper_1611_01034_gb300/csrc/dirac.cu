@@ -11,7 +11,10 @@
 // (Q_mu_nu - Q_nu_mu) is block diagonal in chirality because gamma_mu gamma_nu
 // is; it is stored as two Hermitian 6x6 blocks.  Hops across the T boundary
 // carry the factor bc_t.
+#include <type_traits>
+
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 #include "tm_stencil.cuh"
 
 namespace tmamg {
@@ -293,43 +296,112 @@ struct DslashArgs {
   T rho;  // odd sites carry mu + rho (Sec. 2: a different twisted mass on even and odd sites)
 };
 
-// right-hand sides vary fastest over the CTAs so the links and clover of a site
-// block are read from DRAM once and reused from L2 by the other right-hand sides
-template <typename T, bool RES>
-__global__ void __launch_bounds__(128) k_dslash(DslashArgs<T> a) {
-  const int rhs = a.nrhs == 1 ? 0 : (int)(blockIdx.x % a.nrhs);
-  const int s = (a.nrhs == 1 ? blockIdx.x : blockIdx.x / a.nrhs) * blockDim.x + threadIdx.x;
+// RB right-hand sides per thread share the link and clover loads and the third
+// link rows; groups of them vary fastest over the CTAs, so that the links and
+// clover of a site block are read from DRAM once.  FP32 waits on spinor loads
+// (DRAM at 37 %, issue 45 %) and gains from four CTAs per SM: 12 right-hand
+// sides at 48 x 24^3, 835 us -> 681 us (one per thread), 630 us (two).
+// Measured and left out: three per thread 624 us, four 749 us, two as packed
+// lanes 701 us (packing moves), five CTAs per SM 691 us, 64-thread CTAs 637 us.
+// FP64 is bound by the FP64 units and keeps one per thread, unbounded registers.
+template <typename T, bool RES, int RB>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_dslash(DslashArgs<T> a) {
+  const int ngrp = a.nrhs / RB;
+  const int grp = ngrp == 1 ? 0 : (int)(blockIdx.x % ngrp);
+  const int s = (ngrp == 1 ? blockIdx.x : blockIdx.x / ngrp) * blockDim.x + threadIdx.x;
   if (s >= a.g.V) return;
-  const long off = (long)rhs * NR_SPINOR * a.g.V;
+  const long fs = (long)NR_SPINOR * a.g.V;
+  const long off = (long)grp * RB * fs;
   const T* in = a.in + off;
   int c[4];
   site_coords(a.g, s, c);
-  cx<T> acc[12];
-  all_hops_global<T>(in, a.gauge, a.g, s, c, a.bc, acc);
-  cx<T> p[12], y[12];
-  ld_cx<T, 12>(in, a.g.V, s, p);
-  site_diag<T>(a.clover, a.g.V, s, ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu + a.rho : a.mu, p, y);
-  const T half = T(0.5);
+  cx<T> acc[RB][12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) y[k] = y[k] - half * acc[k];
-  if constexpr (RES) {
-    cx<T> bb[12];
-    ld_cx<T, 12>(a.b + off, a.g.V, s, bb);
+  for (int j = 0; j < RB; ++j)
 #pragma unroll
-    for (int k = 0; k < 12; ++k) y[k] = bb[k] - y[k];
+    for (int k = 0; k < 12; ++k) acc[j][k] = cx<T>{0, 0};
+  auto hop = [&](auto MUC, auto FWD) {
+    constexpr int MU = decltype(MUC)::value;
+    constexpr bool fwd = decltype(FWD)::value;
+    const int sn = fwd ? nb_fwd(a.g, s, c, MU) : nb_bwd(a.g, s, c, MU);
+    cx<T> p[RB][12];
+#pragma unroll
+    for (int j = 0; j < RB; ++j) ld_cx<T, 12>(in + j * fs, a.g.V, sn, p[j]);
+    cx<T> z[6];
+    ld_cx<T, 6>(a.gauge + (long)MU * NR_LINK * a.g.V, a.g.V, fwd ? s : sn, z);
+    Link<T> U;
+    link_from_rows(z, U);
+    if (MU == 0 && c[0] == (fwd ? a.g.L[0] - 1 : 0)) {
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) U.u[r][k] = a.bc * U.u[r][k];
+    }
+#pragma unroll
+    for (int j = 0; j < RB; ++j) hop_lanes<T, T, MU, fwd>([&](int i) { return p[j][i]; }, U, acc[j]);
+  };
+  using std::integral_constant;
+  hop(integral_constant<int, 0>{}, std::true_type{});
+  hop(integral_constant<int, 0>{}, std::false_type{});
+  hop(integral_constant<int, 1>{}, std::true_type{});
+  hop(integral_constant<int, 1>{}, std::false_type{});
+  hop(integral_constant<int, 2>{}, std::true_type{});
+  hop(integral_constant<int, 2>{}, std::false_type{});
+  hop(integral_constant<int, 3>{}, std::true_type{});
+  hop(integral_constant<int, 3>{}, std::false_type{});
+  // acc = A p + i mu gamma5 p - acc / 2
+  const T mus = ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu + a.rho : a.mu;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    T m[36];
+    ld_re<T, 36>(a.clover + (long)h * 36 * a.g.V, a.g.V, s, m);
+#pragma unroll
+    for (int j = 0; j < RB; ++j) {
+      cx<T> p[6];
+      ld_cx<T, 6>(in + j * fs + (long)h * 12 * a.g.V, a.g.V, s, p);
+      cx<T>* y = acc[j] + 6 * h;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) y[k] = T(-0.5) * y[k];
+      herm6_lanes<T, T>(m, h == 0 ? -mus : mus, p, y);
+    }
   }
-  st_cx<T, 12>(a.out + off, a.g.V, s, y);
+#pragma unroll
+  for (int j = 0; j < RB; ++j) {
+    const long o = off + j * fs;
+    if constexpr (RES) {
+      cx<T> bb[12];
+      ld_cx<T, 12>(a.b + o, a.g.V, s, bb);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[j][k] = bb[k] - acc[j][k];
+    }
+    st_cx<T, 12>(a.out + o, a.g.V, s, acc[j]);
+  }
+}
+
+template <typename T, int RB>
+void dslash_r(const DslashArgs<T>& a, cudaStream_t st) {
+  dim3 grid((unsigned)((a.g.V + 127) / 128) * (unsigned)(a.nrhs / RB));
+  if (a.b)
+    k_dslash<T, true, RB><<<grid, 128, 0, st>>>(a);
+  else
+    k_dslash<T, false, RB><<<grid, 128, 0, st>>>(a);
 }
 
 template <typename T>
 void launch_dslash(const T* gauge, const T* clover, const T* in, T* out, const T* b, const Lat& g, double mu,
                    double bc_t, int nrhs, cudaStream_t st, double rho) {
   DslashArgs<T> a{gauge, clover, in, out, b, g, (T)mu, (T)bc_t, nrhs, (T)rho};
-  dim3 grid((unsigned)((g.V + 127) / 128) * (unsigned)nrhs);
-  if (b)
-    k_dslash<T, true><<<grid, 128, 0, st>>>(a);
-  else
-    k_dslash<T, false><<<grid, 128, 0, st>>>(a);
+  if constexpr (sizeof(T) == 4) {
+    a.nrhs = nrhs & ~1;
+    if (a.nrhs) dslash_r<T, 2>(a, st);
+    if (!(nrhs & 1)) return;
+    const long off = (long)a.nrhs * NR_SPINOR * g.V;
+    a.in += off;
+    a.out += off;
+    if (b) a.b += off;
+    a.nrhs = 1;
+  }
+  dslash_r<T, 1>(a, st);
 }
 template void launch_dslash<double>(const double*, const double*, const double*, double*, const double*,
                                     const Lat&, double, double, int, cudaStream_t, double);
