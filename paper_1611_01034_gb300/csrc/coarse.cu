@@ -12,7 +12,11 @@
 // chi * N_v + i.  D_c is stored per coarse site as 9 blocks (self, then
 // forward/backward per direction T, Z, Y, X), each column-major [col][row] so
 // that one thread per row reads consecutive addresses.
+#include <algorithm>
+#include <type_traits>
+
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 #include "tm_stencil.cuh"
 
 namespace tmamg {
@@ -125,6 +129,7 @@ __device__ __forceinline__ void ld_pcol(const void* __restrict__ P, int i, long 
     ld_cx16<T, S, 12>(static_cast<const unsigned short*>(P) + (long)i * NR_SPINOR * V, V, s, p);
 }
 
+// one right-hand side, FP64 and narrow aggregates (k_restrict_l takes other FP32 batches)
 template <typename T, int S>
 __global__ void k_restrict(const void* __restrict__ P, const T* __restrict__ fine, T* __restrict__ coarse,
                            AggGeom ag, int nrhs) {
@@ -169,22 +174,12 @@ __global__ void k_restrict(const void* __restrict__ P, const T* __restrict__ fin
   }
 }
 
-template <typename T>
-void launch_restrict(const T* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st,
-                     const void* P16, int p16) {
-  const int threads = (ag.asites + 31) / 32 * 32;
-  dim3 grid((unsigned)ag.gc.V * (unsigned)nrhs);
-  if (P16 && p16 == ST_F16)
-    k_restrict<T, ST_F16><<<grid, threads, 0, st>>>(P16, fine, coarse, ag, nrhs);
-  else if (P16 && p16 == ST_BF16)
-    k_restrict<T, ST_BF16><<<grid, threads, 0, st>>>(P16, fine, coarse, ag, nrhs);
-  else
-    k_restrict<T, ST_NATIVE><<<grid, threads, 0, st>>>(P, fine, coarse, ag, nrhs);
-}
-
 // ===========================================================================
 // prolongation  fine(x, comp in chi) (+)= sum_i P_i(x, comp) coarse(a(x), chi*Nv + i)
 // ===========================================================================
+// One right-hand side, FP64, and aggregates narrower than four sites in X, whose
+// site order would break up the loads of k_prolong_l (which takes FP32 batches
+// on the others): threads in lattice order.
 // RG right-hand sides per thread: every P value loaded serves all of them
 // (with one right-hand side per thread the CTAs of the other right-hand sides
 // read P again through L2)
@@ -232,9 +227,247 @@ __global__ void __launch_bounds__(128) k_prolong(const void* __restrict__ P, con
     if (j < R) st_cx<T, 12>(f + (long)j * NR_SPINOR * V, V, s, out[j]);
 }
 
-template <typename T, int S>
-void prolong_s(const void* P, const T* coarse, T* fine, const AggGeom& ag, int nrhs, bool accumulate,
+// ===========================================================================
+// FP32 transfers for a batch: pairs of right-hand sides as the lanes of packed
+// FP32, one chirality per CTA, and P, the largest operand, read from DRAM once
+// for all right-hand sides of a CTA.
+// ===========================================================================
+// half h (one chirality, 6 complex = 3 chunks) of column i of P at site s
+template <int S>
+__device__ __forceinline__ void ld_phalf(const void* __restrict__ P, int i, int h, long V, long s, cx<float> (&p)[6]) {
+  const long off = (long)i * NR_SPINOR * V + (long)h * 12 * V;
+  if constexpr (S == ST_NATIVE)
+    ld_cx<float, 6>(static_cast<const float*>(P) + off, V, s, p);
+  else
+    ld_cx16<float, S, 6>(static_cast<const unsigned short*>(P) + off, V, s, p);
+}
+
+constexpr int kTrSites = 128;    // sites per CTA of the prolongation
+#ifndef TRC
+#define TRC 4
+#endif
+constexpr int kTrThreads = 256;  // of the restriction
+constexpr int kTrPairs = 12;     // pairs per CTA of the restriction
+
+// Restriction: CTA = one aggregate, one chirality and up to kTrPairs pairs;
+// thread = site.  Four columns at a time, pair after pair: 16 sums per thread, reduced over the warp by a reduce-scatter
+// that leaves each lane one of them; the warps' sums meet in shared memory at the
+// end.  Bound by the latency of the P loads (from L1 and L2 for all pairs but the
+// first), so the batch of columns is what 64 registers (32 warps per SM) hold: 6
+// right-hand sides, N_v 24, FP16 P at 48 x 24^3, 716 -> 540 us; 8 columns with 80
+// registers 574 us, 128 registers 650 us; the fine vectors staged in shared memory
+// and P read once for three pairs, 168 registers, 570 us.
+template <int S>
+__global__ void __launch_bounds__(kTrThreads, 4) k_restrict_l(const void* __restrict__ P, const float* __restrict__ fine,
+                                                             float* __restrict__ coarse, AggGeom ag, int nrhs,
+                                                             int ngrp) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* red = reinterpret_cast<float*>(smem_raw);  // [ceil(nv / C)][pairs][warps][16]
+  const int h = blockIdx.x & 1, a = (blockIdx.x >> 1) / ngrp;
+  constexpr int C = 4;  // columns at a time
+  const int p0 = ((blockIdx.x >> 1) % ngrp) * kTrPairs, pairs = min(kTrPairs, (nrhs + 1) / 2 - p0);
+  const int nv = ag.nv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const long V = ag.g.V, fs = (long)NR_SPINOR * V;
+  int lc[4], c[4];
+  const int s0 = agg_site(ag, a, min((int)threadIdx.x, ag.asites - 1), lc, c);
+  const float* f = fine + (long)h * 12 * V;
+  const int nib = (nv + C - 1) / C;
+  for (int ib = 0; ib < nib; ++ib) {
+#pragma unroll 1
+    for (int q = 0; q < pairs; ++q) {
+      const int r = 2 * (p0 + q);
+      const float* f0 = f + r * fs;
+      const float* f1 = r + 1 < nrhs ? f0 + fs : f0;
+      cx<f2> acc[C];
+#pragma unroll
+      for (int ii = 0; ii < C; ++ii) acc[ii] = czero<f2>();
+#pragma unroll 1
+      for (int l = threadIdx.x; l < ag.asites; l += blockDim.x) {
+        const int s = l == (int)threadIdx.x ? s0 : agg_site(ag, a, l, lc, c);
+        cx<f2> z[6];
+        ld_lanes<f2, 6, float>(f0, f1, V, s, z);
+#pragma unroll
+        for (int ii = 0; ii < C; ++ii) {
+          if (ib * C + ii < nv) {
+            cx<float> p[6];
+            ld_phalf<S>(P, ib * C + ii, h, V, s, p);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) lcfmac(acc[ii], p[k], z[k]);
+          }
+        }
+      }
+      float v[16];  // sum k = 4 ii + 2 (second right-hand side) + (imaginary part)
+#pragma unroll
+      for (int ii = 0; ii < C; ++ii) {
+        const float2 x = f2_unpack(acc[ii].r), y = f2_unpack(acc[ii].i);
+        v[4 * ii] = x.x;
+        v[4 * ii + 1] = y.x;
+        v[4 * ii + 2] = x.y;
+        v[4 * ii + 3] = y.y;
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int m = 0; m < o; ++m)
+          v[m] = (hi ? v[o + m] : v[m]) + __shfl_xor_sync(0xffffffffu, hi ? v[m] : v[o + m], o);
+      }
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+      if (lane < 16) red[((ib * pairs + q) * nw + warp) * 16 + lane] = v[0];
+    }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nib * pairs * 16; e += blockDim.x) {
+    const int k = e & 15, q = (e >> 4) % pairs, i = (e >> 4) / pairs * C + (k >> 2);
+    const int r = 2 * (p0 + q) + ((k >> 1) & 1);
+    if (i >= nv || r >= nrhs) continue;
+    const float* src = red + (e >> 4) * nw * 16 + k;
+    float sum = src[0];
+    for (int w = 1; w < nw; ++w) sum += src[w * 16];
+    coarse[(((long)r * ag.gc.V + a) * 2 * nv + h * nv + i) * 2 + (k & 1)] = sum;
+  }
+}
+
+// Prolongation: CTA = kTrSites sites of whole aggregates (or a chunk of one) and one
+// chirality, thread = site; the coarse vectors of its aggregates wait in shared
+// memory as lane pairs, every P value serves 2 PR right-hand sides.
+template <int S, int PR, bool ACC>
+__global__ void __launch_bounds__(kTrSites, 4) k_prolong_l(const void* __restrict__ P, const float* __restrict__ coarse,
+                                                           float* __restrict__ fine, AggGeom ag, int nrhs, int ngrp,
+                                                           int napc, int cpa) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<f2>* es = reinterpret_cast<cx<f2>*>(smem_raw);  // [napc][nv][PR]
+  const int nv = ag.nv, h = blockIdx.x & 1;
+  int b = blockIdx.x >> 1;
+  const int r0 = (b % ngrp) * 2 * PR;
+  b /= ngrp;
+  const int a0 = (b / cpa) * napc, l0 = (b % cpa) * kTrSites;  // cpa chunks per aggregate or napc aggregates per CTA
+  const long V = ag.g.V, fs = (long)NR_SPINOR * V, cs = (long)ag.gc.V * 2 * nv;
+  for (int e = threadIdx.x; e < napc * nv * PR; e += kTrSites) {
+    const int q = e % PR, i = (e / PR) % nv, a = a0 + e / (PR * nv), r = r0 + 2 * q;
+    if (a >= ag.gc.V || r >= nrhs) continue;
+    const cx<float>* src = reinterpret_cast<const cx<float>*>(coarse) + r * cs + (long)a * 2 * nv + h * nv + i;
+    const cx<float> u = src[0], v = r + 1 < nrhs ? src[cs] : cx<float>{0.f, 0.f};
+    st_shared(es + e, cx<f2>{f2_pack(u.r, v.r), f2_pack(u.i, v.i)});
+  }
+  __syncthreads();
+  const int al = cpa > 1 ? 0 : threadIdx.x / ag.asites, l = cpa > 1 ? l0 + threadIdx.x : threadIdx.x % ag.asites;
+  if (al >= napc || l >= ag.asites || a0 + al >= ag.gc.V) return;
+  int lc[4], c[4];
+  const int s = agg_site(ag, a0 + al, l, lc, c);
+  cx<f2> out[PR][6];
+  float* f = fine + (long)h * 12 * V;
+#pragma unroll
+  for (int q = 0; q < PR; ++q) {
+    const int r = r0 + 2 * q;
+    if (ACC && r < nrhs) {
+      ld_lanes<f2, 6, float>(f + r * fs, f + (r + 1 < nrhs ? r + 1 : r) * fs, V, s, out[q]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) out[q][k] = czero<f2>();
+    }
+  }
+  const cx<f2>* ea = es + (size_t)al * nv * PR;
+#pragma unroll 3
+  for (int i = 0; i < nv; ++i) {
+    cx<float> p[6];
+    ld_phalf<S>(P, i, h, V, s, p);
+#pragma unroll
+    for (int q = 0; q < PR; ++q) {
+      if (r0 + 2 * q >= nrhs) continue;
+      const cx<f2> e = ld_shared(ea + i * PR + q);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) lcfma(out[q][k], p[k], e);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < PR; ++q) {
+    const int r = r0 + 2 * q;
+    if (r + 1 < nrhs) {
+      st_lanes<f2, 6, float>(f + r * fs, f + (r + 1) * fs, V, s, out[q]);
+    } else if (r < nrhs) {
+      cx<float> one[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) one[k] = cx<float>{f2_unpack(out[q][k].r).x, f2_unpack(out[q][k].i).x};
+      st_cx<float, 6>(f + r * fs, V, s, one);
+    }
+  }
+}
+
+// pairs per CTA: the fewest CTAs per aggregate with up to 3 pairs each, evenly filled
+static int transfer_pairs(int nrhs, int* ngrp) {
+  const int pairs = (nrhs + 1) / 2;
+  *ngrp = (pairs + 2) / 3;
+  return (pairs + *ngrp - 1) / *ngrp;
+}
+
+template <int S>
+void restrict_l(const void* P, const float* fine, float* coarse, const AggGeom& ag, int nrhs, cudaStream_t st) {
+  const int pairs = (nrhs + 1) / 2, ngrp = (pairs + kTrPairs - 1) / kTrPairs;
+  const int threads = std::min(kTrThreads, (ag.asites + 31) / 32 * 32);
+  const size_t smem = (size_t)((ag.nv + 3) / 4) * std::min(pairs, kTrPairs) * (threads / 32) * 16 * sizeof(float);
+  k_restrict_l<S><<<(unsigned)ag.gc.V * (unsigned)ngrp * 2u, threads, smem, st>>>(P, fine, coarse, ag, nrhs, ngrp);
+}
+
+template <int S, int PR>
+void prolong_l(const void* P, const float* coarse, float* fine, const AggGeom& ag, int nrhs, int ngrp, bool acc,
                cudaStream_t st) {
+  const int cpa = (ag.asites + kTrSites - 1) / kTrSites, napc = cpa > 1 ? 1 : kTrSites / ag.asites;
+  const size_t smem = (size_t)napc * ag.nv * PR * sizeof(cx<f2>);
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_prolong_l<S, PR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_prolong_l<S, PR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    attr = true;
+  }
+  const unsigned grid = (unsigned)((ag.gc.V + napc - 1) / napc * cpa) * (unsigned)ngrp * 2u;
+  if (acc)
+    k_prolong_l<S, PR, true><<<grid, kTrSites, smem, st>>>(P, coarse, fine, ag, nrhs, ngrp, napc, cpa);
+  else
+    k_prolong_l<S, PR, false><<<grid, kTrSites, smem, st>>>(P, coarse, fine, ag, nrhs, ngrp, napc, cpa);
+}
+template <int S>
+void prolong_s(const void* P, const float* coarse, float* fine, const AggGeom& ag, int nrhs, bool acc,
+               cudaStream_t st) {
+  int ngrp;
+  switch (transfer_pairs(nrhs, &ngrp)) {
+    case 1: return prolong_l<S, 1>(P, coarse, fine, ag, nrhs, ngrp, acc, st);
+    case 2: return prolong_l<S, 2>(P, coarse, fine, ag, nrhs, ngrp, acc, st);
+    default: return prolong_l<S, 3>(P, coarse, fine, ag, nrhs, ngrp, acc, st);
+  }
+}
+
+template <typename T, int S>
+void restrict_any(const void* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st) {
+  if constexpr (std::is_same<T, float>::value) {
+    // pairs beat one right-hand side per CTA from two on (6: 540 against 716 us); one
+    // alone is 1 to 9 % faster in the form that keeps both chiralities in a thread,
+    // as are half-empty warps (2^4 aggregates, 3 right-hand sides: 146 and 150 us)
+    if (nrhs > 1 && ag.agg[3] >= 4) return restrict_l<S>(P, fine, coarse, ag, nrhs, st);
+  }
+  const int threads = (ag.asites + 31) / 32 * 32;
+  k_restrict<T, S><<<(unsigned)ag.gc.V * (unsigned)nrhs, threads, 0, st>>>(P, fine, coarse, ag, nrhs);
+}
+
+template <typename T>
+void launch_restrict(const T* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st,
+                     const void* P16, int p16) {
+  if (P16 && p16 == ST_F16)
+    restrict_any<T, ST_F16>(P16, fine, coarse, ag, nrhs, st);
+  else if (P16 && p16 == ST_BF16)
+    restrict_any<T, ST_BF16>(P16, fine, coarse, ag, nrhs, st);
+  else
+    restrict_any<T, ST_NATIVE>(P, fine, coarse, ag, nrhs, st);
+}
+
+template <typename T, int S>
+void prolong_any(const void* P, const T* coarse, T* fine, const AggGeom& ag, int nrhs, bool accumulate,
+                 cudaStream_t st) {
+  if constexpr (std::is_same<T, float>::value) {
+    // 2^4 aggregates, 3 right-hand sides, FP32 P at 24 x 24 x 16^2: 61.5 us in lattice
+    // order, 63 in aggregate order; 4^4 and 2 right-hand sides at 8^4: 8.4 and 6.4 us
+    if (nrhs > 1 && ag.agg[3] >= 4) return prolong_s<S>(P, coarse, fine, ag, nrhs, accumulate, st);
+  }
   constexpr int RG = sizeof(T) == 4 ? 3 : 1;
   const unsigned ngrp = (unsigned)((nrhs + RG - 1) / RG);
   dim3 grid((unsigned)((ag.g.V + 127) / 128) * ngrp);
@@ -248,11 +481,11 @@ template <typename T>
 void launch_prolong(const T* P, const T* coarse, T* fine, const AggGeom& ag, int nrhs, bool accumulate,
                     cudaStream_t st, const void* P16, int p16) {
   if (P16 && p16 == ST_F16)
-    prolong_s<T, ST_F16>(P16, coarse, fine, ag, nrhs, accumulate, st);
+    prolong_any<T, ST_F16>(P16, coarse, fine, ag, nrhs, accumulate, st);
   else if (P16 && p16 == ST_BF16)
-    prolong_s<T, ST_BF16>(P16, coarse, fine, ag, nrhs, accumulate, st);
+    prolong_any<T, ST_BF16>(P16, coarse, fine, ag, nrhs, accumulate, st);
   else
-    prolong_s<T, ST_NATIVE>(P, coarse, fine, ag, nrhs, accumulate, st);
+    prolong_any<T, ST_NATIVE>(P, coarse, fine, ag, nrhs, accumulate, st);
 }
 
 // 16-bit copy of n_cx FP32 complex numbers (element order kept)

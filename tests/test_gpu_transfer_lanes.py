@@ -1,0 +1,47 @@
+"""FP32 restriction and prolongation of batches (pairs of right-hand sides share a thread).
+
+Every right-hand side against the oracle's P: one alone, whole pairs, an odd one out, and more pairs than
+one CTA takes; aggregates below a warp, of one CTA and beyond one CTA; N_v that leaves columns over.
+FP32 sums of at most 6144 terms: 1e-5; a 16-bit P rounds every entry by 2^-11 (FP16) or 2^-8 (BF16).
+"""
+import numpy as np
+import pytest
+
+import inputs
+import paper_1611_01034_gb300 as tm
+from oracle.coarse import Interpolation
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from tests.gpu_helpers import GPU, rel  # noqa: E402
+
+F32 = tm.TM_F32
+
+
+@pytest.mark.parametrize("L,agg,nv,nrhs", [((4, 4, 8, 8), (2, 2, 2, 2), 5, 1), ((4, 4, 8, 8), (2, 2, 2, 2), 7, 5),
+                                           ((8, 8, 8, 8), (4, 4, 4, 4), 9, 1), ((8, 8, 8, 8), (4, 4, 4, 4), 8, 27),
+                                           ((8, 8, 16, 12), (4, 4, 4, 6), 6, 3), ((8, 8, 16, 16), (4, 4, 8, 8), 3, 2),
+                                           ((4, 4, 4, 8), (2, 1, 1, 4), 5, 6)])
+@pytest.mark.parametrize("prec,tol", [(tm.TM_F32, 1e-5), (tm.TM_F16, 5e-3), (tm.TM_BF16, 3e-2)])
+def test_transfer_batches(L, agg, nv, nrhs, prec, tol):
+    U = inputs.gauge_field(L, 0.3, 3)
+    g = GPU(U, m0=0.1, c_sw=1.0, mu=0.1, nv=nv, agg=agg, sap_block=(2, 2, 2, 2),
+            cycle_prec=F32, max_rhs=nrhs, transfer_prec=prec)
+    tv = inputs.random_test_vectors(L, nv, 4)
+    tm.tm_setup_from_vectors(g.h, tv)
+    P = Interpolation(tv, agg)
+    psi, c = inputs.gaussian_spinor(L, 5, nrhs), inputs.random_coarse_vectors(g.Lc, 2 * nv, nrhs, 6)
+    fc, ff = g.field(1, F32, nrhs), g.pack(0, F32, psi, nrhs)
+    tm.tm_restrict(g.h, F32, ff, fc, nrhs)
+    got = g.unpack(1, F32, fc, c.shape, nrhs)
+    tm.tm_prolong(g.h, F32, g.pack(1, F32, c, nrhs), ff, nrhs, 1)  # psi += P c
+    acc = g.unpack(0, F32, ff, psi.shape, nrhs)
+    fz = g.field(0, F32, nrhs)
+    tm.tm_prolong(g.h, F32, g.pack(1, F32, c, nrhs), fz, nrhs, 0)
+    new = g.unpack(0, F32, fz, psi.shape, nrhs)
+    for r in range(nrhs):
+        assert rel(got[r], P.restrict(psi[r])) <= tol
+        want = P.prolong(c[r])
+        assert rel(new[r], want) <= tol
+        assert rel(acc[r], psi[r] + want) <= tol
