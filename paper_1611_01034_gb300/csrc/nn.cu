@@ -7,228 +7,356 @@
 //
 // W[o][i][d] a complex 4 x 4 spin matrix acting trivially on colour, the
 // fermion boundary factor on hops across T.  The preconditioner applies
-// z = B(v) + N(v - D B(v)).  Kernels: the layer (one thread per site and
-// output channel, FP32 arithmetic, hidden channels stored in FP32 or FP16),
-// the same kernel with conjugate-transposed, direction-reversed weights as the
-// adjoint layer, and the weight gradient sum_x g_o(x) (T_d psi_i)(x)^dagger
-// (per-CTA partial sums over a tile of sites, reduced in FP64 in a second pass).
+// z = B(v) + N(v - D B(v)).
+//
+// All kernels are bound by FP32 arithmetic (issue 55 to 72 %, FP32 pipe 50 to
+// 67 %).  A transport acts on colour and position, a weight on spin, so they
+// commute and every transport is done on the single-channel side: L1 and the
+// adjoint of L2 (1 -> 8) transport the input once for all 8 outputs, L2 (8 -> 1)
+// sums its channels at the neighbour before transporting, and the gradients use
+// <g, T_d h> = <T_d^+ g, h>.  16 samples on 16^4: L1 1.19 -> 0.79 ms, L2 1.14 ->
+// 0.74 ms, gradients 2.53 + 1.79 -> 0.98 + 0.98 ms, inference and gradient
+// together 10.7 -> 6.0 ms.
 #include <cuda_fp16.h>
 
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 
 namespace tmamg {
 
 namespace {
 
 constexpr int kNdir = 9;
+constexpr int kC = kNnHidden;
 
-// fine field in the library's chunked layout: rhs r, channel c at f + (r * C + c) * 24 V
-struct FineIn {
-  const float* f;
-  int C;
-  __device__ __forceinline__ void load(long V, int r, int c, long s, cx<float> (&p)[12]) const {
-    ld_cx<float, 12>(f + ((long)r * C + c) * NR_SPINOR * V, V, s, p);
-  }
-};
-struct FineOut {
-  float* f;
-  int C;
-  __device__ __forceinline__ void store(long V, int r, int c, long s, const cx<float> (&p)[12], bool acc) const {
-    float* base = f + ((long)r * C + c) * NR_SPINOR * V;
-    if (acc) {
-      cx<float> q[12];
-      ld_cx<float, 12>(base, V, s, q);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) q[k] = q[k] + p[k];
-      st_cx<float, 12>(base, V, s, q);
-    } else {
-      st_cx<float, 12>(base, V, s, p);
-    }
-  }
-};
-// hidden channels: [rhs][C][V][12 complex] contiguous per site, FP32 or FP16
+// hidden channels: [rhs][8][component 12][V] complex, FP32 or FP16 (re, im)
 template <typename Th>
-struct HiddenIn {
-  const Th* f;
-  int C;
-  __device__ __forceinline__ void load(long V, int r, int c, long s, cx<float> (&p)[12]) const {
-    const Th* q = f + (((long)r * C + c) * V + s) * 24;
-    if constexpr (sizeof(Th) == 4) {
-      const float4* v = reinterpret_cast<const float4*>(q);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const float4 a = v[k];
-        p[2 * k] = cx<float>{a.x, a.y};
-        p[2 * k + 1] = cx<float>{a.z, a.w};
-      }
-    } else {
-      const __half2* v = reinterpret_cast<const __half2*>(q);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const float2 a = __half22float2(v[k]);
-        p[k] = cx<float>{a.x, a.y};
-      }
-    }
-  }
+struct Cx2;
+template <>
+struct Cx2<float> {
+  using V = float2;
+  static __device__ __forceinline__ cx<float> get(float2 v) { return {v.x, v.y}; }
+  static __device__ __forceinline__ float2 put(cx<float> z) { return make_float2(z.r, z.i); }
 };
-template <typename Th>
-struct HiddenOut {
-  Th* f;
-  int C;
-  __device__ __forceinline__ void store(long V, int r, int c, long s, const cx<float> (&p)[12], bool) const {
-    Th* q = f + (((long)r * C + c) * V + s) * 24;
-    if constexpr (sizeof(Th) == 4) {
-      float4* v = reinterpret_cast<float4*>(q);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) v[k] = make_float4(p[2 * k].r, p[2 * k].i, p[2 * k + 1].r, p[2 * k + 1].i);
-    } else {
-      __half2* v = reinterpret_cast<__half2*>(q);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) v[k] = __floats2half2_rn(p[k].r, p[k].i);
-    }
+template <>
+struct Cx2<__half> {
+  using V = __half2;
+  static __device__ __forceinline__ cx<float> get(__half2 v) {
+    const float2 f = __half22float2(v);
+    return {f.x, f.y};
   }
+  static __device__ __forceinline__ __half2 put(cx<float> z) { return __floats2half2_rn(z.r, z.i); }
 };
 
-// phi = T_d psi_c(x) at site s (coordinates cs) of rhs r
-template <class In>
-__device__ __forceinline__ void transported(const In& in, const float* __restrict__ gauge, const Lat& g, float bc,
-                                            int r, int ch, int s, const int (&cs)[4], int d, cx<float> (&phi)[12]) {
-  if (d == 0) {
-    in.load(g.V, r, ch, s, phi);
-    return;
-  }
+// site, link site and boundary factor of direction d at site s
+struct Nb {
+  int s, link;
+  float sg;
+};
+__device__ __forceinline__ Nb neighbour(const Lat& g, float bc, int s, const int (&cs)[4], int d) {
+  if (d == 0) return {s, s, 1.f};
   const int mu = (d - 1) >> 1;
   const bool fwd = ((d - 1) & 1) == 0;
-  const int nb = fwd ? nb_fwd(g, s, cs, mu) : nb_bwd(g, s, cs, mu);
-  const float sg = (mu == 0 && (fwd ? cs[0] == g.L[0] - 1 : cs[0] == 0)) ? bc : 1.f;
-  cx<float> p[12];
-  in.load(g.V, r, ch, nb, p);
+  const int cm = mu == 0 ? cs[0] : mu == 1 ? cs[1] : mu == 2 ? cs[2] : cs[3];
+  const int Lm = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+  const int sm = mu == 0 ? g.st[0] : mu == 1 ? g.st[1] : mu == 2 ? g.st[2] : g.st[3];
+  const bool edge = fwd ? cm + 1 == Lm : cm == 0;
+  const int nb = fwd ? (edge ? s - (Lm - 1) * sm : s + sm) : (edge ? s + (Lm - 1) * sm : s - sm);
+  return {nb, fwd ? s : nb, mu == 0 && edge ? bc : 1.f};
+}
+
+// phi = T_d p for the neighbour's spinor p
+__device__ __forceinline__ void transport(const float* __restrict__ gauge, const Lat& g, const Nb& n, int d,
+                                          const cx<float> (&p)[12], cx<float> (&phi)[12]) {
+  if (d == 0) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) phi[k] = p[k];
+    return;
+  }
   Link<float> U;
-  ld_link(gauge, g.V, mu, fwd ? s : nb, U);
+  ld_link(gauge, g.V, (d - 1) >> 1, n.link, U);
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp) {
-    cx<float> x[3] = {sg * p[3 * sp], sg * p[3 * sp + 1], sg * p[3 * sp + 2]}, y[3];
-    if (fwd)
-      su3_mul(U, x, y);
-    else
+    const cx<float> x[3] = {n.sg * p[3 * sp], n.sg * p[3 * sp + 1], n.sg * p[3 * sp + 2]};
+    cx<float> y[3];
+    if ((d - 1) & 1)
       su3_dag_mul(U, x, y);
+    else
+      su3_mul(U, x, y);
     phi[3 * sp] = y[0];
     phi[3 * sp + 1] = y[1];
     phi[3 * sp + 2] = y[2];
   }
 }
 
-// one layer: thread per (site, output channel); blockIdx.y = rhs
-template <class In, class Out, int CIN, int COUT>
-__global__ void __launch_bounds__(128) k_layer(In in, Out out, const float* __restrict__ gauge,
-                                               const float2* __restrict__ W, Lat g, float bc, int accumulate) {
-  __shared__ float2 Ws[COUT * CIN * kNdir * 16];
-  for (int e = threadIdx.x; e < COUT * CIN * kNdir * 16; e += blockDim.x) Ws[e] = W[e];
+// One channel to eight (L1, and the adjoint of L2 with its weights): thread =
+// (site, colour), the colour fixed per warp, all 32 output spinor components of
+// its colour in registers, two output channels as the lanes of packed FP32.  The
+// three warps of a site group read the same neighbours (L1).
+constexpr int kExpandSites = 64;
+template <typename Th>
+__global__ void __launch_bounds__(3 * kExpandSites, 2) k_expand(const float* __restrict__ in,
+                                                             typename Cx2<Th>::V* __restrict__ out,
+                                                             const float* __restrict__ gauge,
+                                                             const float2* __restrict__ W, Lat g, float bc) {
+  __shared__ float4 Ws[kC / 2 * kNdir * 16];  // [o / 2][d][s][t]: (re, re, im, im) of the two channels
+  for (int e = threadIdx.x; e < kC / 2 * kNdir * 16; e += blockDim.x) {
+    const int o = e / (kNdir * 16) * 2, k = e % (kNdir * 16);
+    const float2 a = W[o * kNdir * 16 + k], b = W[(o + 1) * kNdir * 16 + k];
+    Ws[e] = make_float4(a.x, b.x, a.y, b.y);
+  }
   __syncthreads();
-  const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long)g.V * COUT) return;
-  const int o = (int)(idx / g.V), s = (int)(idx % g.V), r = blockIdx.y;
+  const int warp = threadIdx.x >> 5, c = warp % 3, r = blockIdx.y;
+  const int s = blockIdx.x * kExpandSites + (warp / 3) * 32 + (threadIdx.x & 31);
+  if (s >= g.V) return;
+  const float* f = in + (long)r * NR_SPINOR * g.V;
+  int cs[4];
+  site_coords(g, s, cs);
+  cx<f2> acc[kC / 2 * 4];
+#pragma unroll
+  for (int k = 0; k < kC / 2 * 4; ++k) acc[k] = czero<f2>();
+#pragma unroll 1
+  for (int d = 0; d < kNdir; ++d) {
+    const Nb n = neighbour(g, bc, s, cs, d);
+    cx<float> p[12], phi[4];
+    ld_cx<float, 12>(f, g.V, n.s, p);
+    if (d == 0) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) phi[t] = c == 0 ? p[3 * t] : c == 1 ? p[3 * t + 1] : p[3 * t + 2];
+    } else {
+      // row c of U, or of U^dagger
+      Link<float> U;
+      ld_link(gauge, g.V, (d - 1) >> 1, n.link, U);
+      cx<float> u[3];
+      if ((d - 1) & 1) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u[k] = conj(c == 0 ? U.u[k][0] : c == 1 ? U.u[k][1] : U.u[k][2]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u[k] = c == 0 ? U.u[0][k] : c == 1 ? U.u[1][k] : U.u[2][k];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) u[k] = n.sg * u[k];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        phi[t] = u[0] * p[3 * t];
+        cfma(phi[t], u[1], p[3 * t + 1]);
+        cfma(phi[t], u[2], p[3 * t + 2]);
+      }
+    }
+    f2 pr[4], pi[4], pn[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      pr[t] = bcast<f2>(phi[t].r);
+      pi[t] = bcast<f2>(phi[t].i);
+      pn[t] = bcast<f2>(-phi[t].i);
+    }
+#pragma unroll
+    for (int o = 0; o < kC / 2; ++o)
+#pragma unroll
+      for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(Ws + ((o * kNdir + d) * 4 + sp) * 4 + t);
+          cx<f2>& y = acc[o * 4 + sp];
+          y.r = lfma(f2{w.x}, pr[t], y.r);
+          y.r = lfma(f2{w.y}, pn[t], y.r);
+          y.i = lfma(f2{w.x}, pi[t], y.i);
+          y.i = lfma(f2{w.y}, pr[t], y.i);
+        }
+  }
+  typename Cx2<Th>::V* q = out + (long)r * kC * 12 * g.V + s;
+#pragma unroll
+  for (int o = 0; o < kC / 2; ++o)
+#pragma unroll
+    for (int sp = 0; sp < 4; ++sp) {
+      const float2 re = f2_unpack(acc[o * 4 + sp].r), im = f2_unpack(acc[o * 4 + sp].i);
+      q[(long)(2 * o * 12 + 3 * sp + c) * g.V] = Cx2<Th>::put(cx<float>{re.x, im.x});
+      q[(long)((2 * o + 1) * 12 + 3 * sp + c) * g.V] = Cx2<Th>::put(cx<float>{re.y, im.y});
+    }
+}
+
+// Eight channels to one (L2): thread = site; per direction the channels are
+// summed over their weights at the neighbour, then transported once.
+template <typename Th>
+__global__ void __launch_bounds__(128, 4) k_reduce(const typename Cx2<Th>::V* __restrict__ in, float* __restrict__ out,
+                                                const float* __restrict__ gauge, const float2* __restrict__ W, Lat g,
+                                                float bc, int accumulate) {
+  __shared__ __align__(16) float2 Ws[kC * kNdir * 16];  // [i][d][s][t]
+  for (int e = threadIdx.x; e < kC * kNdir * 16; e += blockDim.x) Ws[e] = W[e];
+  __syncthreads();
+  const int s = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (s >= g.V) return;
+  const typename Cx2<Th>::V* f = in + (long)r * kC * 12 * g.V;
   int cs[4];
   site_coords(g, s, cs);
   cx<float> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = cx<float>{0.f, 0.f};
-  for (int d = 0; d < kNdir; ++d)
-    for (int i = 0; i < CIN; ++i) {
-      cx<float> phi[12];
-      transported(in, gauge, g, bc, r, i, s, cs, d, phi);
-      const float2* w = Ws + ((o * CIN + i) * kNdir + d) * 16;
+#pragma unroll 1
+  for (int d = 0; d < kNdir; ++d) {
+    const Nb n = neighbour(g, bc, s, cs, d);
+    cx<float> v[12], phi[12];
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
+    for (int k = 0; k < 12; ++k) v[k] = cx<float>{0.f, 0.f};
+#pragma unroll 2
+    for (int i = 0; i < kC; ++i) {
+      cx<float> h[12];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const cx<float> wst{w[sp * 4 + t].x, w[sp * 4 + t].y};
+      for (int k = 0; k < 12; ++k) h[k] = Cx2<Th>::get(f[(long)(i * 12 + k) * g.V + n.s]);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) cfma(acc[3 * sp + c], wst, phi[3 * t + c]);
+      for (int sp = 0; sp < 4; ++sp) {
+        const float4* w = reinterpret_cast<const float4*>(Ws + ((i * kNdir + d) * 4 + sp) * 4);
+        const float4 w0 = w[0], w1 = w[1];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          cfma(v[3 * sp + c], cx<float>{w0.x, w0.y}, h[c]);
+          cfma(v[3 * sp + c], cx<float>{w0.z, w0.w}, h[3 + c]);
+          cfma(v[3 * sp + c], cx<float>{w1.x, w1.y}, h[6 + c]);
+          cfma(v[3 * sp + c], cx<float>{w1.z, w1.w}, h[9 + c]);
         }
+      }
     }
-  out.store(g.V, r, o, s, acc, accumulate != 0);
-}
-
-template <class In, class Out, int CIN, int COUT>
-void run_layer(In in, Out out, const float* gauge, const float2* W, const Lat& g, double bc, int nrhs, bool acc,
-               cudaStream_t st) {
-  const long tot = (long)g.V * COUT;
-  dim3 grid((unsigned)((tot + 127) / 128), nrhs);
-  k_layer<In, Out, CIN, COUT><<<grid, 128, 0, st>>>(in, out, gauge, W, g, (float)bc, acc ? 1 : 0);
-}
-
-// weight gradient partials: CTA = 64 sites of one rhs; partial[cta][o][i][d][s][t] =
-// sum over its sites and colours of g_o(x)[s] conj(phi_{i,d}(x)[t])
-constexpr int kGradSites = 64;
-template <class In, class G, int CIN, int COUT>
-__global__ void __launch_bounds__(128) k_wgrad(In in, G gin, const float* __restrict__ gauge, Lat g, float bc,
-                                               float2* __restrict__ partial) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<float>* gs = reinterpret_cast<cx<float>*>(smem_raw);  // [COUT][64][12]
-  cx<float>* ph = gs + COUT * kGradSites * 12;              // [64][12]
-  cx<float>* red = ph + kGradSites * 12;                    // [128]
-  constexpr int E = COUT * 16;
-  constexpr int NG = 128 / E;
-  const int r = blockIdx.y;
-  const long s0 = (long)blockIdx.x * kGradSites;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < COUT * kGradSites; e += blockDim.x) {
-    const int o = e / kGradSites, k = e % kGradSites;
-    cx<float> p[12];
-    if (s0 + k < g.V) {
-      gin.load(g.V, r, o, s0 + k, p);
-    } else {
+    transport(gauge, g, n, d, v, phi);
 #pragma unroll
-      for (int q = 0; q < 12; ++q) p[q] = cx<float>{0.f, 0.f};
-    }
-#pragma unroll
-    for (int q = 0; q < 12; ++q) gs[(o * kGradSites + k) * 12 + q] = p[q];
+    for (int k = 0; k < 12; ++k) acc[k] = acc[k] + phi[k];
   }
-  const long cta = (long)blockIdx.y * gridDim.x + blockIdx.x;
-  const int grp = tid / E, ent = tid % E;
-  const int o = ent / 16, sp = (ent % 16) / 4, t = ent % 4;
-  for (int i = 0; i < CIN; ++i)
-    for (int d = 0; d < kNdir; ++d) {
-      __syncthreads();
-      if (tid < kGradSites) {
-        cx<float> phi[12];
-        const long s = s0 + tid;
-        if (s < g.V) {
-          int cs[4];
-          site_coords(g, (int)s, cs);
-          transported(in, gauge, g, bc, r, i, (int)s, cs, d, phi);
-        } else {
+  float* o = out + (long)r * NR_SPINOR * g.V;
+  if (accumulate) {
+    cx<float> q[12];
+    ld_cx<float, 12>(o, g.V, s, q);
 #pragma unroll
-          for (int q = 0; q < 12; ++q) phi[q] = cx<float>{0.f, 0.f};
+    for (int k = 0; k < 12; ++k) acc[k] = acc[k] + q[k];
+  }
+  st_cx<float, 12>(o, g.V, s, acc);
+}
+
+// Weight gradients, a contraction over sites and colours of the eight-channel
+// side h with the transported one-channel side A_d = T_d a:
+//   FIRST (W1):  G[o][d][s][t] = sum h_o[s] conj(A_d[t])              (h = g_h, a = r)
+//   else  (W2):  G[i][d][s][t] = sum A_opp(d)[s] conj(h_i[t])         (a = g_y; T_d^+ = T_opp(d))
+// Persistent CTAs stage tiles of 32 sites in shared memory (one transport per
+// thread: 9 directions x 32 sites) and keep the 32 x 36 complex sums in
+// registers: 2 groups of 144 threads, each 4 x 2 outputs and half of the sites.
+// Every 24 terms are added to a running FP32 pair, so the length of the plain
+// FP32 sums does not grow with the lattice.
+__device__ __forceinline__ void add_two_sum(float& h, float& l, float x) {
+  const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
+  h = s;
+}
+constexpr int kGTile = 32, kGThreads = 288, kGRows = 4 * kC, kGCols = 4 * kNdir;
+// site strides (complex numbers, 2 mod 16): staging stores of neighbouring sites fall on distinct banks
+constexpr int kGHs = 3 * kGRows + 2, kGAs = 3 * kGCols + 6;
+template <bool FIRST>
+__global__ void __launch_bounds__(kGThreads, 2) k_wgrad(const float2* __restrict__ hid, const float* __restrict__ one,
+                                                        const float* __restrict__ gauge, Lat g, float bc, int nrhs,
+                                                        double2* __restrict__ partial) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<float>* Hs = reinterpret_cast<cx<float>*>(smem_raw);  // [site 32][kGHs]: [colour 3][kGRows]
+  cx<float>* As = Hs + kGTile * kGHs;                       // [site 32][kGAs]: [colour 3][kGCols]
+  const int tid = threadIdx.x, grp = tid / 144, tg = tid % 144;
+  const int row0 = (tg / 18) * 4, col0 = (tg % 18) * 2;  // one channel's spins, two of a direction's
+  cx<float> hi[4][2], lo[4][2];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) hi[a][b] = lo[a][b] = cx<float>{0.f, 0.f};
+  const int tpr = (g.V + kGTile - 1) / kGTile;
+  const int dl = tid / 32, sl = tid & 31;  // this thread's direction and site when staging
+  for (long tile = blockIdx.x; tile < (long)tpr * nrhs; tile += gridDim.x) {
+    const int r = (int)(tile / tpr), s = (int)(tile % tpr) * kGTile + sl;
+    __syncthreads();
+    {
+      cx<float> phi[12];
+      if (s < g.V) {
+        int cs[4];
+        site_coords(g, s, cs);
+        const Nb n = neighbour(g, bc, s, cs, dl);
+        cx<float> p[12];
+        ld_cx<float, 12>(one + (long)r * NR_SPINOR * g.V, g.V, n.s, p);
+        transport(gauge, g, n, dl, p, phi);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) phi[k] = cx<float>{0.f, 0.f};
+      }
+#pragma unroll
+      for (int k = 0; k < 12; ++k) As[sl * kGAs + (k % 3) * kGCols + dl * 4 + k / 3] = phi[k];
+    }
+    if (dl < kC) {  // channel dl
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        const float2 v = s < g.V ? hid[((long)r * kC * 12 + dl * 12 + k) * g.V + s] : make_float2(0.f, 0.f);
+        Hs[sl * kGHs + (k % 3) * kGRows + dl * 4 + k / 3] = cx<float>{v.x, v.y};
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int s0 = grp * 16; s0 < grp * 16 + 16; s0 += 8) {
+      cx<float> acc[4][2];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) acc[a][b] = cx<float>{0.f, 0.f};
+#pragma unroll 6
+      for (int k = 0; k < 24; ++k) {
+        const int st = s0 + k / 3, c = k % 3;
+        const float4* hp = reinterpret_cast<const float4*>(Hs + st * kGHs + c * kGRows + row0);
+        const float4 a0 = *reinterpret_cast<const float4*>(As + st * kGAs + c * kGCols + col0);
+        const float4 h0 = hp[0], h1 = hp[1];
+        const cx<float> hv[4] = {{h0.x, h0.y}, {h0.z, h0.w}, {h1.x, h1.y}, {h1.z, h1.w}};
+        const cx<float> av[2] = {{a0.x, a0.y}, {a0.z, a0.w}};
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            if (FIRST)
+              cfmac(acc[a][b], av[b], hv[a]);
+            else
+              cfmac(acc[a][b], hv[a], av[b]);
+          }
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          add_two_sum(hi[a][b].r, lo[a][b].r, acc[a][b].r);
+          add_two_sum(hi[a][b].i, lo[a][b].i, acc[a][b].i);
         }
+    }
+  }
+  // the two groups' sums, then one partial per CTA
+  __syncthreads();
+  double2* red = reinterpret_cast<double2*>(smem_raw);  // [kGRows * kGCols]
+  if (grp == 1) {
 #pragma unroll
-        for (int q = 0; q < 12; ++q) ph[tid * 12 + q] = phi[q];
-      }
-      __syncthreads();
-      cx<float> sum{0.f, 0.f};
-      if (grp < NG)
-        for (int k = grp; k < kGradSites; k += NG)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) cfmac(sum, ph[k * 12 + 3 * t + c], gs[(o * kGradSites + k) * 12 + 3 * sp + c]);
-      red[tid] = sum;
-      __syncthreads();
-      if (tid < E) {
-        cx<float> tot = red[tid];
-        for (int q = 1; q < NG; ++q) tot = tot + red[q * E + tid];
-        const long nct = (long)gridDim.x * gridDim.y;
-        partial[(((long)o * CIN + i) * kNdir * 16 + d * 16 + sp * 4 + t) * nct + cta] = make_float2(tot.r, tot.i);
-      }
+      for (int b = 0; b < 2; ++b)
+        red[tg * 8 + a * 2 + b] = make_double2((double)hi[a][b].r + lo[a][b].r, (double)hi[a][b].i + lo[a][b].i);
+  }
+  __syncthreads();
+  if (grp == 1) return;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const double2 u = red[tg * 8 + a * 2 + b];
+      const double2 v = make_double2((double)hi[a][b].r + lo[a][b].r + u.x, (double)hi[a][b].i + lo[a][b].i + u.y);
+      const int ch = row0 / 4, dc = col0 / 4, t = (col0 & 3) + b;
+      const int d = FIRST || dc == 0 ? dc : (((dc - 1) & 1) ? dc - 1 : dc + 1);
+      const int e = (ch * kNdir + d) * 16 + (FIRST ? a * 4 + t : t * 4 + a);
+      partial[(long)e * gridDim.x + blockIdx.x] = v;
     }
 }
 
-// out[e] = sum_cta partial[cta][e] in FP64
-__global__ void k_wgrad_reduce(const float2* __restrict__ partial, long ncta, double2* __restrict__ out) {
+// out[e] = sum_cta partial[e][cta]
+__global__ void k_wgrad_reduce(const double2* __restrict__ partial, int ncta, double2* __restrict__ out) {
   __shared__ double red[2 * 128];
   const int e = blockIdx.x;
   double a = 0, b = 0;
-  for (long c = threadIdx.x; c < ncta; c += blockDim.x) {
-    const float2 v = partial[(long)e * ncta + c];
+  for (int c = threadIdx.x; c < ncta; c += blockDim.x) {
+    const double2 v = partial[(long)e * ncta + c];
     a += v.x;
     b += v.y;
   }
@@ -245,66 +373,74 @@ __global__ void k_wgrad_reduce(const float2* __restrict__ partial, long ncta, do
   if (threadIdx.x == 0) out[e] = make_double2(red[0], red[128]);
 }
 
-template <class In, class G, int CIN, int COUT>
-void run_wgrad(In in, G gin, const float* gauge, const Lat& g, double bc, int nrhs, float2* partial, double2* out,
-               cudaStream_t st) {
-  const int nx = (g.V + kGradSites - 1) / kGradSites;
-  const size_t smem = (size_t)(COUT * kGradSites * 12 + kGradSites * 12 + 128) * sizeof(cx<float>);
+constexpr int kGCtas = 2 * 152;
+
+template <bool FIRST>
+void run_wgrad(const float* hid, const float* one, const float* gauge, const Lat& g, double bc, int nrhs,
+               double2* partial, double2* out, cudaStream_t st) {
+  const size_t smem = (size_t)kGTile * (kGHs + kGAs) * sizeof(cx<float>);
+  static_assert(kGRows * kGCols * sizeof(double2) <= (size_t)kGTile * (kGHs + kGAs) * sizeof(cx<float>),
+                "the second group's sums reuse the tiles");
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_wgrad<In, G, CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    cudaFuncSetAttribute(k_wgrad<FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr = true;
   }
-  dim3 grid(nx, nrhs);
-  k_wgrad<In, G, CIN, COUT><<<grid, 128, smem, st>>>(in, gin, gauge, g, (float)bc, partial);
-  const int nent = COUT * CIN * kNdir * 16;
-  k_wgrad_reduce<<<nent, 128, 0, st>>>(partial, (long)nx * nrhs, out);
+  const long tiles = (long)((g.V + kGTile - 1) / kGTile) * nrhs;
+  const int ncta = (int)(tiles < kGCtas ? tiles : kGCtas);
+  k_wgrad<FIRST><<<ncta, kGThreads, smem, st>>>(reinterpret_cast<const float2*>(hid), one, gauge, g, (float)bc, nrhs,
+                                                partial);
+  k_wgrad_reduce<<<kC * kNdir * 16, 128, 0, st>>>(partial, ncta, out);
+}
+
+template <typename Th>
+void run_expand(const float* in, void* out, const float* gauge, const float2* W, const Lat& g, double bc, int nrhs,
+                cudaStream_t st) {
+  dim3 grid((unsigned)((g.V + kExpandSites - 1) / kExpandSites), nrhs);
+  k_expand<Th><<<grid, 3 * kExpandSites, 0, st>>>(in, static_cast<typename Cx2<Th>::V*>(out), gauge, W, g, (float)bc);
+}
+
+template <typename Th>
+void run_reduce(const void* in, float* out, const float* gauge, const float2* W, const Lat& g, double bc, int nrhs,
+                bool acc, cudaStream_t st) {
+  dim3 grid((unsigned)((g.V + 127) / 128), nrhs);
+  k_reduce<Th><<<grid, 128, 0, st>>>(static_cast<const typename Cx2<Th>::V*>(in), out, gauge, W, g, (float)bc,
+                                     acc ? 1 : 0);
 }
 
 }  // namespace
 
-long nn_wgrad_partial_floats2(const Lat& g, int nrhs) {
-  return (long)((g.V + kGradSites - 1) / kGradSites) * nrhs * kNnHidden * kNdir * 16;
-}
+long nn_wgrad_partial_doubles2() { return (long)kGCtas * kC * kNdir * 16; }
 
 void nn_layer1(const float* r, void* hid, bool half, const float* gauge, const float2* W1, const Lat& g, double bc,
                int nrhs, cudaStream_t st) {
   if (half)
-    run_layer<FineIn, HiddenOut<__half>, 1, kNnHidden>(FineIn{r, 1}, HiddenOut<__half>{static_cast<__half*>(hid),
-                                                                                         kNnHidden},
-                                                      gauge, W1, g, bc, nrhs, false, st);
+    run_expand<__half>(r, hid, gauge, W1, g, bc, nrhs, st);
   else
-    run_layer<FineIn, HiddenOut<float>, 1, kNnHidden>(FineIn{r, 1}, HiddenOut<float>{static_cast<float*>(hid),
-                                                                                       kNnHidden},
-                                                     gauge, W1, g, bc, nrhs, false, st);
+    run_expand<float>(r, hid, gauge, W1, g, bc, nrhs, st);
 }
 
 void nn_layer2(const void* hid, bool half, float* y, bool accumulate, const float* gauge, const float2* W2,
                const Lat& g, double bc, int nrhs, cudaStream_t st) {
   if (half)
-    run_layer<HiddenIn<__half>, FineOut, kNnHidden, 1>(HiddenIn<__half>{static_cast<const __half*>(hid), kNnHidden},
-                                                      FineOut{y, 1}, gauge, W2, g, bc, nrhs, accumulate, st);
+    run_reduce<__half>(hid, y, gauge, W2, g, bc, nrhs, accumulate, st);
   else
-    run_layer<HiddenIn<float>, FineOut, kNnHidden, 1>(HiddenIn<float>{static_cast<const float*>(hid), kNnHidden},
-                                                     FineOut{y, 1}, gauge, W2, g, bc, nrhs, accumulate, st);
+    run_reduce<float>(hid, y, gauge, W2, g, bc, nrhs, accumulate, st);
 }
 
 void nn_layer2_adjoint(const float* gy, float* gh, const float* gauge, const float2* W2adj, const Lat& g, double bc,
                        int nrhs, cudaStream_t st) {
-  run_layer<FineIn, HiddenOut<float>, 1, kNnHidden>(FineIn{gy, 1}, HiddenOut<float>{gh, kNnHidden}, gauge, W2adj, g,
-                                                   bc, nrhs, false, st);
+  run_expand<float>(gy, gh, gauge, W2adj, g, bc, nrhs, st);
 }
 
 void nn_grad_w2(const float* hid, const float* gy, const float* gauge, const Lat& g, double bc, int nrhs,
-                float2* partial, double2* out, cudaStream_t st) {
-  run_wgrad<HiddenIn<float>, FineIn, kNnHidden, 1>(HiddenIn<float>{hid, kNnHidden}, FineIn{gy, 1}, gauge, g, bc,
-                                                  nrhs, partial, out, st);
+                double2* partial, double2* out, cudaStream_t st) {
+  run_wgrad<false>(hid, gy, gauge, g, bc, nrhs, partial, out, st);
 }
 
 void nn_grad_w1(const float* r, const float* gh, const float* gauge, const Lat& g, double bc, int nrhs,
-                float2* partial, double2* out, cudaStream_t st) {
-  run_wgrad<FineIn, HiddenIn<float>, 1, kNnHidden>(FineIn{r, 1}, HiddenIn<float>{gh, kNnHidden}, gauge, g, bc, nrhs,
-                                                  partial, out, st);
+                double2* partial, double2* out, cudaStream_t st) {
+  run_wgrad<true>(gh, r, gauge, g, bc, nrhs, partial, out, st);
 }
 
 }  // namespace tmamg

@@ -1335,7 +1335,7 @@ double nn_grad_sum(tm_handle* h, const float* r, const float* e, int npairs, std
   float* hb = W<float>(h, "nn_hid", hid);
   float* gh = W<float>(h, "nn_gh", hid);
   float* y = W<float>(h, "nn_y", (size_t)fr * chunk);
-  float2* part = W<float2>(h, "nn_part", (size_t)nn_wgrad_partial_floats2(h->g, chunk));
+  double2* part = W<double2>(h, "nn_part", (size_t)nn_wgrad_partial_doubles2());
   G.assign(kNnWeights, std::complex<double>(0, 0));
   double loss = 0;
   esum = 0;

@@ -221,10 +221,10 @@ void launch_tc_schur(const TcGeom& tg, const OEGeom& oe, const float* ve, float*
 
 // ---- learned gauge-covariant layer (nn.cu) ------------------------------------
 // weights: complex float2 [Cout][Cin][9 directions][4][4]; hidden fields
-// [rhs][8][V][12 complex] in FP32 or FP16; fine fields in the chunked layout
+// [rhs][8][12 components][V] complex in FP32 or FP16; fine fields in the chunked layout
 constexpr int kNnHidden = 8;
 constexpr int kNnWeights = 2 * kNnHidden * 9 * 16;  // complex weights of both layers
-long nn_wgrad_partial_floats2(const Lat& g, int nrhs);
+long nn_wgrad_partial_doubles2();
 void nn_layer1(const float* r, void* hid, bool half, const float* gauge, const float2* W1, const Lat& g, double bc,
                int nrhs, cudaStream_t st);
 void nn_layer2(const void* hid, bool half, float* y, bool accumulate, const float* gauge, const float2* W2,
@@ -234,9 +234,9 @@ void nn_layer2_adjoint(const float* gy, float* gh, const float* gauge, const flo
                        int nrhs, cudaStream_t st);
 // summed over the nrhs samples: out[o][i][d][s][t] = sum_x g_o(x)[s] conj(T_d psi_i(x)[t]) (FP64)
 void nn_grad_w2(const float* hid, const float* gy, const float* gauge, const Lat& g, double bc, int nrhs,
-                float2* partial, double2* out, cudaStream_t st);
+                double2* partial, double2* out, cudaStream_t st);
 void nn_grad_w1(const float* r, const float* gh, const float* gauge, const Lat& g, double bc, int nrhs,
-                float2* partial, double2* out, cudaStream_t st);
+                double2* partial, double2* out, cudaStream_t st);
 
 // ---- level-1 vectors (blas.cu) ----------------------------------------------
 // all BLAS works on flat arrays of n complex numbers stored as (re, im) pairs
