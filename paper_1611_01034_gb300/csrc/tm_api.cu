@@ -767,6 +767,31 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
   const long ds = 4 * kMaxDots + 2;              // per-rhs small-result stride (doubles)
   const T* Dc = static_cast<const T*>(lv.Dc);
   const T* Di = static_cast<const T*>(lv.Dinv);
+  bool use_tc = false;
+  if constexpr (std::is_same<T, float>::value)
+    use_tc = lv.tc && nrhs >= 2 && tc_supported(lv.oe.nv, nrhs, h->p.coarse_mma);  // one rhs: CUDA cores
+  if (!use_tc && coarse_cluster_fits(lv.oe, m, nrhs, sizeof(T))) {
+    // a system small enough for one cluster per right-hand side: the whole solve in one launch
+    T* xe = W<T>(h, "cb_xe", cv * nrhs);
+    T* uo = W<T>(h, "cb_uo", cv * nrhs);
+    T* Vb = Wz<T>(h, "cb_V", vstr * nrhs);
+    int* out = W<int>(h, "cb_out", 2 * nrhs);
+    int* ho = reinterpret_cast<int*>(host_scratch(h, "cbc", nrhs));
+    {
+      Prof pf(h, PK_COARSE_OE, nrhs);
+      launch_coarse_gmres<T>(Dc, Di, b, x, Vb, uo, xe, out, lv.oe, lv.mu_c, tol, m, maxit, nrhs, h->st);
+      CKL();
+    }
+    CK(cudaMemcpyAsync(ho, out, (size_t)2 * nrhs * sizeof(int), cudaMemcpyDeviceToHost, h->st));
+    sync(h);
+    std::vector<int> steps(nrhs);
+    for (int r = 0; r < nrhs; ++r) {
+      if (ho[2 * r + 1]) raise(TM_ERR_NONFINITE, "non-finite coarse solve");
+      steps[r] = ho[2 * r];
+      h->coarse_iters += steps[r];
+    }
+    return steps;
+  }
   T* to = W<T>(h, "cb_to", cv * nrhs);
   T* bh = W<T>(h, "cb_bh", cv * nrhs);
   T* xe = W<T>(h, "cb_xe", cv * nrhs);
@@ -812,9 +837,6 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
     sync(h);
     slot = 0;
   };
-  bool use_tc = false;
-  if constexpr (std::is_same<T, float>::value)
-    use_tc = lv.tc && nrhs >= 2 && tc_supported(lv.oe.nv, nrhs, h->p.coarse_mma);  // one rhs: CUDA cores
   auto schur = [&](const T* v, long vs, int units) {
     Prof pf(h, PK_COARSE_OE, units, 2);
     if constexpr (std::is_same<T, float>::value) {

@@ -219,6 +219,16 @@ void launch_tc_schur(const TcGeom& tg, const OEGeom& oe, const float* ve, float*
                      int nrhs, long vstr, long ustr, long ystr, const int* active, int split, int* err,
                      cudaStream_t st, unsigned spin = 0);
 
+// ---- one-launch coarse solve (coarse_cluster.cu) --------------------------------
+// whether the odd-even system is small enough for a cluster per right-hand side
+bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes);
+// GMRES(restart) on the odd-even Schur complement, from zero, to tol or maxit steps, and x_o from
+// x_e.  b, x full vectors [rhs][Vc][n]; V [rhs][restart + 1][Vc/2][n], u, xe [rhs][Vc/2][n] work;
+// out [rhs][2] = steps, 1 if a norm was not finite.
+template <typename T>
+void launch_coarse_gmres(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* u, T* xe, int* out, const OEGeom& oe,
+                         double mu_c, double tol, int restart, int maxit, int nrhs, cudaStream_t st);
+
 // ---- learned gauge-covariant layer (nn.cu) ------------------------------------
 // weights: complex float2 [Cout][Cin][9 directions][4][4]; hidden fields
 // [rhs][8][12 components][V] complex in FP32 or FP16; fine fields in the chunked layout

@@ -1,0 +1,57 @@
+"""The coarse solve in one launch (small systems) against the step-by-step solve.
+
+The one-launch form takes restart lengths up to 48; 49 takes the other form, with the same steps until the
+first restart.  FP64 to 1e-9 (rounding of 24 Arnoldi steps of another summation order), FP32 to 1e-3; a zero
+right-hand side gives zero in no steps; a batch through the K-cycle gives every right-hand side what it gets
+alone (FP64).
+"""
+import numpy as np
+import pytest
+
+import inputs
+import paper_1611_01034_gb300 as tm
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from tests.gpu_helpers import GPU, rel  # noqa: E402
+
+
+def _gpu(L, agg, nv, prec, **kw):
+    g = GPU(inputs.gauge_field(L, 0.5, 5), m0=-0.4, c_sw=1.5, mu=0.005, delta=5.0, nv=nv, agg=agg, sap_block=(2, 2, 2, 2),
+            cycle_prec=prec, **kw)
+    tm.tm_setup_from_vectors(g.h, inputs.random_test_vectors(L, nv, 2005))
+    return g
+
+
+@pytest.mark.parametrize("L,agg,nv", [((4, 4, 4, 4), (2, 2, 2, 2), 3), ((8, 8, 8, 8), (4, 4, 4, 4), 9),
+                                      ((4, 4, 8, 12), (2, 2, 2, 2), 8), ((8, 8, 8, 16), (4, 4, 4, 4), 28)])
+@pytest.mark.parametrize("prec,tol", [(tm.TM_F64, 1e-9), (tm.TM_F32, 1e-3)])
+def test_one_launch_solve(L, agg, nv, prec, tol):
+    one, ref = _gpu(L, agg, nv, prec, coarse_restart=48), _gpu(L, agg, nv, prec, coarse_restart=49)
+    rng = np.random.default_rng(3)
+    b = rng.standard_normal(one.coarse_shape()) + 1j * rng.standard_normal(one.coarse_shape())
+    for target, maxit in ((0.0, 24), (1e-4, 200)):
+        xs, its = [], []
+        for g in (one, ref):
+            fx = g.field(1, prec)
+            its.append(tm.tm_coarse_solve(g.h, prec, g.pack(1, prec, b), fx, target, maxit))
+            xs.append(g.unpack(1, prec, fx, b.shape))
+        assert its[0] == its[1]
+        assert rel(xs[0], xs[1]) <= tol
+    fx = one.pack(1, prec, b)
+    assert tm.tm_coarse_solve(one.h, prec, one.pack(1, prec, 0 * b), fx, 0.0, 24) == 0
+    assert not one.unpack(1, prec, fx, b.shape).any()
+
+
+def test_one_launch_solve_of_a_batch():
+    L = (8, 8, 8, 8)
+    g = _gpu(L, (4, 4, 4, 4), 8, tm.TM_F64, max_rhs=3, coarse_tol=0.0, coarse_maxit=7, coarse_restart=3)
+    v = inputs.gaussian_spinor(L, 11, 3)
+    z = g.field(0, tm.TM_F64, 3)
+    tm.tm_kcycle(g.h, tm.TM_F64, g.pack(0, tm.TM_F64, v, 3), z, 3)
+    got = g.unpack(0, tm.TM_F64, z, v.shape, 3)
+    for r in range(3):
+        z1 = g.field(0, tm.TM_F64)
+        tm.tm_kcycle(g.h, tm.TM_F64, g.pack(0, tm.TM_F64, v[r]), z1, 1)
+        assert rel(got[r], g.unpack(0, tm.TM_F64, z1, v[r].shape)) <= 1e-12
