@@ -10,7 +10,10 @@
 // coarse operator: [site][9 blocks][col][row].
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "tm_kernels.h"
+#include "tm_lane.cuh"
 
 namespace tmamg {
 
@@ -130,22 +133,70 @@ __global__ void k_csap(const void* __restrict__ Dc, const T* __restrict__ b, T* 
   if (act) xx[(long)s * n + row] = xx[(long)s * n + row] + e;
 }
 
-// The same colour for up to RB right-hand sides per CTA: every block entry a
-// thread loads serves all of them (the separate-rhs form reads the block's
-// D_c1 entries once per right-hand side and MR step).  Each right-hand side
-// keeps its own residual, correction and MR coefficients.
-template <typename T, int H, int RB>
-__global__ void __launch_bounds__(768) k_csap_b(const void* __restrict__ Dc, const T* __restrict__ b, T* __restrict__ x, CSapGeom sg, T mu,
-                         int n_mr, int colour, int nrhs) {
+// The same colour in FP32 for PR pairs of right-hand sides per CTA, the pairs as
+// lanes of packed FP32.  A thread owns two consecutive rows of one site: one
+// vector load brings both entries of a column, and the PR shared-memory reads of
+// the column's vector serve both rows (one row per thread: 6 reads per 24
+// multiply-adds).  r and e live in shared memory, the residual's neighbours are
+// staged there one direction at a time.  Now bound by the latency of the block
+// loads (1.1 GB from DRAM per colour: the blocks in flight exceed L2) with 24
+// warps per SM: two sweeps of 6 right-hand sides at 16 x 8^3, FP16 blocks, N_v 24
+// 3.24 -> 2.01 ms, N_v 28 (8^4) 4.56 -> 1.66 ms, FP32 blocks 4.12 -> 2.18 ms.
+// Measured and left out: four rows per thread 2.71 ms (12 warps per SM; with the
+// blocks through a cp.async ring 2.59 ms), columns unrolled by four 2.28 ms.
+constexpr int kRows = 2;  // n is even
+// entries idx and idx + 1 (two rows of a column) of the blocks
+template <int S>
+__device__ __forceinline__ void ld_rows(const void* __restrict__ Dc, long idx, cx<float> (&m)[kRows]) {
+  if constexpr (S == ST_NATIVE) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(static_cast<const float2*>(Dc) + idx));
+    m[0] = cx<float>{v.x, v.y};
+    m[1] = cx<float>{v.z, v.w};
+  } else {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(static_cast<const unsigned*>(Dc) + idx));
+    const float2 f = unpack16x2<S>(v.x), h = unpack16x2<S>(v.y);
+    m[0] = cx<float>{f.x, f.y};
+    m[1] = cx<float>{h.x, h.y};
+  }
+}
+
+// acc[i][q] += sum_col B[row0 + i][col] v[col][q]
+template <int S, int PR>
+__device__ __forceinline__ void block_rows(const void* __restrict__ Dc, long idx, int n, const cx<f2>* v,
+                                           cx<f2> (&acc)[kRows][PR]) {
+#pragma unroll 8
+  for (int col = 0; col < n; ++col) {
+    cx<float> m[kRows];
+    ld_rows<S>(Dc, idx + (long)col * n, m);
+    cx<f2> x[PR];
+#pragma unroll
+    for (int q = 0; q < PR; ++q) x[q] = ld_shared(v + col * PR + q);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const f2 ur = bcast<f2>(m[i].r), ui = bcast<f2>(m[i].i), un = bcast<f2>(-m[i].i);
+#pragma unroll
+      for (int q = 0; q < PR; ++q) {
+        acc[i][q].r = lfma(ur, x[q].r, acc[i][q].r);
+        acc[i][q].r = lfma(un, x[q].i, acc[i][q].r);
+        acc[i][q].i = lfma(ur, x[q].i, acc[i][q].i);
+        acc[i][q].i = lfma(ui, x[q].r, acc[i][q].i);
+      }
+    }
+  }
+}
+
+template <int S, int PR, int MT>
+__global__ void __launch_bounds__(MT, MT == 384 ? 2 : 1) k_csap_l(const void* __restrict__ Dc, const float* __restrict__ b,
+                                                           float* __restrict__ x, CSapGeom sg, float mu, int n_mr,
+                                                           int colour, int nrhs, int ngrp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = sg.n, BS = sg.bsites;
-  cx<T>* rs = reinterpret_cast<cx<T>*>(smem_raw);  // [RB][BS][n]
-  T* red = reinterpret_cast<T*>(rs + (size_t)RB * BS * n);
+  cx<f2>* rs = reinterpret_cast<cx<f2>*>(smem_raw);  // [BS][n][PR]
+  cx<f2>* es = rs + (size_t)BS * n * PR;             // [BS][n][PR]; first the staged neighbours
+  f2* red = reinterpret_cast<f2*>(es + (size_t)BS * n * PR);
   const Lat& g = sg.g;
-  const int ngrp = (nrhs + RB - 1) / RB;
-  const int r0 = (blockIdx.x % ngrp) * RB;  // groups of right-hand sides fastest (block reuse in L2)
-  const int R = min(RB, nrhs - r0);
-  const long vs = (long)g.V * n;  // complex numbers per level-1 vector
+  const int r0 = (blockIdx.x % ngrp) * 2 * PR;  // groups of right-hand sides fastest (block reuse in L2)
+  const long vs = (long)g.V * n;                // complex numbers per level-1 vector
   int k = blockIdx.x / ngrp;
   const int nbxh = sg.nb[3] / 2;
   int bc4[4];
@@ -156,148 +207,215 @@ __global__ void __launch_bounds__(768) k_csap_b(const void* __restrict__ Dc, con
   bc4[1] = k % sg.nb[1];
   bc4[0] = k / sg.nb[1];
   bc4[3] = 2 * bxh + ((bc4[0] + bc4[1] + bc4[2] + colour) & 1);
-  const int l = threadIdx.x / n, row = threadIdx.x % n;
+  auto site = [&](int l, int (&lc)[4]) {
+    lc[3] = l % sg.blk[3];
+    l /= sg.blk[3];
+    lc[2] = l % sg.blk[2];
+    l /= sg.blk[2];
+    lc[1] = l % sg.blk[1];
+    lc[0] = l / sg.blk[1];
+    return (((bc4[0] * sg.blk[0] + lc[0]) * g.L[1] + bc4[1] * sg.blk[1] + lc[1]) * g.L[2] + bc4[2] * sg.blk[2] + lc[2]) *
+               g.L[3] +
+           bc4[3] * sg.blk[3] + lc[3];
+  };
+  const int rpt = n / kRows;  // threads per site
+  const int l = threadIdx.x / rpt, row0 = (threadIdx.x % rpt) * kRows;
   const bool act = l < BS;
-  int lc[4], c[4], lst[4];
-  lst[3] = 1;
-  lst[2] = sg.blk[3];
-  lst[1] = sg.blk[3] * sg.blk[2];
-  lst[0] = lst[1] * sg.blk[1];
-  {
-    int q = act ? l : 0;
-    lc[3] = q % sg.blk[3];
-    q /= sg.blk[3];
-    lc[2] = q % sg.blk[2];
-    q /= sg.blk[2];
-    lc[1] = q % sg.blk[1];
-    lc[0] = q / sg.blk[1];
-  }
-  for (int d = 0; d < 4; ++d) c[d] = bc4[d] * sg.blk[d] + lc[d];
-  const int s = ((c[0] * g.L[1] + c[1]) * g.L[2] + c[2]) * g.L[3] + c[3];
-  const long B = (long)s * 9 * n * n;
-  const T sg5 = row < n / 2 ? -mu : mu;
-  const cx<T>* xx = reinterpret_cast<const cx<T>*>(x) + r0 * vs;
-  const cx<T>* bb = b ? reinterpret_cast<const cx<T>*>(b) + r0 * vs : nullptr;
-  cx<T> r[RB], e[RB];
+  int lc[4];
+  const int s = site(act ? l : 0, lc);
+  const int lst[4] = {sg.blk[3] * sg.blk[2] * sg.blk[1], sg.blk[3] * sg.blk[2], sg.blk[3], 1};
+  const long B = (long)s * 9 * n * n + row0;
+  const float sg5 = row0 < n / 2 ? -mu : mu;  // i mu Gamma5_c (n / 2 is a multiple of kRows, or the rows split below)
+  const cx<float>* xx = reinterpret_cast<const cx<float>*>(x);
+  const cx<float>* bb = reinterpret_cast<const cx<float>*>(b);
+  // right-hand sides 2 q, 2 q + 1 of the group; a missing one repeats an existing one and is not stored
+  auto rhs0 = [&](int q) { return min(r0 + 2 * q, nrhs - 1); };
+  auto rhs1 = [&](int q) { return min(r0 + 2 * q + 1, nrhs - 1); };
+  auto pair_at = [&](const cx<float>* f, int q, long i) {
+    const cx<float> u = f[rhs0(q) * vs + i], v = f[rhs1(q) * vs + i];
+    return cx<f2>{f2_pack(u.r, v.r), f2_pack(u.i, v.i)};
+  };
+  auto gamma5 = [&](int i) { return n / 2 % kRows == 0 ? sg5 : (row0 + i < n / 2 ? -mu : mu); };
+  cx<f2> acc[kRows][PR];
 #pragma unroll
-  for (int j = 0; j < RB; ++j) r[j] = e[j] = cx<T>{0, 0};
+  for (int i = 0; i < kRows; ++i)
+#pragma unroll
+    for (int q = 0; q < PR; ++q) acc[i][q] = czero<f2>();
+  unsigned inside = 1;  // blocks of this site that stay inside
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    if (lc[d] < sg.blk[d] - 1) inside |= 2u << (2 * d);
+    if (lc[d] > 0) inside |= 4u << (2 * d);
+  }
+  // D x, the neighbours of direction t staged for all sites of the block
+#pragma unroll 1
+  for (int t = 0; t < 9; ++t) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < BS * n * PR; e += blockDim.x) {
+      const int q = e % PR, col = (e / PR) % n, ls = e / (PR * n);
+      int tmp[4];
+      st_shared(es + e, pair_at(xx, q, (long)c_nb(g, site(ls, tmp), t) * n + col));
+    }
+    __syncthreads();
+    if (act) block_rows<S, PR>(Dc, B + (long)t * n * n, n, es + (size_t)l * n * PR, acc);
+  }
+  __syncthreads();
+  cx<f2>* own_r = rs + ((size_t)l * n + row0) * PR;
+  cx<f2>* own_e = es + ((size_t)l * n + row0) * PR;
   if (act) {
-    cx<T> acc[RB];
 #pragma unroll
-    for (int j = 0; j < RB; ++j) acc[j] = cx<T>{0, 0};
-    for (int t = 0; t < 9; ++t) {
-      const long src = (long)c_nb(g, s, t) * n;
-      const long Bt = B + (long)t * n * n;
-#pragma unroll 4
-      for (int col = 0; col < n; ++col) {
-        const cx<T> m = ld_blk<T, H>(Dc, Bt + (long)col * n + row);
+    for (int i = 0; i < kRows; ++i)
 #pragma unroll
-        for (int j = 0; j < RB; ++j)
-          if (j < R) cfma(acc[j], m, xx[j * vs + src + col]);
+      for (int q = 0; q < PR; ++q) {
+        const long at = (long)s * n + row0 + i;
+        const cx<f2> xs = pair_at(xx, q, at);
+        const f2 gp = bcast<f2>(gamma5(i)), gn = bcast<f2>(-gamma5(i));
+        cx<f2> v = bb ? pair_at(bb, q, at) : czero<f2>();
+        v.r = v.r - lfma(gn, xs.i, acc[i][q].r);
+        v.i = v.i - lfma(gp, xs.r, acc[i][q].i);
+        st_shared(own_r + i * PR + q, v);
+        st_shared(own_e + i * PR + q, czero<f2>());
       }
-    }
-#pragma unroll
-    for (int j = 0; j < RB; ++j) {
-      if (j < R) {
-        const cx<T> xs = xx[j * vs + (long)s * n + row];
-        acc[j].r -= sg5 * xs.i;
-        acc[j].i += sg5 * xs.r;
-        r[j] = (bb ? bb[j * vs + (long)s * n + row] : cx<T>{0, 0}) - acc[j];
-        rs[((size_t)j * BS + l) * n + row] = r[j];
-      }
-    }
   }
+#pragma unroll 1
   for (int it = 0; it < n_mr; ++it) {
     __syncthreads();
-    cx<T> q[RB];
 #pragma unroll
-    for (int j = 0; j < RB; ++j) q[j] = cx<T>{0, 0};
-    T dots[3 * RB];
+    for (int i = 0; i < kRows; ++i)
 #pragma unroll
-    for (int j = 0; j < 3 * RB; ++j) dots[j] = 0;
+      for (int q = 0; q < PR; ++q) acc[i][q] = czero<f2>();
+    f2 dots[3 * PR];
+#pragma unroll
+    for (int j = 0; j < 3 * PR; ++j) dots[j] = bcast<f2>(0.f);
     if (act) {
+#pragma unroll 1
       for (int t = 0; t < 9; ++t) {
+        if (!(inside >> t & 1)) continue;  // leaves the block
         int ln = l;
         if (t > 0) {
           const int mu_d = (t - 1) >> 1;
-          const bool bwd = (t - 1) & 1;
-          if (bwd ? lc[mu_d] == 0 : lc[mu_d] == sg.blk[mu_d] - 1) continue;  // leaves the block
-          ln = bwd ? l - lst[mu_d] : l + lst[mu_d];
+          const int sm = mu_d == 0 ? lst[0] : mu_d == 1 ? lst[1] : mu_d == 2 ? lst[2] : lst[3];
+          ln = (t - 1) & 1 ? l - sm : l + sm;
         }
-        const long Bt = B + (long)t * n * n;
-#pragma unroll 4
-        for (int col = 0; col < n; ++col) {
-          const cx<T> m = ld_blk<T, H>(Dc, Bt + (long)col * n + row);
-#pragma unroll
-          for (int j = 0; j < RB; ++j)
-            if (j < R) cfma(q[j], m, rs[((size_t)j * BS + ln) * n + col]);
-        }
+        block_rows<S, PR>(Dc, B + (long)t * n * n, n, rs + (size_t)ln * n * PR, acc);
       }
 #pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        q[j].r -= sg5 * r[j].i;
-        q[j].i += sg5 * r[j].r;
-        dots[3 * j] = q[j].r * r[j].r + q[j].i * r[j].i;
-        dots[3 * j + 1] = q[j].r * r[j].i - q[j].i * r[j].r;
-        dots[3 * j + 2] = q[j].r * q[j].r + q[j].i * q[j].i;
-      }
+      for (int i = 0; i < kRows; ++i)
+#pragma unroll
+        for (int q = 0; q < PR; ++q) {
+          const cx<f2> r = ld_shared(own_r + i * PR + q);
+          cx<f2>& z = acc[i][q];
+          z.r = lfma(bcast<f2>(-gamma5(i)), r.i, z.r);
+          z.i = lfma(bcast<f2>(gamma5(i)), r.r, z.i);
+          dots[3 * q] = lfma(z.r, r.r, lfma(z.i, r.i, dots[3 * q]));
+          dots[3 * q + 1] = dots[3 * q + 1] + (z.r * r.i - z.i * r.r);
+          dots[3 * q + 2] = lfma(z.r, z.r, lfma(z.i, z.i, dots[3 * q + 2]));
+        }
     }
-    block_allreduce<T, 3 * RB>(dots, red);
-    if (act) {
 #pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        const cx<T> alpha = dots[3 * j + 2] > T(0) ? cx<T>{dots[3 * j] / dots[3 * j + 2], dots[3 * j + 1] / dots[3 * j + 2]}
-                                                   : cx<T>{0, 0};
-        cfma(e[j], alpha, r[j]);
-        cfma(r[j], -alpha, q[j]);
-      }
+    for (int j = 0; j < 3 * PR; ++j) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dots[j] = dots[j] + f2{__shfl_xor_sync(0xffffffffu, dots[j].v, o)};
+    }
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+      for (int j = 0; j < 3 * PR; ++j) red[(threadIdx.x >> 5) * 3 * PR + j] = dots[j];
     }
     __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 3 * PR; ++j) {
+      f2 sum = red[j];
+      for (int w = 1; w < (int)blockDim.x >> 5; ++w) sum = sum + red[w * 3 * PR + j];
+      dots[j] = sum;
+    }
     if (act) {
 #pragma unroll
-      for (int j = 0; j < RB; ++j)
-        if (j < R) rs[((size_t)j * BS + l) * n + row] = r[j];
+      for (int q = 0; q < PR; ++q) {
+        const float2 dr = f2_unpack(dots[3 * q]), di = f2_unpack(dots[3 * q + 1]), dq = f2_unpack(dots[3 * q + 2]);
+        const f2 ar = f2_pack(dq.x > 0.f ? dr.x / dq.x : 0.f, dq.y > 0.f ? dr.y / dq.y : 0.f);
+        const f2 ai = f2_pack(dq.x > 0.f ? di.x / dq.x : 0.f, dq.y > 0.f ? di.y / dq.y : 0.f);
+        const f2 nr = bcast<f2>(0.f) - ar, ni = bcast<f2>(0.f) - ai;
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          cx<f2> r = ld_shared(own_r + i * PR + q), e = ld_shared(own_e + i * PR + q);
+          e.r = lfma(ni, r.i, lfma(ar, r.r, e.r));
+          e.i = lfma(ai, r.r, lfma(ar, r.i, e.i));
+          st_shared(own_e + i * PR + q, e);
+          const cx<f2> z = acc[i][q];
+          r.r = lfma(ai, z.i, lfma(nr, z.r, r.r));
+          r.i = lfma(ni, z.r, lfma(nr, z.i, r.i));
+          st_shared(own_r + i * PR + q, r);
+        }
+      }
     }
   }
-  __syncthreads();
   if (act) {
-    cx<T>* xw = reinterpret_cast<cx<T>*>(x) + r0 * vs;
+    cx<float>* xw = reinterpret_cast<cx<float>*>(x);
 #pragma unroll
-    for (int j = 0; j < RB; ++j)
-      if (j < R) xw[j * vs + (long)s * n + row] = xw[j * vs + (long)s * n + row] + e[j];
+    for (int i = 0; i < kRows; ++i)
+#pragma unroll
+      for (int q = 0; q < PR; ++q) {
+        const cx<f2> e = ld_shared(own_e + i * PR + q);
+        const float2 er = f2_unpack(e.r), ei = f2_unpack(e.i);
+        const long at = (long)s * n + row0 + i;
+        if (r0 + 2 * q < nrhs) {
+          cx<float>* w = xw + (r0 + 2 * q) * vs + at;
+          *w = *w + cx<float>{er.x, ei.x};
+        }
+        if (r0 + 2 * q + 1 < nrhs) {
+          cx<float>* w = xw + (r0 + 2 * q + 1) * vs + at;
+          *w = *w + cx<float>{er.y, ei.y};
+        }
+      }
   }
 }
 
-constexpr int kCsapRhs = 6;  // right-hand sides per CTA of the batched level-1 SAP
-
-template <typename T, int H>
-void csap_b(const void* Dc, const T* b, T* x, const CSapGeom& sg, double mu, int n_mr, int colour, int nrhs,
-            cudaStream_t st) {
-  const int threads = (sg.bsites * sg.n + 31) / 32 * 32;
-  const size_t smem = (size_t)kCsapRhs * sg.bsites * sg.n * sizeof(cx<T>) + 32 * 3 * kCsapRhs * sizeof(T);
+template <int S, int PR, int MT>
+void csap_l(const void* Dc, const float* b, float* x, const CSapGeom& sg, double mu, int n_mr, int colour, int nrhs,
+            int ngrp, int threads, cudaStream_t st) {
+  const size_t smem = (size_t)2 * sg.bsites * sg.n * PR * sizeof(cx<f2>) + (size_t)threads / 32 * 3 * PR * sizeof(f2);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_csap_b<T, H, kCsapRhs>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_csap_l<S, PR, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
-  const int ngrp = (nrhs + kCsapRhs - 1) / kCsapRhs;
-  dim3 grid((unsigned)(sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2) * (unsigned)ngrp);
-  k_csap_b<T, H, kCsapRhs><<<grid, threads, smem, st>>>(Dc, b, x, sg, (T)mu, n_mr, colour, nrhs);
+  const unsigned grid = (unsigned)(sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2) * (unsigned)ngrp;
+  k_csap_l<S, PR, MT><<<grid, threads, smem, st>>>(Dc, b, x, sg, (float)mu, n_mr, colour, nrhs, ngrp);
+}
+template <int S, int MT>
+void csap_t(const void* Dc, const float* b, float* x, const CSapGeom& sg, double mu, int n_mr, int colour, int nrhs,
+            int threads, cudaStream_t st) {
+  const int pairs = (nrhs + 1) / 2, ngrp = (pairs + 2) / 3;  // up to 3 pairs per CTA, evenly filled
+  switch ((pairs + ngrp - 1) / ngrp) {
+    case 1: return csap_l<S, 1, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);
+    case 2: return csap_l<S, 2, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);
+    default: return csap_l<S, 3, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);
+  }
+}
+template <int S>
+void csap_s(const void* Dc, const float* b, float* x, const CSapGeom& sg, double mu, int n_mr, int colour, int nrhs,
+            cudaStream_t st) {
+  const int threads = (sg.bsites * sg.n / kRows + 31) / 32 * 32;
+  if (threads <= 384)  // 2^4 blocks up to N_v 24: two CTAs per SM
+    csap_t<S, 384>(Dc, b, x, sg, mu, n_mr, colour, nrhs, threads, st);
+  else
+    csap_t<S, 512>(Dc, b, x, sg, mu, n_mr, colour, nrhs, threads, st);
 }
 
 template <typename T>
 void launch_csap_colour(const T* Dc, const T* b, T* x, const CSapGeom& sg, double mu, int n_mr, int colour,
                         int nrhs, cudaStream_t st, const void* Dc_half, int half_kind) {
-  // several right-hand sides share every block-entry load (its 80 registers per
-  // thread allow up to 768 threads: 2^4 blocks of N_v1 <= 24)
-  if (nrhs > 1 && sizeof(T) == 4 && sg.bsites * sg.n <= 768) {
-    if (Dc_half && half_kind == ST_BF16)
-      csap_b<T, ST_BF16>(Dc_half, b, x, sg, mu, n_mr, colour, nrhs, st);
-    else if (Dc_half)
-      csap_b<T, ST_F16>(Dc_half, b, x, sg, mu, n_mr, colour, nrhs, st);
-    else
-      csap_b<T, ST_NATIVE>(Dc, b, x, sg, mu, n_mr, colour, nrhs, st);
-    return;
+  // several right-hand sides share every block-entry load
+  if constexpr (std::is_same<T, float>::value) {
+    if (nrhs > 1) {
+      if (Dc_half && half_kind == ST_BF16)
+        csap_s<ST_BF16>(Dc_half, b, x, sg, mu, n_mr, colour, nrhs, st);
+      else if (Dc_half)
+        csap_s<ST_F16>(Dc_half, b, x, sg, mu, n_mr, colour, nrhs, st);
+      else
+        csap_s<ST_NATIVE>(Dc, b, x, sg, mu, n_mr, colour, nrhs, st);
+      return;
+    }
   }
   const int threads = (sg.bsites * sg.n + 31) / 32 * 32;
   const size_t smem = (size_t)sg.bsites * sg.n * sizeof(cx<T>) + 32 * 3 * sizeof(T);
