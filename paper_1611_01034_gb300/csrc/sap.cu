@@ -174,6 +174,312 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_sap(SapArgs<T> 
   }
 }
 
+namespace {
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) {
+  return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// sums of 3 values over the CTA; red holds 3 values per warp, read by the next call only after a barrier
+template <class R>
+__device__ __forceinline__ void lanes_allreduce3(R (&v)[3], R* red) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if constexpr (LaneOf<R>::n == 2)
+        v[k] = v[k] + f2{__shfl_xor_sync(0xffffffffu, v[k].v, o)};
+      else
+        v[k] = v[k] + __shfl_xor_sync(0xffffffffu, v[k], o);
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) red[(threadIdx.x >> 5) * 3 + k] = v[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    R s = red[k];
+    for (int w = 1; w < (int)blockDim.x >> 5; ++w) s = s + red[w * 3 + k];
+    v[k] = s;
+  }
+}
+
+// <q, r> / <q, q> from the three sums, 0 where <q, q> is not positive
+__device__ __forceinline__ float mr_ratio(float n, float d) { return d > 0.f ? n / d : 0.f; }
+__device__ __forceinline__ double mr_ratio(double n, double d) { return d > 0.0 ? n / d : 0.0; }
+__device__ __forceinline__ f2 mr_ratio(f2 n, f2 d) {
+  const float2 a = f2_unpack(n), b = f2_unpack(d);
+  return f2_pack(mr_ratio(a.x, b.x), mr_ratio(a.y, b.y));
+}
+
+}  // namespace
+
+// The same for 4^4 blocks in FP32, with everything that the MR steps read on the
+// chip: the block's links in shared memory (48 KB), the site's clover blocks and e,
+// which only their own thread reads, in tensor memory (96 columns per warp), r in
+// shared memory.  The general kernel reads links and clover from L1 and L2 in every
+// step and waits for them: four sweeps, one right-hand side, 32 x 16^3, 335 -> 285
+// us; 8^4 218 -> 169 us; three sweeps of 7 at 24^2 x 16^2 1.63 -> 1.37 ms.  Measured
+// and left out: two right-hand sides per thread as packed lanes, as in the odd-even
+// form (4 right-hand sides 878 -> 900 us: eight warps per SM wait longer); e alone
+// moved to shared memory (320 us).
+namespace {
+
+// N words per thread to and from tensor memory (the loads wait; tmem_wait_st for the stores)
+__device__ __forceinline__ void tmem_st8(unsigned ta, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(ta), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st4w(unsigned ta, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ta), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(unsigned ta, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "r"(ta)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld4w(unsigned ta, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+               : "r"(ta)
+               : "memory");
+}
+// after this the loaded registers may be read: they pass through it
+template <int N>
+__device__ __forceinline__ void tmem_loaded(float (&v)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < N; ++k) asm volatile("" : "+f"(v[k])::"memory");
+}
+
+constexpr int kS4 = 256;                 // sites of a block
+constexpr unsigned kS4Cols = 256;        // tensor memory columns: (72 clover + 24 e) for two warps per quarter
+constexpr size_t kS4Smem = 12 * kS4 * sizeof(float4) + 12 * kS4 * sizeof(cx<float>);
+
+__global__ void __launch_bounds__(kS4, 2) k_sap4(SapArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned tmem_base;
+  __shared__ float red[8 * 3];
+  float4* lk = reinterpret_cast<float4*>(smem_raw);                       // [mu][chunk][site]
+  cx<float>* rs = reinterpret_cast<cx<float>*>(lk + 12 * kS4);            // [12][site]
+  const SapGeom& sg = a.sg;
+  const Lat& g = sg.g;
+  const long V = g.V;
+  const int l = threadIdx.x, warp = l >> 5;
+  const long off = (long)(blockIdx.x % a.nrhs) * NR_SPINOR * V;  // right-hand sides fastest (operator reuse in L2)
+  float* x = a.x + off;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(kS4Cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  int k = blockIdx.x / a.nrhs;
+  const int nbxh = sg.nb[3] / 2;
+  int bc4[4];
+  const int bxh = k % nbxh;
+  k /= nbxh;
+  bc4[2] = k % sg.nb[2];
+  k /= sg.nb[2];
+  bc4[1] = k % sg.nb[1];
+  bc4[0] = k / sg.nb[1];
+  bc4[3] = 2 * bxh + ((bc4[0] + bc4[1] + bc4[2] + a.colour) & 1);
+  const int lc[4] = {l >> 6, (l >> 4) & 3, (l >> 2) & 3, l & 3};
+  constexpr int lst[4] = {64, 16, 4, 1};
+  int c[4];
+#pragma unroll
+  for (int d = 0; d < 4; ++d) c[d] = 4 * bc4[d] + lc[d];
+  const int s = ((c[0] * g.L[1] + c[1]) * g.L[2] + c[2]) * g.L[3] + c[3];
+  const float mus = ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu + a.rho : a.mu;
+  auto rows = [&](const float4 (&v)[3], Link<float>& U) {
+    const cx<float> z[6] = {{v[0].x, v[0].y}, {v[0].z, v[0].w}, {v[1].x, v[1].y},
+                            {v[1].z, v[1].w}, {v[2].x, v[2].y}, {v[2].z, v[2].w}};
+    link_from_rows(z, U);
+  };
+  auto scale = [&](Link<float>& U) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) U.u[i][j] = a.bc * U.u[i][j];
+  };
+  const float4* gl = reinterpret_cast<const float4*>(a.gauge);
+
+  // r = b - D x: forward hops with the site's own links, which go to shared memory
+  cx<float> acc[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) acc[i] = cx<float>{0.f, 0.f};
+  auto fwd = [&](auto MUC) {
+    constexpr int MU = decltype(MUC)::value;
+    cx<float> p[12];
+    ld_cx<float, 12>(x, V, nb_fwd(g, s, c, MU), p);
+    float4 v[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      v[q] = __ldg(gl + (MU * 3 + q) * V + s);
+      lk[(MU * 3 + q) * kS4 + l] = v[q];
+    }
+    Link<float> U;
+    rows(v, U);
+    if (MU == 0 && c[0] == g.L[0] - 1) scale(U);
+    hop_lanes<float, float, MU, true>([&](int i) { return p[i]; }, U, acc);
+  };
+  fwd(std::integral_constant<int, 0>{});
+  fwd(std::integral_constant<int, 1>{});
+  fwd(std::integral_constant<int, 2>{});
+  fwd(std::integral_constant<int, 3>{});
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned ta = tmem_base + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * 96;  // clover, e at + 72
+  auto bwd = [&](auto MUC) {
+    constexpr int MU = decltype(MUC)::value;
+    const int sb = nb_bwd(g, s, c, MU);
+    cx<float> p[12];
+    ld_cx<float, 12>(x, V, sb, p);
+    float4 v[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      v[q] = lc[MU] > 0 ? lk[(MU * 3 + q) * kS4 + l - lst[MU]] : __ldg(gl + (MU * 3 + q) * V + sb);
+    Link<float> U;
+    rows(v, U);
+    if (MU == 0 && c[0] == 0) scale(U);
+    hop_lanes<float, float, MU, false>([&](int i) { return p[i]; }, U, acc);
+  };
+  bwd(std::integral_constant<int, 0>{});
+  bwd(std::integral_constant<int, 1>{});
+  bwd(std::integral_constant<int, 2>{});
+  bwd(std::integral_constant<int, 3>{});
+  __syncwarp();  // the tensor-memory accesses are warp-wide
+  {
+    cx<float> p[12];
+    ld_cx<float, 12>(x, V, s, p);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) acc[i] = -0.5f * acc[i];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float m[36];
+      ld_re<float, 36>(a.clover + (long)h * 36 * V, V, s, m);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) tmem_st8(ta + 36 * h + 8 * q, m + 8 * q);
+      tmem_st4w(ta + 36 * h + 32, m + 32);
+      herm6_lanes<float, float>(m, h == 0 ? -mus : mus, p + 6 * h, acc + 6 * h);
+    }
+    const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) tmem_st8(ta + 72 + 8 * q, z);
+    if (a.b) {
+      ld_cx<float, 12>(a.b + off, V, s, p);
+#pragma unroll
+      for (int i = 0; i < 12; ++i) acc[i] = p[i] - acc[i];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) acc[i] = -acc[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 12; ++i) rs[i * kS4 + l] = acc[i];
+    tmem_wait_st();
+  }
+#pragma unroll 1
+  for (int it = 0; it < a.n_mr; ++it) {
+    __syncthreads();
+    cx<float> q[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) q[i] = cx<float>{0.f, 0.f};
+    auto hop = [&](auto MUC) {
+      constexpr int MU = decltype(MUC)::value;
+      if (lc[MU] < 3) {
+        const cx<float>* sp = rs + l + lst[MU];
+        const float4 v[3] = {lk[(MU * 3) * kS4 + l], lk[(MU * 3 + 1) * kS4 + l], lk[(MU * 3 + 2) * kS4 + l]};
+        Link<float> U;
+        rows(v, U);
+        hop_lanes<float, float, MU, true>([&](int i) { return sp[i * kS4]; }, U, q);
+      }
+      if (lc[MU] > 0) {
+        const int ln = l - lst[MU];
+        const cx<float>* sp = rs + ln;
+        const float4 v[3] = {lk[(MU * 3) * kS4 + ln], lk[(MU * 3 + 1) * kS4 + ln], lk[(MU * 3 + 2) * kS4 + ln]};
+        Link<float> U;
+        rows(v, U);
+        hop_lanes<float, float, MU, false>([&](int i) { return sp[i * kS4]; }, U, q);
+      }
+    };
+    hop(std::integral_constant<int, 0>{});
+    hop(std::integral_constant<int, 1>{});
+    hop(std::integral_constant<int, 2>{});
+    hop(std::integral_constant<int, 3>{});
+    __syncwarp();
+    cx<float> r[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      r[i] = rs[i * kS4 + l];
+      q[i] = -0.5f * q[i];
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float m[36];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) tmem_ld8(ta + 36 * h + 8 * w, m + 8 * w);
+      tmem_ld4w(ta + 36 * h + 32, m + 32);
+      tmem_loaded(m);
+      herm6_lanes<float, float>(m, h == 0 ? -mus : mus, r + 6 * h, q + 6 * h);
+    }
+    float dots[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      dots[0] = fmaf(q[i].r, r[i].r, fmaf(q[i].i, r[i].i, dots[0]));   // Re <q, r>
+      dots[1] = fmaf(q[i].r, r[i].i, fmaf(-q[i].i, r[i].r, dots[1]));  // Im <q, r>
+      dots[2] = fmaf(q[i].r, q[i].r, fmaf(q[i].i, q[i].i, dots[2]));   // <q, q>
+    }
+    lanes_allreduce3<float>(dots, red);  // its barrier: every neighbour's r has been read
+    const cx<float> al{mr_ratio(dots[0], dots[2]), mr_ratio(dots[1], dots[2])};
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      float e[8];
+      tmem_ld8(ta + 72 + 8 * w, e);
+      tmem_loaded(e);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        cx<float> z{e[2 * i], e[2 * i + 1]};
+        cfma(z, al, r[4 * w + i]);
+        e[2 * i] = z.r;
+        e[2 * i + 1] = z.i;
+      }
+      tmem_st8(ta + 72 + 8 * w, e);
+    }
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      cfma(r[i], -al, q[i]);
+      rs[i * kS4 + l] = r[i];
+    }
+    tmem_wait_st();
+  }
+  {
+    cx<float> p[12];
+    ld_cx<float, 12>(x, V, s, p);
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      float e[8];
+      tmem_ld8(ta + 72 + 8 * w, e);
+      tmem_loaded(e);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p[4 * w + i] = p[4 * w + i] + cx<float>{e[2 * i], e[2 * i + 1]};
+    }
+    st_cx<float, 12>(x, V, s, p);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kS4Cols) : "memory");
+}
+
+}  // namespace
+
 template <typename T>
 void launch_sap_colour(const T* gauge, const T* clover, const T* b, T* x, const SapGeom& sg, double mu,
                        double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st, double rho) {
@@ -186,6 +492,19 @@ void launch_sap_colour(const T* gauge, const T* clover, const T* b, T* x, const 
   }
   const int nblk_colour = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2;
   SapArgs<T> a{gauge, clover, b, x, sg, (T)mu, (T)bc_t, n_mr, colour, nrhs, (T)rho};
+  if constexpr (std::is_same<T, float>::value) {
+    bool b4 = true;
+    for (int d = 0; d < 4; ++d) b4 = b4 && sg.blk[d] == 4;
+    if (b4) {
+      static bool attr4 = false;
+      if (!attr4) {
+        cudaFuncSetAttribute(k_sap4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kS4Smem);
+        attr4 = true;
+      }
+      k_sap4<<<nblk_colour * nrhs, kS4, kS4Smem, st>>>(a);
+      return;
+    }
+  }
   dim3 grid(nblk_colour * nrhs);
   k_sap<T><<<grid, threads, smem, st>>>(a);
 }
@@ -245,40 +564,6 @@ __device__ __forceinline__ void ld_op(const void* __restrict__ base, long off, l
     ld_cx<T, NC>(static_cast<const T*>(base) + off, V, s, z);
   else
     ld_cx16<T, S, NC>(static_cast<const unsigned short*>(base) + off, V, s, z);
-}
-
-// sums of 3 values over the CTA; red holds 3 values per warp, read by the next call only after a barrier
-template <class R>
-__device__ __forceinline__ void lanes_allreduce3(R (&v)[3], R* red) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      if constexpr (LaneOf<R>::n == 2)
-        v[k] = v[k] + f2{__shfl_xor_sync(0xffffffffu, v[k].v, o)};
-      else
-        v[k] = v[k] + __shfl_xor_sync(0xffffffffu, v[k], o);
-    }
-  }
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) red[(threadIdx.x >> 5) * 3 + k] = v[k];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    R s = red[k];
-    for (int w = 1; w < (int)blockDim.x >> 5; ++w) s = s + red[w * 3 + k];
-    v[k] = s;
-  }
-}
-
-// <q, r> / <q, q> from the three sums, 0 where <q, q> is not positive
-__device__ __forceinline__ float mr_ratio(float n, float d) { return d > 0.f ? n / d : 0.f; }
-__device__ __forceinline__ double mr_ratio(double n, double d) { return d > 0.0 ? n / d : 0.0; }
-__device__ __forceinline__ f2 mr_ratio(f2 n, f2 d) {
-  const float2 a = f2_unpack(n), b = f2_unpack(d);
-  return f2_pack(mr_ratio(a.x, b.x), mr_ratio(a.y, b.y));
 }
 
 }  // namespace
@@ -628,9 +913,6 @@ namespace {
 constexpr int kB4 = 256, kH4 = 128;           // sites of a 4^4 block, of one parity
 constexpr unsigned kTmemCols = 128;  // e_e at column 0, e_o at 48
 
-__device__ __forceinline__ unsigned smem_u32(const void* p) {
-  return static_cast<unsigned>(__cvta_generic_to_shared(p));
-}
 // four complex pairs (16 words per thread) to and from tensor memory; the caller waits
 __device__ __forceinline__ void tmem_st4(unsigned ta, const cx<f2>* z) {
   float2 v[8];
@@ -657,7 +939,6 @@ __device__ __forceinline__ void tmem_ld4(unsigned ta, cx<f2>* z) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) z[k] = cx<f2>{f2_pack(v[4 * k], v[4 * k + 1]), f2_pack(v[4 * k + 2], v[4 * k + 3])};
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // two complex numbers of a 16-bit chunk
 template <int S>
@@ -857,6 +1138,7 @@ __global__ void __launch_bounds__(kH4, 3) k_sap_oe4(SapOeArgs<float> a) {
         hops(std::integral_constant<int, 2>{});
         hops(std::integral_constant<int, 3>{});
       }
+      __syncwarp();  // the tensor-memory accesses below are warp-wide
       if (parity) {
         if (st == 0) {
 #pragma unroll

@@ -290,18 +290,6 @@ __device__ __forceinline__ void ld_link(const T* __restrict__ gauge, long V, int
   link_from_rows(z, U);
 }
 
-// the link from links stored as T (S = ST_NATIVE) or in 16 bits (ST_F16, ST_BF16)
-template <typename T, int S>
-__device__ __forceinline__ void ld_link_s(const void* __restrict__ gauge, long V, int mu, long s, Link<T>& U) {
-  if constexpr (S == ST_NATIVE) {
-    ld_link(static_cast<const T*>(gauge), V, mu, s, U);
-  } else {
-    cx<T> z[6];
-    ld_cx16<T, S, 6>(static_cast<const unsigned short*>(gauge) + (long)mu * NR_LINK * V, V, s, z);
-    link_from_rows(z, U);
-  }
-}
-
 // NR reals of site s, stored as T or in 16 bits (chunks of 4 reals)
 template <typename T, int S, int NR>
 __device__ __forceinline__ void ld_re_s(const void* __restrict__ base, long V, long s, T (&r)[NR]) {
@@ -319,15 +307,6 @@ __device__ __forceinline__ void ld_re_s(const void* __restrict__ base, long V, l
       r[4 * k + 3] = (T)b.y;
     }
   }
-}
-
-// NC complex numbers of site s, stored as T or in 16 bits
-template <typename T, int S, int NC>
-__device__ __forceinline__ void ld_cx_s(const void* __restrict__ base, long V, long s, cx<T> (&z)[NC]) {
-  if constexpr (S == ST_NATIVE)
-    ld_cx<T, NC>(static_cast<const T*>(base), V, s, z);
-  else
-    ld_cx16<T, S, NC>(base, V, s, z);
 }
 
 // y = U x (colour)

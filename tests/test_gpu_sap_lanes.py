@@ -46,3 +46,19 @@ def test_odd_even_sap_batches(L, blk, nrhs, prec, tol):
         sap = SAP(Operator(U, -0.3, 1.3, 0.05), blk, n_mr=4, block_oe=True)
         assert rel(got[-1], sap.smooth(b[-1], x0[-1], 2)) <= tol
         assert rel(got0[0], sap.smooth(np.zeros_like(b[0]), x0[0], 1)) <= tol
+
+
+@pytest.mark.parametrize("prec,tol", [(tm.TM_F32, 1e-4), (tm.TM_F64, 1e-10)])
+def test_full_block_sap_batch(prec, tol):
+    # 4^4 blocks: FP32 keeps the block's operator on the chip, with and without b, across the T boundary
+    L, blk, nrhs = (8, 16, 8, 8), (4, 4, 4, 4), 3
+    U = inputs.gauge_field(L, 0.5, 19)
+    g = GPU(U, m0=-0.3, c_sw=1.3, mu=0.05, nv=2, agg=blk, sap_block=blk, cycle_prec=prec, max_rhs=nrhs)
+    sap = SAP(Operator(U, -0.3, 1.3, 0.05), blk, n_mr=4)
+    b, x0 = inputs.gaussian_spinor(L, 1, nrhs), inputs.gaussian_spinor(L, 2, nrhs)
+    for bb in (b, None):
+        fx = g.pack(0, prec, x0, nrhs)
+        tm.tm_sap(g.h, prec, None if bb is None else g.pack(0, prec, bb, nrhs), fx, 2, nrhs)
+        got = g.unpack(0, prec, fx, x0.shape, nrhs)
+        for r in range(nrhs):
+            assert rel(got[r], sap.smooth(np.zeros_like(b[r]) if bb is None else b[r], x0[r], 2)) <= tol
