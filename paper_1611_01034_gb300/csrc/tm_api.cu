@@ -643,6 +643,23 @@ std::vector<int> coarse_solve_graph(tm_handle* h, const OELevel& lv, const T* b,
   const long ds = 4 * kMaxDots + 2;
   const T* Dc = static_cast<const T*>(lv.Dc);
   const T* Di = static_cast<const T*>(lv.Dinv);
+  if (nrhs == 1 && coarse_grid_fits(lv.oe, K, sizeof(T))) {
+    // one right-hand side: the K steps in one cooperative launch
+    T* xe = W<T>(h, "gq_xe", cv);
+    T* uo = W<T>(h, "gq_uo", cv);
+    T* Vb = W<T>(h, "gq_V", vstr);
+    int* out = W<int>(h, "gq_out", 2);
+    double* scratch = W<double>(h, "gq_grid", coarse_grid_scratch_doubles(K));
+    {
+      Prof pf(h, PK_COARSE_OE, K);
+      launch_coarse_gmres_grid<T>(Dc, Di, b, x, Vb, uo, xe, out, scratch, h->d_err, lv.oe, lv.mu_c, tol, K, K, true,
+                                  h->st);
+      CKL();
+    }
+    h->coarse_iters += K;
+    check_flags(h);  // bounded waits
+    return std::vector<int>(1, K);
+  }
   T* to = W<T>(h, "gq_to", cv * nrhs);
   T* bh = W<T>(h, "gq_bh", cv * nrhs);
   T* xe = W<T>(h, "gq_xe", cv * nrhs);
@@ -770,20 +787,28 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
   bool use_tc = false;
   if constexpr (std::is_same<T, float>::value)
     use_tc = lv.tc && nrhs >= 2 && tc_supported(lv.oe.nv, nrhs, h->p.coarse_mma);  // one rhs: CUDA cores
-  if (!use_tc && coarse_cluster_fits(lv.oe, m, nrhs, sizeof(T))) {
-    // a system small enough for one cluster per right-hand side: the whole solve in one launch
+  const bool cluster = !use_tc && coarse_cluster_fits(lv.oe, m, nrhs, sizeof(T));
+  if (cluster || (nrhs == 1 && coarse_grid_fits(lv.oe, m, sizeof(T)))) {
+    // a system small enough for one cluster per right-hand side, or one right-hand side on the
+    // whole chip: the whole solve in one launch
     T* xe = W<T>(h, "cb_xe", cv * nrhs);
     T* uo = W<T>(h, "cb_uo", cv * nrhs);
     T* Vb = Wz<T>(h, "cb_V", vstr * nrhs);
     int* out = W<int>(h, "cb_out", 2 * nrhs);
     int* ho = reinterpret_cast<int*>(host_scratch(h, "cbc", nrhs));
     {
+      double* scratch = cluster ? nullptr : W<double>(h, "cb_grid", coarse_grid_scratch_doubles(m));
       Prof pf(h, PK_COARSE_OE, nrhs);
-      launch_coarse_gmres<T>(Dc, Di, b, x, Vb, uo, xe, out, lv.oe, lv.mu_c, tol, m, maxit, nrhs, h->st);
+      if (cluster)
+        launch_coarse_gmres<T>(Dc, Di, b, x, Vb, uo, xe, out, lv.oe, lv.mu_c, tol, m, maxit, nrhs, h->st);
+      else
+        launch_coarse_gmres_grid<T>(Dc, Di, b, x, Vb, uo, xe, out, scratch, h->d_err, lv.oe, lv.mu_c, tol, m, maxit,
+                                    false, h->st);
       CKL();
     }
     CK(cudaMemcpyAsync(ho, out, (size_t)2 * nrhs * sizeof(int), cudaMemcpyDeviceToHost, h->st));
     sync(h);
+    if (!cluster) check_flags(h);  // bounded waits
     std::vector<int> steps(nrhs);
     for (int r = 0; r < nrhs; ++r) {
       if (ho[2 * r + 1]) raise(TM_ERR_NONFINITE, "non-finite coarse solve");

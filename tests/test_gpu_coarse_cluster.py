@@ -1,6 +1,6 @@
 """The coarse solve in one launch (small systems) against the step-by-step solve.
 
-The one-launch form takes restart lengths up to 48; 49 takes the other form, with the same steps until the
+The one-launch forms (a cluster per right-hand side, the whole chip) take restart lengths up to 48; 49 takes the other form, with the same steps until the
 first restart.  FP64 to 1e-9 (rounding of 24 Arnoldi steps of another summation order), FP32 to 1e-3; a zero
 right-hand side gives zero in no steps; a batch through the K-cycle gives every right-hand side what it gets
 alone (FP64).
@@ -25,7 +25,8 @@ def _gpu(L, agg, nv, prec, **kw):
 
 
 @pytest.mark.parametrize("L,agg,nv", [((4, 4, 4, 4), (2, 2, 2, 2), 3), ((8, 8, 8, 8), (4, 4, 4, 4), 9),
-                                      ((4, 4, 8, 12), (2, 2, 2, 2), 8), ((8, 8, 8, 16), (4, 4, 4, 4), 28)])
+                                      ((4, 4, 8, 12), (2, 2, 2, 2), 8), ((8, 8, 8, 16), (4, 4, 4, 4), 28),
+                                      ((8, 8, 16, 16), (2, 2, 2, 2), 12)])
 @pytest.mark.parametrize("prec,tol", [(tm.TM_F64, 1e-9), (tm.TM_F32, 1e-3)])
 def test_one_launch_solve(L, agg, nv, prec, tol):
     one, ref = _gpu(L, agg, nv, prec, coarse_restart=48), _gpu(L, agg, nv, prec, coarse_restart=49)
@@ -44,9 +45,11 @@ def test_one_launch_solve(L, agg, nv, prec, tol):
     assert not one.unpack(1, prec, fx, b.shape).any()
 
 
-def test_one_launch_solve_of_a_batch():
+@pytest.mark.parametrize("steps", [0, 5])
+def test_one_launch_solve_of_a_batch(steps):
     L = (8, 8, 8, 8)
-    g = _gpu(L, (4, 4, 4, 4), 8, tm.TM_F64, max_rhs=3, coarse_tol=0.0, coarse_maxit=7, coarse_restart=3)
+    g = _gpu(L, (4, 4, 4, 4), 8, tm.TM_F64, max_rhs=3, coarse_tol=0.0, coarse_maxit=7, coarse_restart=3,
+             coarsest_steps=steps)
     v = inputs.gaussian_spinor(L, 11, 3)
     z = g.field(0, tm.TM_F64, 3)
     tm.tm_kcycle(g.h, tm.TM_F64, g.pack(0, tm.TM_F64, v, 3), z, 3)
