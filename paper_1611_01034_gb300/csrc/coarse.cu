@@ -331,7 +331,7 @@ __global__ void k_restrict(const void* __restrict__ P, const T* __restrict__ fin
         }
       }
     }
-    block_reduce16<T>(d, red, fin);
+    block_reduce_n<T, 16>(d, red, fin);
     if (l < 8) {
       const int ii = l >> 1, h = l & 1;
       if (i0 + ii < nv) out[h * nv + i0 + ii] = cx<T>{fin[4 * ii + 2 * h], fin[4 * ii + 2 * h + 1]};

@@ -541,7 +541,7 @@ __global__ void k_crestrict(const T* __restrict__ P2, const T* __restrict__ r1, 
           d[4 * jj + 2 * chi + 1] = pr.i;
         }
     }
-    block_reduce16<T>(d, red, fin);
+    block_reduce_n<T, 16>(d, red, fin);
     if (threadIdx.x < 8) {
       const int jj = threadIdx.x >> 1, h = threadIdx.x & 1;
       if (j0 + jj < nv2) out[h * nv2 + j0 + jj] = cx<T>{fin[4 * jj + 2 * h], fin[4 * jj + 2 * h + 1]};

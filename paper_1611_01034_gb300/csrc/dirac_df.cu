@@ -25,54 +25,6 @@ namespace tmamg {
 
 namespace {
 
-// A complex pair number with its real and imaginary parts as the lanes of packed
-// FP32 arithmetic: h = (re.h, im.h), l = (re.l, im.l).
-struct pk2 {
-  f2 h, l;
-};
-
-__device__ __forceinline__ pk2 two_sum2(f2 a, f2 b) {
-  const f2 s = a + b;
-  const f2 bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ void add_to(pk2& acc, pk2 a) {
-  const pk2 s = two_sum2(acc.h, a.h);
-  acc.h = s.h;
-  acc.l = acc.l + (s.l + a.l);
-}
-// a pair of scalars broadcast to both lanes: h, -h and -l
-struct bc2 {
-  f2 h, nh, nl;
-};
-__device__ __forceinline__ bc2 bc_pair(float h, float l) {
-  return {f2_pack(h, h), f2_pack(-h, -h), f2_pack(-l, -l)};
-}
-// acc += a x for x exact in FP32, and for x a pair (l l, 2^-48 relative, is dropped);
-// ne = minus the rounding error of a.h x.h and the cross terms
-__device__ __forceinline__ void fma_px(pk2& acc, bc2 a, f2 x) {
-  const f2 p = a.h * x;
-  f2 ne = lfma(a.nh, x, p);
-  ne = lfma(a.nl, x, ne);
-  const pk2 s = two_sum2(acc.h, p);
-  acc.h = s.h;
-  acc.l = acc.l + (s.l - ne);
-}
-__device__ __forceinline__ void fma_px(pk2& acc, bc2 a, pk2 x) {
-  const f2 p = a.h * x.h;
-  f2 ne = lfma(a.nh, x.h, p);
-  ne = lfma(a.nh, x.l, ne);
-  ne = lfma(a.nl, x.h, ne);
-  const pk2 s = two_sum2(acc.h, p);
-  acc.h = s.h;
-  acc.l = acc.l + (s.l - ne);
-}
-// i x
-__device__ __forceinline__ f2 times_i(f2 x) {
-  const float2 v = f2_unpack(x);
-  return f2_pack(-v.y, v.x);
-}
-__device__ __forceinline__ pk2 times_i(pk2 x) { return {times_i(x.h), times_i(x.l)}; }
 // i^q x, q at run time (exact; branch-free selects)
 __device__ __forceinline__ f2 times_ph(f2 x, int q) {
   const float2 v = f2_unpack(x);
@@ -127,7 +79,7 @@ __device__ __forceinline__ void hop_df_rt(const PT (&p)[12], const float4* __res
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const float4 u = __ldg(lk + (long)(fwd ? 3 * a + b : 3 * b + a) * V);
-      const bc2 ur = bc_pair(u.x, u.z), ui = bc_pair(cj * u.y, cj * u.w);
+      const pn2 ur = bc_pair(u.x, u.z), ui = bc_pair(cj * u.y, cj * u.w);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         fma_px(w[r][a], ur, h[r][b]);
@@ -254,13 +206,13 @@ __global__ void __launch_bounds__(128, 3) k_dslash_df(DfArgs a) {
       for (int j = i + 1; j < 6; ++j) {
         const float4 u = __ldg(c4 + (3 + q) * V);
         ++q;
-        const bc2 ur = bc_pair(u.x, u.z), ui = bc_pair(u.y, u.w), un = bc_pair(-u.y, -u.w);
+        const pn2 ur = bc_pair(u.x, u.z), ui = bc_pair(u.y, u.w), un = bc_pair(-u.y, -u.w);
         fma_px(y[i], ur, p[j]);
         fma_px(y[i], ui, ip[j]);
         fma_px(y[j], ur, p[i]);
         fma_px(y[j], un, ip[i]);
       }
-    const bc2 m = bc_pair(h == 0 ? -mus.h : mus.h, h == 0 ? -mus.l : mus.l);
+    const pn2 m = bc_pair(h == 0 ? -mus.h : mus.h, h == 0 ? -mus.l : mus.l);
 #pragma unroll
     for (int i = 0; i < 6; ++i) fma_px(y[i], m, ip[i]);
     // FP64 output: h + l (or sub - (h + l))

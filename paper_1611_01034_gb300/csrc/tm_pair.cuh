@@ -14,6 +14,7 @@
 //   f2d_bits: FP32 -> FP64 exactly (normal numbers).
 #pragma once
 #include "tm_internal.cuh"
+#include "tm_lane.cuh"
 
 namespace tmamg {
 
@@ -29,64 +30,66 @@ __device__ __forceinline__ dfl two_sum(float a, float b) {
   const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
   return {s, e};
 }
-// acc += a * b, a a pair, b an exact FP32 number
-__device__ __forceinline__ void fma_pf(dfl& acc, dfl a, float b) {
-  const float p = __fmul_rn(a.h, b);
-  float e = __fmaf_rn(a.h, b, -p);
-  e = __fmaf_rn(a.l, b, e);
-  const dfl s = two_sum(acc.h, p);
-  acc.h = s.h;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
-}
-// acc += a * b, both pairs (the l * l term, 2^-48 relative, is dropped)
-__device__ __forceinline__ void fma_pp(dfl& acc, dfl a, dfl b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  const dfl s = two_sum(acc.h, p);
-  acc.h = s.h;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
-}
-__device__ __forceinline__ dfl neg(dfl a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ void add_to(dfl& acc, dfl a) {
   const dfl s = two_sum(acc.h, a.h);
   acc.h = s.h;
   acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, a.l));
 }
 
-struct cdf {
-  dfl r, i;
+// A complex pair number with its real and imaginary parts as the lanes of packed
+// FP32 arithmetic: h = (re.h, im.h), l = (re.l, im.l).
+struct pk2 {
+  f2 h, l;
 };
 
-// acc += u * x (pairs)
-__device__ __forceinline__ void cfma_pp(cdf& acc, cdf u, cdf x) {
-  fma_pp(acc.r, u.r, x.r);
-  fma_pp(acc.r, neg(u.i), x.i);
-  fma_pp(acc.i, u.r, x.i);
-  fma_pp(acc.i, u.i, x.r);
+__device__ __forceinline__ pk2 two_sum2(f2 a, f2 b) {
+  const f2 s = a + b;
+  const f2 bb = s - a;
+  return {s, (a - (s - bb)) + (b - bb)};
 }
-// acc += conj(u) * x (pairs)
-__device__ __forceinline__ void cfmac_pp(cdf& acc, cdf u, cdf x) {
-  fma_pp(acc.r, u.r, x.r);
-  fma_pp(acc.r, u.i, x.i);
-  fma_pp(acc.i, u.r, x.i);
-  fma_pp(acc.i, neg(u.i), x.r);
+__device__ __forceinline__ void add_to(pk2& acc, pk2 a) {
+  const pk2 s = two_sum2(acc.h, a.h);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l + a.l);
 }
-// acc += u * x, x exact FP32
-__device__ __forceinline__ void cfma_pf(cdf& acc, cdf u, cx<float> x) {
-  fma_pf(acc.r, u.r, x.r);
-  fma_pf(acc.r, neg(u.i), x.i);
-  fma_pf(acc.i, u.r, x.i);
-  fma_pf(acc.i, u.i, x.r);
+// a factor as fma_px wants it: h, -h and -l
+struct pn2 {
+  f2 h, nh, nl;
+};
+// a pair broadcast to both lanes
+__device__ __forceinline__ pn2 bc_pair(float h, float l) {
+  return {f2_pack(h, h), f2_pack(-h, -h), f2_pack(-l, -l)};
 }
-__device__ __forceinline__ void cfmac_pf(cdf& acc, cdf u, cx<float> x) {
-  fma_pf(acc.r, u.r, x.r);
-  fma_pf(acc.r, u.i, x.i);
-  fma_pf(acc.i, u.r, x.i);
-  fma_pf(acc.i, neg(u.i), x.r);
+// each lane its own factor
+__device__ __forceinline__ pn2 lane_pair(pk2 a) {
+  const float2 h = f2_unpack(a.h), l = f2_unpack(a.l);
+  return {a.h, f2_pack(-h.x, -h.y), f2_pack(-l.x, -l.y)};
 }
-
+// acc += a x per lane, for x exact in FP32, and for x a pair (l l, 2^-48 relative, is dropped);
+// ne = minus the rounding error of a.h x.h and the cross terms
+__device__ __forceinline__ void fma_px(pk2& acc, pn2 a, f2 x) {
+  const f2 p = a.h * x;
+  f2 ne = lfma(a.nh, x, p);
+  ne = lfma(a.nl, x, ne);
+  const pk2 s = two_sum2(acc.h, p);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l - ne);
+}
+__device__ __forceinline__ void fma_px(pk2& acc, pn2 a, pk2 x) {
+  const f2 p = a.h * x.h;
+  f2 ne = lfma(a.nh, x.h, p);
+  ne = lfma(a.nh, x.l, ne);
+  ne = lfma(a.nl, x.h, ne);
+  const pk2 s = two_sum2(acc.h, p);
+  acc.h = s.h;
+  acc.l = acc.l + (s.l - ne);
+}
+// i x
+__device__ __forceinline__ f2 times_i(f2 x) {
+  const float2 v = f2_unpack(x);
+  return f2_pack(-v.y, v.x);
+}
+__device__ __forceinline__ pk2 times_i(pk2 x) { return {times_i(x.h), times_i(x.l)}; }
 // FP32 bits -> FP64 with integer operations (exact for normal numbers; FP32
 // subnormals, below 1.2e-38, become zero)
 __device__ __forceinline__ double f2d_bits(float f) {
@@ -123,6 +126,23 @@ __device__ __forceinline__ dfl d2pair(double x) {
 // pair -> FP64 (one FP64 addition)
 __device__ __forceinline__ double pair2d(dfl a) { return f2d_bits(a.h) + f2d_bits(a.l); }
 
-__device__ __forceinline__ cdf cx2pair(double re, double im) { return cdf{d2pair(re), d2pair(im)}; }
+// both parts of a complex FP64 number, with fewer instructions where both are in range: shifted left
+// by three, the high word has the FP32 mantissa in place and the exponent short of its bias; the
+// sign goes with both numbers whose difference is l
+__device__ __forceinline__ pk2 cx2pair(double re, double im) {
+  const unsigned hr = (unsigned)__double2hiint(re), lr = (unsigned)__double2loint(re);
+  const unsigned hm = (unsigned)__double2hiint(im), lm = (unsigned)__double2loint(im);
+  const unsigned er = ((hr >> 20) & 0x7ffu) - 920u, ei = ((hm >> 20) & 0x7ffu) - 920u;
+  if (max(er, ei) > 230u) {  // exponents beyond -103 .. 127, zeros too
+    const dfl a = d2pair(re), b = d2pair(im);
+    return {f2_pack(a.h, b.h), f2_pack(a.l, b.l)};
+  }
+  const unsigned ar = ((__funnelshift_l(lr, hr, 3) + 0x40000000u) & 0x7fffffffu) | (hr & 0x80000000u);
+  const unsigned ai = ((__funnelshift_l(lm, hm, 3) + 0x40000000u) & 0x7fffffffu) | (hm & 0x80000000u);
+  const unsigned br = (ar & 0xff800000u) - (23u << 23), bi = (ai & 0xff800000u) - (23u << 23);
+  const unsigned cr = br | ((lr >> 6) & 0x7fffffu), ci = bi | ((lm >> 6) & 0x7fffffu);
+  return {f2_pack(__uint_as_float(ar), __uint_as_float(ai)),
+          f2_pack(__uint_as_float(cr), __uint_as_float(ci)) - f2_pack(__uint_as_float(br), __uint_as_float(bi))};
+}
 
 }  // namespace tmamg
