@@ -300,12 +300,12 @@ struct DslashArgs {
 // link rows; groups of them vary fastest over the CTAs, so that the links and
 // clover of a site block are read from DRAM once.  FP32 waits on spinor loads
 // (DRAM at 37 %, issue 45 %) and gains from four CTAs per SM: 12 right-hand
-// sides at 48 x 24^3, 835 us -> 681 us (one per thread), 630 us (two).
-// Measured and left out: three per thread 624 us, four 749 us, two as packed
-// lanes 701 us (packing moves), five CTAs per SM 691 us, 64-thread CTAs 637 us.
+// sides at 48 x 24^3, 819 us (one per thread, unbounded) -> 687 us (one, four
+// CTAs) -> 622 us (two).  Measured and left out: three per thread, four, two as
+// packed lanes (packing moves), five CTAs per SM, 64-thread CTAs: 1 to 20 % slower.
 // FP64 is bound by the FP64 units and keeps one per thread, unbounded registers.
-template <typename T, bool RES, int RB>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_dslash(DslashArgs<T> a) {
+template <typename T, bool RES, int RB, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_dslash(DslashArgs<T> a) {
   const int ngrp = a.nrhs / RB;
   const int grp = ngrp == 1 ? 0 : (int)(blockIdx.x % ngrp);
   const int s = (ngrp == 1 ? blockIdx.x : blockIdx.x / ngrp) * blockDim.x + threadIdx.x;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_dslash(DslashAr
   hop(integral_constant<int, 2>{}, std::false_type{});
   hop(integral_constant<int, 3>{}, std::true_type{});
   hop(integral_constant<int, 3>{}, std::false_type{});
-  // acc = A p + i mu gamma5 p - acc / 2
+  // acc = A p + i mu gamma5 p - acc / 2, the large diagonal last: the sums before it round at a smaller size
   const T mus = ((c[0] + c[1] + c[2] + c[3]) & 1) ? a.mu + a.rho : a.mu;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_dslash(DslashAr
       cx<T>* y = acc[j] + 6 * h;
 #pragma unroll
       for (int k = 0; k < 6; ++k) y[k] = T(-0.5) * y[k];
-      herm6_lanes<T, T>(m, h == 0 ? -mus : mus, p, y);
+      herm6_lanes<T, T, true>(m, h == 0 ? -mus : mus, p, y);
     }
   }
 #pragma unroll
@@ -378,13 +378,13 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_dslash(DslashAr
   }
 }
 
-template <typename T, int RB>
+template <typename T, int RB, int MINB>
 void dslash_r(const DslashArgs<T>& a, cudaStream_t st) {
   dim3 grid((unsigned)((a.g.V + 127) / 128) * (unsigned)(a.nrhs / RB));
   if (a.b)
-    k_dslash<T, true, RB><<<grid, 128, 0, st>>>(a);
+    k_dslash<T, true, RB, MINB><<<grid, 128, 0, st>>>(a);
   else
-    k_dslash<T, false, RB><<<grid, 128, 0, st>>>(a);
+    k_dslash<T, false, RB, MINB><<<grid, 128, 0, st>>>(a);
 }
 
 template <typename T>
@@ -392,16 +392,16 @@ void launch_dslash(const T* gauge, const T* clover, const T* in, T* out, const T
                    double bc_t, int nrhs, cudaStream_t st, double rho) {
   DslashArgs<T> a{gauge, clover, in, out, b, g, (T)mu, (T)bc_t, nrhs, (T)rho};
   if constexpr (sizeof(T) == 4) {
-    a.nrhs = nrhs & ~1;
-    if (a.nrhs) dslash_r<T, 2>(a, st);
-    if (!(nrhs & 1)) return;
-    const long off = (long)a.nrhs * NR_SPINOR * g.V;
-    a.in += off;
-    a.out += off;
-    if (b) a.b += off;
-    a.nrhs = 1;
+    // two right-hand sides per thread where that still fills the chip with four CTAs per SM: 309 against
+    // 340 us at 48 x 24^3 and 11.1 against 12.3 us at 16^3 x 8, six right-hand sides, but 8.3 against
+    // 6.3 us for two there; an odd count in one launch (three at 48 x 24^3: 183 us; two and one: 202 us)
+    if (nrhs % 2 == 0 && (long)((g.V + 127) / 128) * (nrhs / 2) >= 4 * 152)
+      dslash_r<T, 2, 4>(a, st);
+    else
+      dslash_r<T, 1, 4>(a, st);
+  } else {
+    dslash_r<T, 1, 1>(a, st);
   }
-  dslash_r<T, 1>(a, st);
 }
 template void launch_dslash<double>(const double*, const double*, const double*, double*, const double*,
                                     const Lat&, double, double, int, cudaStream_t, double);
