@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(128, MINB) k_dslash(DslashArgs<T> a) {
       cx<T>* y = acc[j] + 6 * h;
 #pragma unroll
       for (int k = 0; k < 6; ++k) y[k] = T(-0.5) * y[k];
-      herm6_lanes<T, T, true>(m, h == 0 ? -mus : mus, p, y);
+      herm6_lanes<T, T>(m, h == 0 ? -mus : mus, p, y);
     }
   }
 #pragma unroll

@@ -225,22 +225,11 @@ __device__ __forceinline__ void hop_lanes(P p, const Link<T>& U, cx<R> (&acc)[12
     }
 }
 
-// y[h] += (M + i sg mu) x for one chirality: M Hermitian 6x6 packed as 36 reals;
-// DIAG_LAST: the large diagonal after the rest, for a y that starts at another term's size
-template <class R, class T, bool DIAG_LAST = false>
+// y[h] += (M + i sg mu) x for one chirality: M Hermitian 6x6 packed as 36 reals; the large
+// diagonal last, so that the sums before it round at a smaller size
+template <class R, class T>
 __device__ __forceinline__ void herm6_lanes(const T (&m)[36], T sgmu, const cx<R>* x, cx<R>* y) {
   const R mp = bcast<R>(sgmu), mn = bcast<R>(-sgmu);
-  auto diag = [&]() {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const R d = bcast<R>(m[i]);
-      y[i].r = lfma(d, x[i].r, y[i].r);
-      y[i].i = lfma(d, x[i].i, y[i].i);
-      y[i].r = lfma(mn, x[i].i, y[i].r);
-      y[i].i = lfma(mp, x[i].r, y[i].i);
-    }
-  };
-  if constexpr (!DIAG_LAST) diag();
   int k = 6;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
@@ -258,7 +247,14 @@ __device__ __forceinline__ void herm6_lanes(const T (&m)[36], T sgmu, const cx<R
       y[j].i = lfma(un, x[i].r, y[j].i);
     }
   }
-  if constexpr (DIAG_LAST) diag();
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const R d = bcast<R>(m[i]);
+    y[i].r = lfma(d, x[i].r, y[i].r);
+    y[i].i = lfma(d, x[i].i, y[i].i);
+    y[i].r = lfma(mn, x[i].i, y[i].r);
+    y[i].i = lfma(mp, x[i].r, y[i].i);
+  }
 }
 
 }  // namespace tmamg
