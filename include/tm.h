@@ -178,8 +178,9 @@ typedef struct {
      complement to coarse_tol / coarsest_tol with the host deciding each step;
      k in 1..64 = exactly k GMRES steps (a right-hand side whose residual
      estimate reaches the tolerance stops updating), all bookkeeping on the
-     device, captured once as a CUDA graph and replayed for every later
-     coarsest solve with the same buffers and twisted mass. */
+     device: for one right-hand side a single launch, else captured once as a
+     CUDA graph and replayed for every later coarsest solve with the same
+     buffers and twisted mass. */
   int coarsest_steps;
 } tm_params;
 
@@ -514,7 +515,7 @@ tm_status tm_synchronize(tm_handle* h);
  * nn, dslash_f32x2 (FP32-pair products and restart residuals),
  * level1_transfer (P2 and P2^dagger), oecg_operator, oecg_blas; a
  * graph-captured coarsest solve counts as coarse_oe with its node count as
- * launches).  With enable != 0
+ * launches, a coarse solve in one launch as one).  With enable != 0
  * every launch is counted (launches
  * and right-hand-side units) and the launches of class k are also bracketed
  * by a pair of CUDA events on the handle's stream when bit k of enable is set
