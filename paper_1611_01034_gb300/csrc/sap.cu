@@ -15,6 +15,7 @@
 // Block colour = parity of the sum of block coordinates; every dimension has
 // an even number (>= 2) of blocks, so no block touches itself or a block of
 // its own colour.
+#include <algorithm>
 #include <type_traits>
 
 #include "tm_kernels.h"
@@ -1291,12 +1292,16 @@ void launch_sap_oe_colour(const void* gauge, const void* clover, const void* din
   const int nblk_colour = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2;
   SapOeArgs<T> a{gauge, clover, dinv, b, x, sg, (T)mu, (T)bc_t, n_mr, colour, nrhs, (T)rho};
   if constexpr (std::is_same<T, float>::value) {
-    // whole pairs two to a thread; an odd one out alone (a pair with an idle lane
-    // costs 1.8 times a single right-hand side).  While one CTA per right-hand
-    // side still fits the chip at once (3 CTAs on each of 152 SMs) pairs would
-    // only make the longest CTA longer: 8^4 with 2 right-hand sides, 3 sweeps,
-    // 331 us in pairs, 276 us alone.
-    const bool alone = (long)nblk_colour * nrhs <= 3 * 152;
+    // whole pairs two to a thread and an odd one out in a launch of its own, or all
+    // alone, by the waves that each takes (168 registers: 12 warps per SM on 152 SMs;
+    // 255: 8; a wave of pairs lasts 1.15 times one of singles, a part of a first
+    // wave as long as a whole one).  Us of 3 FP32 sweeps, pairs (and one) against alone:
+    // 8^4 with 2 right-hand sides 331 to 276; 16 x 8^3 in 2^4 blocks with 3 556 to 313;
+    // 32 x 16^3 with 3 1299 to 1160, with 4 1309 to 1534, with 5 1894 to 1703; 16^4
+    // with 6 1023 to 1117.
+    const long w = (long)nblk_colour * ((sg.bsites / 2 + 31) / 32);  // warps per right-hand side
+    auto waves = [](long warps, int per_sm) { return std::max(1.0, (double)warps / (per_sm * 152)); };
+    const bool alone = waves(w * nrhs, 12) <= 1.15 * waves(w * (nrhs / 2), 8) + (nrhs & 1 ? waves(w, 12) : 0.0);
     a.nrhs = alone ? 0 : nrhs & ~1;
     if (a.nrhs) {
       bool b4 = s16 != ST_NATIVE;  // k_sap_oe4 has the block shape and 16-bit storage built in
