@@ -547,14 +547,14 @@ __device__ __forceinline__ void coarse_gmres(const ClArgs<T>& a) {
     beta = nrm;
     bad = st;
   }
-  if (a.once && bad)  // the caller has no other sign of it
+  if (a.once && (bad || dead))  // the caller has no other sign of it
     for (int i = tid; i < own; i += kClThreads) xe[o0 + i] = cx<T>{(T)NAN, (T)NAN};
   barrier();
-  // x_e, then x_o = D_oo^-1 (b_o - D_oe x_e)
+  // x_e, then x_o = D_oo^-1 (b_o - D_oe x_e); NaN from a CTA that gave up, whose neighbours' x_e may be old
   blocks(1, xe, nullptr, ac);
   for (int e = tid; e < own; e += kClThreads) {
     const int k = e / n, row = e % n;
-    x[(long)site_of(0, k) * n + row] = xe[o0 + e];
+    x[(long)site_of(0, k) * n + row] = dead ? cx<T>{(T)NAN, (T)NAN} : xe[o0 + e];
     ac[e] = b[(long)site_of(1, k) * n + row] - ac[e];
   }
   __syncthreads();

@@ -272,12 +272,19 @@ void check_flags(tm_handle* h) {
   sync(h);
   if (f) {
     CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
+    if (f & ERRF_TIMEOUT) raise(TM_ERR_TIMEOUT, "a bounded device-side wait ran out");  // explains the others
     if (f & ERRF_NOT_SU3) raise(TM_ERR_NOT_SU3, "gauge link not in SU(3) within 1e-10");
     if (f & ERRF_RANK) raise(TM_ERR_ARG, "test vectors are rank deficient on an aggregate");
     if (f & ERRF_SINGULAR) raise(TM_ERR_ARG, "singular coarse self block");
-    if (f & ERRF_TIMEOUT) raise(TM_ERR_TIMEOUT, "a bounded device-side wait ran out");
     raise(TM_ERR_NONFINITE, "non-finite value");
   }
+}
+
+// a non-finite number in a Krylov method: a wait that ran out in its preconditioner leaves
+// NaN behind and is reported as itself
+[[noreturn]] void raise_nonfinite(tm_handle* h, const char* what) {
+  check_flags(h);
+  raise(TM_ERR_NONFINITE, what);
 }
 
 template <typename T>
@@ -410,7 +417,7 @@ KrylovOut krylov(tm_handle* h, const std::string& tag, FA A, FAZ AZ, FM M, bool 
   TZ* Z = flexible ? W<TZ>(h, tag + "Z", (size_t)m * 2 * ncx) : nullptr;
   const long ld = 2 * ncx;
   const double bnorm = std::sqrt(norms2<T>(h, b, ncx, 1, bk)[0]);
-  if (!std::isfinite(bnorm)) raise(TM_ERR_NONFINITE, "non-finite right-hand side");
+  if (!std::isfinite(bnorm)) raise_nonfinite(h, "non-finite right-hand side");
   if (!x0) {
     Prof pf(h, bk);
     launch_zero<T>(x, 2 * ncx, h->st);
@@ -440,7 +447,7 @@ KrylovOut krylov(tm_handle* h, const std::string& tag, FA A, FAZ AZ, FM M, bool 
   std::vector<cd> H((size_t)(m + 1) * m), g(m + 1), sn(m), y(m);
   std::vector<double> cs(m);
   while (beta > tol * bnorm && out.iters < maxit) {
-    if (!std::isfinite(beta)) raise(TM_ERR_NONFINITE, "non-finite residual");
+    if (!std::isfinite(beta)) raise_nonfinite(h, "non-finite residual");
     {
       Prof pf(h, bk);
       launch_caxpby<T>(1.0 / beta, 0, Vb, 0, 0, Vb, ncx, h->st);
@@ -496,7 +503,7 @@ KrylovOut krylov(tm_handle* h, const std::string& tag, FA A, FAZ AZ, FM M, bool 
       CK(cudaMemcpyAsync(h->hsmall, h->dsmall, (4 * kMaxDots + 1) * sizeof(double), cudaMemcpyDeviceToHost, h->st));
       sync(h);
       const double hn = std::sqrt(h->hsmall[4 * kMaxDots]);
-      if (!std::isfinite(hn)) raise(TM_ERR_NONFINITE, "non-finite Arnoldi vector");
+      if (!std::isfinite(hn)) raise_nonfinite(h, "non-finite Arnoldi vector");
       std::vector<cd> col(m + 1, cd(0));
       for (int j = 0; j <= k; ++j)
         col[j] = cd(h->hsmall[2 * j] + h->hsmall[2 * kMaxDots + 2 * j],
@@ -657,8 +664,7 @@ std::vector<int> coarse_solve_graph(tm_handle* h, const OELevel& lv, const T* b,
       CKL();
     }
     h->coarse_iters += K;
-    check_flags(h);  // bounded waits
-    return std::vector<int>(1, K);
+    return std::vector<int>(1, K);  // no wait for the device; a timeout leaves its flag and NaN in x
   }
   T* to = W<T>(h, "gq_to", cv * nrhs);
   T* bh = W<T>(h, "gq_bh", cv * nrhs);
@@ -1563,7 +1569,7 @@ std::vector<KrylovOut> fgmres_b(tm_handle* h, const std::string& tag, int pk, FR
   read_norms();
   for (int r = 0; r < nb; ++r) {
     bnorm[r] = std::sqrt(hn_h[r]);
-    if (!std::isfinite(bnorm[r])) raise(TM_ERR_NONFINITE, "non-finite right-hand side");
+    if (!std::isfinite(bnorm[r])) raise_nonfinite(h, "non-finite right-hand side");
   }
   norms(x, nullptr);  // a zero start vector (the usual case) needs no product: r = b
   read_norms();
@@ -1672,7 +1678,7 @@ std::vector<KrylovOut> fgmres_b(tm_handle* h, const std::string& tag, int pk, FR
       for (int r = 0; r < nb; ++r) {
         if (!inner[r]) continue;
         const double hn = std::sqrt(hn_h[r]);
-        if (!std::isfinite(hn)) raise(TM_ERR_NONFINITE, "non-finite Arnoldi vector");
+        if (!std::isfinite(hn)) raise_nonfinite(h, "non-finite Arnoldi vector");
         const double* hr = hb + (size_t)r * 4 * (k + 1);
         cd* Hr = H.data() + (size_t)r * (m + 1) * m;
         cd* gr = g.data() + (size_t)r * (m + 1);
@@ -1741,7 +1747,7 @@ std::vector<KrylovOut> fgmres_b(tm_handle* h, const std::string& tag, int pk, FR
     for (int r = 0; r < nb; ++r) {
       if (!active[r]) continue;
       beta[r] = std::sqrt(hn_h[r]);
-      if (!std::isfinite(beta[r])) raise(TM_ERR_NONFINITE, "non-finite residual");
+      if (!std::isfinite(beta[r])) raise_nonfinite(h, "non-finite residual");
       active[r] = beta[r] > tol * bnorm[r] && out[r].iters < maxit;
     }
   }
@@ -3267,7 +3273,10 @@ tm_status tm_coarse_solve(tm_handle* h, int prec, const void* b, void* x, double
   else
     r = coarse_solve<float>(h, coarsest_level(h), static_cast<const float*>(b), static_cast<float*>(x), 1, tol,
                             maxit);
-  sync(h);
+  if (h->p.coarsest_steps > 0)
+    check_flags(h);  // the fixed-step solve does not
+  else
+    sync(h);
   if (iters) *iters = r[0];
   API_END
 }
@@ -3521,7 +3530,7 @@ tm_status tm_nn_pairs(tm_handle* h, const double* e0, void* r, void* e, int npai
     }
     dslash<float>(h, ep, rf + (size_t)p0 * fr, nullptr, nr);  // r = D e
   }
-  sync(h);
+  check_flags(h);
   API_END
 }
 

@@ -58,3 +58,20 @@ def test_one_launch_solve_of_a_batch(steps):
         z1 = g.field(0, tm.TM_F64)
         tm.tm_kcycle(g.h, tm.TM_F64, g.pack(0, tm.TM_F64, v[r]), z1, 1)
         assert rel(got[r], g.unpack(0, tm.TM_F64, z1, v[r].shape)) <= 1e-12
+
+
+@pytest.mark.parametrize("nrhs", [1, 2])
+def test_fixed_step_kcycle_does_not_wait(nrhs):
+    # with a fixed step count the host has nothing to decide: tm_kcycle returns while the stream is still busy
+    L = (8, 8, 8, 8)
+    g = _gpu(L, (4, 4, 4, 4), 8, tm.TM_F32, max_rhs=2, coarsest_steps=5)
+    v = g.pack(0, tm.TM_F32, inputs.gaussian_spinor(L, 11, nrhs), nrhs)
+    z = g.field(0, tm.TM_F32, nrhs)
+    tm.tm_kcycle(g.h, tm.TM_F32, v, z, nrhs)  # work buffers are made in the first call
+    tm.tm_synchronize(g.h)
+    slept = torch.cuda.Event()
+    torch.cuda._sleep(400_000_000)  # about 0.2 s of the stream
+    slept.record()
+    tm.tm_kcycle(g.h, tm.TM_F32, v, z, nrhs)
+    assert not slept.query()
+    tm.tm_synchronize(g.h)
