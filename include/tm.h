@@ -57,7 +57,7 @@ typedef enum {
   TM_ERR_CUDA = -2,          /* a CUDA runtime call or kernel launch failed */
   TM_ERR_OOM = -3,           /* device allocation failed */
   TM_ERR_NOT_CONVERGED = -4, /* solve hit maxit; x holds the best iterate */
-  TM_ERR_TIMEOUT = -5,       /* a bounded device-side wait ran out (tensor-core kernels) */
+  TM_ERR_TIMEOUT = -5,       /* a bounded device-side wait ran out (tc_spin_limit) */
   TM_ERR_NOT_SU3 = -6,       /* a link is not unitary with det 1 (tolerance 1e-10) */
   TM_ERR_NONFINITE = -7,     /* NaN or Inf in an input or a reduction */
   TM_ERR_STATE = -8          /* call out of order (e.g. solve before setup) */
@@ -152,11 +152,13 @@ typedef struct {
      and keeps (A(x) + i mu gamma5)^-1 of every odd site (144 reals per odd
      site in cycle_prec); SAP then runs in cycle_prec only. */
   int block_oe;
-  /* Polls of each pipeline mbarrier wait in the tensor-core kernel before it
-     gives up (0 = the default, 2^22).  On a timeout the kernel drains its
-     copies and MMAs, frees its tensor memory and the call returns
-     TM_ERR_TIMEOUT; the context stays usable.  Small values exist to test that
-     path. */
+  /* Polls of each pipeline mbarrier wait in the tensor-core kernel, and of each
+     grid-wide barrier in the one-launch coarse solve of one right-hand side,
+     before it gives up (0 = the default, 2^22).  On a timeout the kernel drains
+     its copies and MMAs, frees its tensor memory and the call returns
+     TM_ERR_TIMEOUT (tm_kcycle and tm_kcycle1 with coarsest_steps > 0 and one
+     right-hand side do not wait: tm_synchronize then returns it); the context
+     stays usable.  Small values exist to test that path. */
   int tc_spin_limit;
   /* Storage of P as read by the K-cycle's restriction P^dagger r and
      prolongation P e between the fine and the first coarse level

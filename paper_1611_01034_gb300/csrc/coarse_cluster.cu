@@ -47,7 +47,7 @@ constexpr int kClMaxRestart = 48;  // Hessenberg matrix in shared memory
 constexpr long kClMaxBytes = 6L << 20;
 constexpr size_t kClSmem = 200 * 1024;
 constexpr int kGridCtas = 152;          // of the whole-chip form, one per SM
-constexpr unsigned kGridPolls = 1u << 22;   // of one barrier before a CTA gives up
+constexpr unsigned kGridPolls = 1u << 22;   // of one barrier before a CTA gives up, unless the caller sets it
 
 struct ClLayout {  // shared memory, in bytes from its start
   size_t H, Q, g, y, hc, rc, part, dots, cf, w, bh, xs, pt, ac, nbr, site, vs, total;
@@ -104,6 +104,7 @@ struct ClArgs {
   double* gpart;       // [3][CTAs][2 (m + 1)] partial sums
   unsigned* count;     // barrier counter, zero at the start
   int* err;            // ERRF_TIMEOUT
+  unsigned polls;      // of one barrier before a CTA gives up
 };
 
 // complex number written by another SM earlier in the kernel: from L2
@@ -174,7 +175,7 @@ __device__ __forceinline__ void coarse_gmres(const ClArgs<T>& a) {
         unsigned polls = 0, seen;
         do {
           asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.count) : "memory");
-        } while (seen < target && ++polls < kGridPolls);
+        } while (seen < target && ++polls < a.polls);
         if (seen < target) {
           dead = 1;
           atomicOr(a.err, ERRF_TIMEOUT);
@@ -563,7 +564,7 @@ __device__ __forceinline__ void coarse_gmres(const ClArgs<T>& a) {
     a.out[2 * rhs] = iters;
     a.out[2 * rhs + 1] = bad;
   }
-  barrier();  // no CTA leaves while another may read its partial sums
+  if constexpr (!GRID) barrier();  // no CTA leaves while another may read its partial sums
 }
 
 template <typename T>
@@ -611,14 +612,14 @@ void launch_coarse_gmres(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* 
     cudaFuncSetAttribute(k_coarse_gmres<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmem);
     attr = true;
   }
-  ClArgs<T> a{Dc, Dinv, oe, b, x, V, u, xe, (T)mu_c, tol, restart, maxit, out, 0, nullptr, nullptr, nullptr};
+  ClArgs<T> a{Dc, Dinv, oe, b, x, V, u, xe, (T)mu_c, tol, restart, maxit, out, 0, nullptr, nullptr, nullptr, 0};
   k_coarse_gmres<T><<<kCl * nrhs, kClThreads, smem, st>>>(a);
 }
 
 template <typename T>
 void launch_coarse_gmres_grid(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* u, T* xe, int* out,
                               double* scratch, int* err, const OEGeom& oe, double mu_c, double tol, int restart,
-                              int maxit, bool once, cudaStream_t st) {
+                              int maxit, bool once, cudaStream_t st, unsigned polls) {
   const int q = (oe.nhalf + kGridCtas - 1) / kGridCtas, ctas = (oe.nhalf + q - 1) / q;
   const size_t smem = cl_layout(restart, q, 2 * oe.nv, 2 * sizeof(T)).total;
   static bool attr = false;
@@ -628,7 +629,8 @@ void launch_coarse_gmres_grid(const T* Dc, const T* Dinv, const T* b, T* x, T* V
   }
   unsigned* count = reinterpret_cast<unsigned*>(scratch);
   cudaMemsetAsync(count, 0, sizeof(double), st);
-  ClArgs<T> a{Dc, Dinv, oe, b, x, V, u, xe, (T)mu_c, tol, restart, maxit, out, once ? 1 : 0, scratch + 1, count, err};
+  ClArgs<T> a{Dc, Dinv, oe, b, x, V, u, xe, (T)mu_c, tol, restart, maxit, out, once ? 1 : 0, scratch + 1, count, err,
+              polls ? polls : kGridPolls};
   void* args[] = {&a};
   cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_coarse_gmres_grid<T>), dim3(ctas), dim3(kClThreads), args,
                               smem, st);
@@ -637,7 +639,7 @@ void launch_coarse_gmres_grid(const T* Dc, const T* Dinv, const T* b, T* x, T* V
   template void launch_coarse_gmres<T>(const T*, const T*, const T*, T*, T*, T*, T*, int*, const OEGeom&, double,     \
                                        double, int, int, int, cudaStream_t);                                          \
   template void launch_coarse_gmres_grid<T>(const T*, const T*, const T*, T*, T*, T*, T*, int*, double*, int*,        \
-                                            const OEGeom&, double, double, int, int, bool, cudaStream_t);
+                                            const OEGeom&, double, double, int, int, bool, cudaStream_t, unsigned);
 TM_INST(double)
 TM_INST(float)
 #undef TM_INST

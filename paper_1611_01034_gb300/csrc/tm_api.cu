@@ -660,7 +660,7 @@ std::vector<int> coarse_solve_graph(tm_handle* h, const OELevel& lv, const T* b,
     {
       Prof pf(h, PK_COARSE_OE, K);
       launch_coarse_gmres_grid<T>(Dc, Di, b, x, Vb, uo, xe, out, scratch, h->d_err, lv.oe, lv.mu_c, tol, K, K, true,
-                                  h->st);
+                                  h->st, (unsigned)h->p.tc_spin_limit);
       CKL();
     }
     h->coarse_iters += K;
@@ -809,7 +809,7 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
         launch_coarse_gmres<T>(Dc, Di, b, x, Vb, uo, xe, out, lv.oe, lv.mu_c, tol, m, maxit, nrhs, h->st);
       else
         launch_coarse_gmres_grid<T>(Dc, Di, b, x, Vb, uo, xe, out, scratch, h->d_err, lv.oe, lv.mu_c, tol, m, maxit,
-                                    false, h->st);
+                                    false, h->st, (unsigned)h->p.tc_spin_limit);
       CKL();
     }
     CK(cudaMemcpyAsync(ho, out, (size_t)2 * nrhs * sizeof(int), cudaMemcpyDeviceToHost, h->st));

@@ -233,11 +233,12 @@ void launch_coarse_gmres(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* 
 bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes);
 long coarse_grid_scratch_doubles(int restart);
 // the same for one right-hand side as a cooperative launch (scratch as above); once: a single
-// cycle of `restart` steps, which ends early when the estimate reaches tol, and no true residual
+// cycle of `restart` steps, which ends early when the estimate reaches tol, and no true residual;
+// polls: of one barrier before a CTA gives up (0: the default)
 template <typename T>
 void launch_coarse_gmres_grid(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* u, T* xe, int* out,
                               double* scratch, int* err, const OEGeom& oe, double mu_c, double tol, int restart,
-                              int maxit, bool once, cudaStream_t st);
+                              int maxit, bool once, cudaStream_t st, unsigned polls = 0);
 
 // ---- learned gauge-covariant layer (nn.cu) ------------------------------------
 // weights: complex float2 [Cout][Cin][9 directions][4][4]; hidden fields

@@ -75,3 +75,35 @@ def test_fixed_step_kcycle_does_not_wait(nrhs):
     tm.tm_kcycle(g.h, tm.TM_F32, v, z, nrhs)
     assert not slept.query()
     tm.tm_synchronize(g.h)
+
+
+@pytest.mark.parametrize("steps", [0, 5])
+def test_whole_chip_barrier_times_out_cleanly(steps):
+    # 64 coarse sites of 40 complex unknowns in FP64 are beyond the cluster's 6 MB: the whole chip, whose barriers
+    # may poll once.  The call says so, nothing stays behind on the handle, and a fresh handle solves.
+    L = (8, 8, 16, 16)
+    kw = dict(L=L, agg=(4, 4, 4, 4), nv=20, prec=tm.TM_F64, coarsest_steps=steps)
+    g = _gpu(**kw, tc_spin_limit=1)
+    rng = np.random.default_rng(5)
+    b = rng.standard_normal(g.coarse_shape()) + 1j * rng.standard_normal(g.coarse_shape())
+    fb, fx = g.pack(1, tm.TM_F64, b), g.field(1, tm.TM_F64)
+    v, z = g.pack(0, tm.TM_F64, inputs.gaussian_spinor(L, 11)), g.field(0, tm.TM_F64)
+
+    def kcycle():
+        tm.tm_kcycle(g.h, tm.TM_F64, v, z, 1)
+        tm.tm_synchronize(g.h)
+
+    bd = inputs.gaussian_spinor(L, 12)
+    for call in (lambda: tm.tm_coarse_solve(g.h, tm.TM_F64, fb, fx, 1e-8, 200), kcycle,
+                 lambda: tm.tm_solve(g.h, bd, np.zeros_like(bd), 1, 1e-6)):
+        with pytest.raises(tm.TMError) as e:
+            call()
+        assert e.value.status == tm.TM_ERR_TIMEOUT
+        tm.tm_synchronize(g.h)
+    fy = g.field(1, tm.TM_F64)
+    tm.tm_apply(g.h, 1, tm.TM_F64, fb, fy, 1)
+    g2 = _gpu(**kw)
+    f2 = g2.field(1, tm.TM_F64)
+    tm.tm_apply(g2.h, 1, tm.TM_F64, fb, f2, 1)
+    assert torch.equal(fy, f2)
+    assert tm.tm_solve(g2.h, bd, np.zeros_like(bd), 1, 1e-6)[0] == tm.TM_OK
