@@ -31,6 +31,7 @@
 //   cluster       13.6  19.3  23.9  27.4  29.0  80     -     -     -     -     -
 //   whole chip    19.8  22.9  25.4  27.4  26.0  28.0  32.8  35.4  50    74    92
 #include <cooperative_groups.h>
+#include <cuda.h>
 
 #include "tm_kernels.h"
 
@@ -586,17 +587,52 @@ long step_bytes(const OEGeom& oe, size_t real_bytes) {
 }
 }  // namespace
 
-bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes) {
-  const int q = (oe.nhalf + kCl - 1) / kCl;
-  return restart <= kClMaxRestart && step_bytes(oe, real_bytes) <= kClMaxBytes && nrhs * kCl <= 152 &&
-         cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total <= kClSmem;
+namespace {
+template <typename F>
+F driver_call(const char* name, unsigned version) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &found) != cudaSuccess ||
+      found != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  return reinterpret_cast<F>(p);
 }
 
-bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < kGridCtas)
-    return false;  // all CTAs have to be resident
+// SMs that work on this stream may run on (a green context has a part of the device's), and how
+// many of them are certain to share a cluster; false if the driver does not say (about 1 us)
+bool stream_sms(cudaStream_t st, int* sms, int* together) {
+  static const auto get_ctx =
+      driver_call<CUresult (*)(CUstream, CUcontext*, CUgreenCtx*)>("cuStreamGetCtx", 12050);
+  static const auto ctx_res =
+      driver_call<CUresult (*)(CUcontext, CUdevResource*, CUdevResourceType)>("cuCtxGetDevResource", 12040);
+  static const auto green_res =
+      driver_call<CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType)>("cuGreenCtxGetDevResource", 12040);
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r{};
+  if (!get_ctx || !ctx_res || !green_res || get_ctx(st, &ctx, &green) != CUDA_SUCCESS ||
+      (green ? green_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) : ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM)) != CUDA_SUCCESS)
+    return false;
+  *sms = (int)r.sm.smCount;
+  *together = (int)r.sm.smCoscheduledAlignment;
+  return true;
+}
+}  // namespace
+
+bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes, cudaStream_t st) {
+  const int q = (oe.nhalf + kCl - 1) / kCl;
+  if (restart > kClMaxRestart || step_bytes(oe, real_bytes) > kClMaxBytes || nrhs * kCl > 152 ||
+      cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total > kClSmem)
+    return false;
+  int sms = 0, together = 0;
+  return stream_sms(st, &sms, &together) && together >= kCl;  // a cluster's CTAs take an SM each
+}
+
+bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes, cudaStream_t st) {
+  int sms = 0, together = 0;
+  if (!stream_sms(st, &sms, &together) || sms < kGridCtas) return false;  // all CTAs have to be resident
   const int q = (oe.nhalf + kGridCtas - 1) / kGridCtas;
   return restart <= kClMaxRestart && cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total <= kClSmem;
 }

@@ -650,7 +650,7 @@ std::vector<int> coarse_solve_graph(tm_handle* h, const OELevel& lv, const T* b,
   const long ds = 4 * kMaxDots + 2;
   const T* Dc = static_cast<const T*>(lv.Dc);
   const T* Di = static_cast<const T*>(lv.Dinv);
-  if (nrhs == 1 && coarse_grid_fits(lv.oe, K, sizeof(T))) {
+  if (nrhs == 1 && coarse_grid_fits(lv.oe, K, sizeof(T), h->st)) {
     // one right-hand side: the K steps in one cooperative launch
     T* xe = W<T>(h, "gq_xe", cv);
     T* uo = W<T>(h, "gq_uo", cv);
@@ -793,8 +793,8 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
   bool use_tc = false;
   if constexpr (std::is_same<T, float>::value)
     use_tc = lv.tc && nrhs >= 2 && tc_supported(lv.oe.nv, nrhs, h->p.coarse_mma);  // one rhs: CUDA cores
-  const bool cluster = !use_tc && coarse_cluster_fits(lv.oe, m, nrhs, sizeof(T));
-  if (cluster || (nrhs == 1 && coarse_grid_fits(lv.oe, m, sizeof(T)))) {
+  const bool cluster = !use_tc && coarse_cluster_fits(lv.oe, m, nrhs, sizeof(T), h->st);
+  if (cluster || (nrhs == 1 && coarse_grid_fits(lv.oe, m, sizeof(T), h->st))) {
     // a system small enough for one cluster per right-hand side, or one right-hand side on the
     // whole chip: the whole solve in one launch
     T* xe = W<T>(h, "cb_xe", cv * nrhs);

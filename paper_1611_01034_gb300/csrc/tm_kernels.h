@@ -220,8 +220,8 @@ void launch_tc_schur(const TcGeom& tg, const OEGeom& oe, const float* ve, float*
                      cudaStream_t st, unsigned spin = 0);
 
 // ---- one-launch coarse solve (coarse_cluster.cu) --------------------------------
-// whether the odd-even system is small enough for a cluster per right-hand side
-bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes);
+// whether the odd-even system is small enough for a cluster per right-hand side, on this stream's SMs
+bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes, cudaStream_t st);
 // GMRES(restart) on the odd-even Schur complement, from zero, to tol or maxit steps, and x_o from
 // x_e.  b, x full vectors [rhs][Vc][n]; V [rhs][restart + 1][Vc/2][n], u, xe [rhs][Vc/2][n] work;
 // out [rhs][2] = steps, 1 if a norm was not finite.
@@ -230,7 +230,8 @@ void launch_coarse_gmres(const T* Dc, const T* Dinv, const T* b, T* x, T* V, T* 
                          double mu_c, double tol, int restart, int maxit, int nrhs, cudaStream_t st);
 
 // whether one right-hand side of this system can run on the whole chip (its vectors in shared memory)
-bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes);
+// and the stream has it (not a green context's part of it)
+bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes, cudaStream_t st);
 long coarse_grid_scratch_doubles(int restart);
 // the same for one right-hand side as a cooperative launch (scratch as above); once: a single
 // cycle of `restart` steps, which ends early when the estimate reaches tol, and no true residual;

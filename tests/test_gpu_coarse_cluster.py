@@ -5,6 +5,8 @@ first restart.  FP64 to 1e-9 (rounding of 24 Arnoldi steps of another summation 
 right-hand side gives zero in no steps; a batch through the K-cycle gives every right-hand side what it gets
 alone (FP64).
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -107,3 +109,60 @@ def test_whole_chip_barrier_times_out_cleanly(steps):
     tm.tm_apply(g2.h, 1, tm.TM_F64, fb, f2, 1)
     assert torch.equal(fy, f2)
     assert tm.tm_solve(g2.h, bd, np.zeros_like(bd), 1, 1e-6)[0] == tm.TM_OK
+
+
+class _Part:
+    """A stream on a part of the GPU's SMs (a green context), for the length of a with block."""
+
+    class Res(ctypes.Structure):  # CUdevResource, with room to spare
+        _fields_ = [("type", ctypes.c_int), ("pad", ctypes.c_ubyte * 92), ("sm", ctypes.c_uint * 64)]
+
+    def __init__(self, sms, flags):
+        cu, ref = ctypes.CDLL("libcuda.so.1"), ctypes.byref
+        dev, part, rest, n = self.Res(), self.Res(), self.Res(), ctypes.c_uint(1)
+        desc, self.ctx, self.st = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+        torch.cuda.synchronize()
+        for r in (cu.cuDeviceGetDevResource(0, ref(dev), 1),
+                  cu.cuDevSmResourceSplitByCount(ref(part), ref(n), ref(dev), ref(rest), flags, sms),
+                  cu.cuDevResourceGenerateDesc(ref(desc), ref(part), 1), cu.cuGreenCtxCreate(ref(self.ctx), desc, 0, 1),
+                  cu.cuGreenCtxStreamCreate(ref(self.st), self.ctx, 1, 0)):
+            if r:
+                pytest.skip(f"no green context on this driver ({r})")
+        self.cu = cu
+
+    def __enter__(self):
+        self.on = torch.cuda.stream(torch.cuda.ExternalStream(self.st.value))
+        self.on.__enter__()
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        self.on.__exit__(*exc)
+        self.cu.cuStreamDestroy_v2(self.st)
+        self.cu.cuGreenCtxDestroy(self.ctx)
+
+
+@pytest.mark.parametrize("sms,flags", [(16, 0), (4, 1)])  # whole clusters of SMs, or SMs from anywhere
+@pytest.mark.parametrize("L,nv", [((8, 8, 8, 8), 9), ((8, 8, 16, 16), 20)])  # a cluster's size, the whole chip's
+def test_stream_on_part_of_the_chip(L, nv, sms, flags):
+    # the one-launch forms need their CTAs resident together: on fewer SMs the step-by-step solve runs
+    rng = np.random.default_rng(3)
+    shape = tuple(n // 4 for n in L) + (2 * nv,)
+    b = rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+
+    def solves():
+        out = []
+        for steps in (0, 7):
+            g = _gpu(L, (4, 4, 4, 4), nv, tm.TM_F64, coarsest_steps=steps)
+            fx = g.field(1, tm.TM_F64)
+            it = tm.tm_coarse_solve(g.h, tm.TM_F64, g.pack(1, tm.TM_F64, b), fx, 1e-6, 24)
+            out.append((it, g.unpack(1, tm.TM_F64, fx, shape)))
+            g.close()
+        return out
+
+    whole = solves()
+    part = _Part(sms, flags)
+    with part:
+        got = solves()
+    for (i0, x0), (i1, x1) in zip(whole, got):
+        assert i0 == i1
+        assert rel(x1, x0) <= 1e-9
