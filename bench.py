@@ -166,8 +166,9 @@ def roofline_model(kind: str, wl: dict, units: float, launches: float, outer: di
         b and x on the half (FP32)
       restrict / prolong: P (24 N_v reals per site) + fine vectors
       level1 (D_c1 v): 9 n^2 complex per level-1 site + 2 vectors
-      coarse_oe (one odd-even Schur application, 2 launches): 9 n^2 complex per
-        coarsest site + 2 vectors
+      coarse_oe: 9 n^2 complex per coarsest site once per odd-even Schur
+        application (two launches, or many applications of a right-hand side
+        in one launch) + 2 vectors per right-hand side
       dslash_f64: 2232 flop per site and rhs (FP64 ALU, 1344 B per site)
       dslash_f32x2: 672 B per site in FP32 input + FP64 output + FP32-pair
         links and clover (576 + 576 B per site once per launch): HBM bytes
@@ -211,7 +212,11 @@ def roofline_model(kind: str, wl: dict, units: float, launches: float, outer: di
                 "peak": hbm, "peak_source": hbm_src}
     if kind == "coarse_oe":
         n, Vc = (2 * wl["nv2"], V2) if wl.get("levels", 2) == 3 else (n1, V1)
-        b = (9 * n * n * 2 * f * Vc + per * 2 * n * 2 * f * Vc) / 2  # two launches per application
+        op, vec = 9 * n * n * 2 * f * Vc, 2 * n * 2 * f * Vc
+        if per > outer["rhs"] / 2:  # a solve in one launch: every right-hand side's applications read the operator
+            b = per * (op + vec)
+        else:  # two launches per application of the batch
+            b = op / 2 + per * vec
         return {"bound": "hbm", "work": b, "unit": "GB/s", "peak": hbm, "peak_source": hbm_src}
     if kind == "dslash_f64":
         return {"bound": "alu", "work": 2232.0 * V * per / 1e3, "unit": "TFLOP/s", "peak": FP64_PEAK_TFLOPS,
@@ -762,8 +767,6 @@ def main_native(args):
                            prof[dom]["units"], prof[dom]["launches"], outer, peaks)
     if model is not None and prof[dom]["launches"]:
         avg_s = prof[dom]["ms"] / prof[dom]["launches"] / 1000.0
-        if dom == "coarse_oe":
-            avg_s *= 2  # the model counts one Schur application (two launches)
         achieved = model["work"] / avg_s / 1e9
         tr = ncu_traffic(args.workload, dom)
         roof = {"kernel": dom, "bound": model["bound"], "achieved": round(achieved, 3), "peak": model["peak"],

@@ -517,8 +517,8 @@ tm_status tm_synchronize(tm_handle* h);
  * nn, dslash_f32x2 (FP32-pair products and restart residuals),
  * level1_transfer (P2 and P2^dagger), oecg_operator, oecg_blas; a
  * graph-captured coarsest solve counts as coarse_oe with its node count as
- * launches, a coarse solve in one launch as one).  With enable != 0
- * every launch is counted (launches
+ * launches, a coarse solve in one launch as one, both with their operator
+ * applications as units).  With enable != 0 every launch is counted (launches
  * and right-hand-side units) and the launches of class k are also bracketed
  * by a pair of CUDA events on the handle's stream when bit k of enable is set
  * (enable = -1 times every class).  tm_profile resets the totals;

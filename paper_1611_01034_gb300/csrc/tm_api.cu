@@ -820,6 +820,9 @@ std::vector<int> coarse_solve(tm_handle* h, const OELevel& lv, const T* b, T* x,
       if (ho[2 * r + 1]) raise(TM_ERR_NONFINITE, "non-finite coarse solve");
       steps[r] = ho[2 * r];
       h->coarse_iters += steps[r];
+      // operator applications as the step-by-step solve counts them: reduced right-hand side,
+      // steps, a residual per cycle (the scope above has counted the odd sites of x)
+      if (h->prof) h->prof_units[PK_COARSE_OE] += 1 + steps[r] + (steps[r] + m - 1) / m;
     }
     return steps;
   }

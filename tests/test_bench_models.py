@@ -1,7 +1,8 @@
 """The roofline work models of bench.py on CPU: the odd-even SAP flop count
 against a term-by-term recount for 4^4 blocks, the interior-hop average for
-other block shapes, and the vector bytes of the pair-arithmetic Arnoldi steps
-against an explicit sum over the steps of the cycles."""
+other block shapes, the vector bytes of the pair-arithmetic Arnoldi steps
+against an explicit sum over the steps of the cycles, and the bytes of the
+coarsest Schur complement for both forms of its solve."""
 import bench
 
 
@@ -39,3 +40,16 @@ def test_pair_arnoldi_bytes_per_cycle():
     for kc in (4, 4, 3):  # 11 iterations in cycles of at most 4
         per_rhs += sum(16 * (3 * k + 7) for k in range(1, kc + 1)) + 8 * kc + 32
     assert abs(m["work"] * 98 - per_rhs * 12 * V * 6) < 1e-3 * m["work"]
+
+
+def test_coarse_solve_bytes():
+    wl = dict(bench.WORKLOADS[bench.DEFAULT_WORKLOAD])
+    V2, n = bench.volumes(wl)[2], 2 * wl["nv2"]
+    op, vec = 9 * n * n * 8 * V2, 2 * n * 8 * V2
+    peaks = {"hbm_gbs": 6795.1}
+    # 40 applications to 6 right-hand sides, two launches each
+    m = bench.roofline_model("coarse_oe", wl, 40 * 6, 80, {"rhs": 6}, peaks)
+    assert abs(m["work"] * 80 - 40 * (op + 6 * vec)) < 1e-9 * m["work"] * 80
+    # 3 solves in one launch each, 20 applications to one right-hand side
+    m = bench.roofline_model("coarse_oe", wl, 3 * 20, 3, {"rhs": 1}, peaks)
+    assert abs(m["work"] * 3 - 60 * (op + vec)) < 1e-9 * m["work"] * 3

@@ -35,12 +35,17 @@ def test_one_launch_solve(L, agg, nv, prec, tol):
     rng = np.random.default_rng(3)
     b = rng.standard_normal(one.coarse_shape()) + 1j * rng.standard_normal(one.coarse_shape())
     for target, maxit in ((0.0, 24), (1e-4, 200)):
-        xs, its = [], []
+        xs, its, units = [], [], []
         for g in (one, ref):
             fx = g.field(1, prec)
+            tm.tm_profile(g.h, True)
             its.append(tm.tm_coarse_solve(g.h, prec, g.pack(1, prec, b), fx, target, maxit))
+            units.append(tm.tm_profile_read(g.h)["coarse_oe"]["units"])
+            tm.tm_profile(g.h, 0)
             xs.append(g.unpack(1, prec, fx, b.shape))
         assert its[0] == its[1]
+        # operator applications; step by step the host may have one more under way when it stops
+        assert units[1] - 1 <= units[0] <= units[1], units
         assert rel(xs[0], xs[1]) <= tol
     fx = one.pack(1, prec, b)
     assert tm.tm_coarse_solve(one.h, prec, one.pack(1, prec, 0 * b), fx, 0.0, 24) == 0
