@@ -1285,6 +1285,45 @@ void sap_oe4_s(const SapOeArgs<float>& a, int nblocks, cudaStream_t st) {
 
 }  // namespace
 
+namespace {
+// time of `warps` warps, up to four per SM at once in each of N slots: whole waves of N and the rest, in
+// units of one slot alone
+template <int N>
+double wave_time(long warps, const double (&t)[N]) {
+  const long c = std::max(1L, (warps + 4 * kSms - 1) / (4 * kSms));
+  return (double)(c / N) * t[N - 1] + (c % N ? t[c % N - 1] : 0.0);
+}
+}  // namespace
+
+// Whole pairs two to a thread and an odd one out in a launch of its own, or all alone: by the waves that each
+// takes.  An SM holds three slots of four warps of k_sap_oe on one right-hand side and of k_sap_oe4 (168
+// registers), two of k_sap_oe on pairs (255); the times of one, two and three slots are relative to one slot of
+// right-hand sides alone.  A lone FP32 right-hand side whose blocks in flight hold more than 64 MB of operator
+// reads it from DRAM in every half-step (twice the time; others on the same block share it in L2).  Us of 3
+// sweeps, alone against pairs (and one), 4^4 blocks:
+//                 FP32 operator                               16-bit
+//   rhs           2          3          4          6          2          3          4          6
+//   16^3 x 8   306  381   395  676   396  394   499  535   271  356   331  615   332  366   423  505
+//   16^4       431  420   556  778   877  599  1112 1013   332  369   429  639   645  523   833  715
+//   32 x 16^3  953  734  1154 1308  1512 1300  2096 1857   655  534   847  906  1129 1027  1557 1412
+//   24^3 x 16 1343 1337  1808 2448  2292 2008  3300 2844   897  800  1305 1293  1699 1483  2480 2122
+// and 2^4 blocks at 16^3 x 8: 2 right-hand sides 642 426, 3 732 745 (FP32), 615 429, 738 743.  Over 722 such pairs
+// of times (blocks of 16 to 256 sites, 8^4 to 48 x 24^3, 2 to 12 right-hand sides) the form taken is at most
+// 1.08 times slower than the other.
+extern "C" int tmamg_sap_oe_paired(const int* nb, const int* blk, int nrhs, int s16) {
+  constexpr double alone[3] = {1, 1.3, 1.65}, pairs[2] = {1.3, 1.75}, pairs4[3] = {1.35, 1.93, 2.64};
+  const long blocks = (long)nb[0] * nb[1] * nb[2] * nb[3] / 2;  // of one colour
+  const int bsites = blk[0] * blk[1] * blk[2] * blk[3];
+  const long wpb = (bsites / 2 + 31) / 32, w = blocks * wpb;  // warps per block, per right-hand side
+  const bool b4 = s16 != ST_NATIVE && blk[0] == 4 && blk[1] == 4 && blk[2] == 4 && blk[3] == 4;
+  double paired = b4 ? wave_time(w * (nrhs / 2), pairs4) : wave_time(w * (nrhs / 2), pairs);
+  if (nrhs & 1) {
+    const long in_flight = std::min(blocks, 12 * kSms / wpb) * bsites * (s16 == ST_NATIVE ? 768 : 384);
+    paired += wave_time(w, alone) * (in_flight > 64e6 ? 2 : 1) + 0.4;
+  }
+  return nrhs < 2 || wave_time(w * nrhs, alone) <= paired ? 0 : nrhs & ~1;
+}
+
 template <typename T>
 void launch_sap_oe_colour(const void* gauge, const void* clover, const void* dinv, const T* b, T* x,
                           const SapGeom& sg, double mu, double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st,
@@ -1292,17 +1331,7 @@ void launch_sap_oe_colour(const void* gauge, const void* clover, const void* din
   const int nblk_colour = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2;
   SapOeArgs<T> a{gauge, clover, dinv, b, x, sg, (T)mu, (T)bc_t, n_mr, colour, nrhs, (T)rho};
   if constexpr (std::is_same<T, float>::value) {
-    // whole pairs two to a thread and an odd one out in a launch of its own, or all
-    // alone, by the waves that each takes (168 registers: 12 warps per SM on 152 SMs;
-    // 255: 8; a wave of pairs lasts 1.15 times one of singles, a part of a first
-    // wave as long as a whole one).  Us of 3 FP32 sweeps, pairs (and one) against alone:
-    // 8^4 with 2 right-hand sides 331 to 276; 16 x 8^3 in 2^4 blocks with 3 556 to 313;
-    // 32 x 16^3 with 3 1299 to 1160, with 4 1309 to 1534, with 5 1894 to 1703; 16^4
-    // with 6 1023 to 1117.
-    const long w = (long)nblk_colour * ((sg.bsites / 2 + 31) / 32);  // warps per right-hand side
-    auto waves = [](long warps, int per_sm) { return std::max(1.0, (double)warps / (per_sm * 152)); };
-    const bool alone = waves(w * nrhs, 12) <= 1.15 * waves(w * (nrhs / 2), 8) + (nrhs & 1 ? waves(w, 12) : 0.0);
-    a.nrhs = alone ? 0 : nrhs & ~1;
+    a.nrhs = tmamg_sap_oe_paired(sg.nb, sg.blk, nrhs, s16);
     if (a.nrhs) {
       bool b4 = s16 != ST_NATIVE;  // k_sap_oe4 has the block shape and 16-bit storage built in
       for (int d = 0; d < 4; ++d) b4 = b4 && sg.blk[d] == 4;

@@ -10,6 +10,8 @@
 
 namespace tmamg {
 
+constexpr int kSms = 152;  // of a GB300
+
 // ---- fine fields (dirac.cu) ----------------------------------------------
 // natural layout: [rhs][V][4 spin][3 colour] complex128, interleaved re/im
 template <typename T>
@@ -64,6 +66,9 @@ template <typename T>
 void launch_sap_oe_colour(const void* gauge, const void* clover, const void* dinv, const T* b, T* x,
                           const SapGeom& sg, double mu, double bc_t, int n_mr, int colour, int nrhs, cudaStream_t st,
                           double rho = 0.0, int s16 = 0);
+// how many of nrhs right-hand sides (a lattice of nb blocks of blk sites) the FP32 form runs two to a
+// thread; the others run alone
+extern "C" int tmamg_sap_oe_paired(const int* nb, const int* blk, int nrhs, int s16);
 // 16-bit copy of `planes` chunk planes of an FP32 field, the sites of each SAP block side by
 // side (even ones first); odd_only: a field over the odd sites (index s >> 1)
 void launch_to16_blocks(const float* in, void* out, const SapGeom& sg, int planes, bool odd_only, int kind,
