@@ -326,9 +326,12 @@ template <typename T>
 void sap_sweeps(tm_handle* h, const T* b, T* x, int sweeps, int nrhs) {
   if (h->p.block_oe && (sizeof(T) == 8) != (h->p.cycle_prec == TM_F64))
     raise(TM_ERR_ARG, "with block_oe = 1 the SAP smoother runs in cycle_prec");
+  const int paired = h->p.block_oe && sizeof(T) == 4
+                         ? tmamg_sap_oe_paired(h->sg.nb, h->sg.blk, nrhs, h->g16 ? h->p.sap_prec : ST_NATIVE) : 0;
+  const int launches = paired > 0 && paired < nrhs ? 2 : 1;  // pairs and an odd one out
   for (int s = 0; s < sweeps; ++s)
     for (int colour = 0; colour < 2; ++colour) {
-      Prof pf(h, PK_SAP, nrhs);
+      Prof pf(h, PK_SAP, nrhs, launches);
       if (h->p.block_oe && h->g16)  // 16-bit links, clover and D_oo^-1 (sap_prec)
         launch_sap_oe_colour<T>(h->g16, h->c16, h->dinv16, b, x, h->sg, h->p.mu, h->p.bc_t, h->p.mr_iters, colour,
                                 nrhs, h->st, h->rho, h->p.sap_prec);

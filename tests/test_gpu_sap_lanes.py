@@ -55,7 +55,11 @@ def test_odd_even_sap_batches(L, blk, nrhs, pairs, prec, tol):
     g = GPU(U, m0=-0.3, c_sw=1.3, mu=0.05, nv=2, agg=blk, sap_block=blk, cycle_prec=F32, max_rhs=nrhs, block_oe=1,
             sap_prec=prec)
     b, x0 = inputs.gaussian_spinor(L, 1, nrhs), inputs.gaussian_spinor(L, 2, nrhs)
+    tm.tm_profile(g.h, True)
     got, got0 = _sweeps(g, b, x0, 2), _sweeps(g, None, x0, 1)
+    two = 0 < paired(L, blk, nrhs, prec) < nrhs  # launches per colour: pairs and an odd one out
+    assert tm.tm_profile_read(g.h)["sap"]["launches"] == 3 * 2 * (2 if two else 1)
+    tm.tm_profile(g.h, 0)
     for r in range(nrhs):
         assert rel(got[r], _sweeps(g, b[r:r + 1], x0[r:r + 1], 2)[0]) <= 5e-6
         assert rel(got0[r], _sweeps(g, None, x0[r:r + 1], 1)[0]) <= 5e-6
