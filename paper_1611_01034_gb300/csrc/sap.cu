@@ -59,9 +59,11 @@ __device__ __forceinline__ void block_hops(const cx<T>* __restrict__ rs, int BS,
   }
 }
 
-// FP32: two CTAs per SM (128 registers); FP64 would spill heavily at that bound
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_sap(SapArgs<T> a) {
+// FP32: two CTAs per SM (128 registers); FP64 would spill heavily at that bound.
+// MT: most threads of a CTA, one per site; blocks of more than 256 sites (1024 at
+// most) take the 64 registers that are left for them and spill the rest.
+template <typename T, int MT>
+__global__ void __launch_bounds__(MT, sizeof(T) == 4 && MT == 256 ? 2 : 1) k_sap(SapArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SapGeom& sg = a.sg;
   const Lat& g = sg.g;
@@ -488,7 +490,8 @@ void launch_sap_colour(const T* gauge, const T* clover, const T* b, T* x, const 
   const size_t smem = 12 * sg.bsites * sizeof(cx<T>) + 32 * 3 * sizeof(T);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_sap<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_sap<T, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_sap<T, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
   const int nblk_colour = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2;
@@ -507,7 +510,10 @@ void launch_sap_colour(const T* gauge, const T* clover, const T* b, T* x, const 
     }
   }
   dim3 grid(nblk_colour * nrhs);
-  k_sap<T><<<grid, threads, smem, st>>>(a);
+  if (threads <= 256)
+    k_sap<T, 256><<<grid, threads, smem, st>>>(a);
+  else
+    k_sap<T, 1024><<<grid, threads, smem, st>>>(a);
 }
 
 template void launch_sap_colour<double>(const double*, const double*, const double*, double*, const SapGeom&,
@@ -587,11 +593,16 @@ struct SapOeArgs {
   T rho;  // odd sites carry mu + rho (D_oo^-1 is built with it)
 };
 
-template <class R, int S>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
+// MT: most threads of a CTA, one per even site.  Blocks of more than 256 sites
+// (1024 at most) run one right-hand side at a time and keep e_e, which only its
+// own thread reads, out of shared memory, which the two fields that the hops
+// gather fill.
+template <class R, int S, int MT>
+__global__ void __launch_bounds__(MT, MT > 128 ? 1 : sizeof(R) == 4 ? 3 : 2)
     k_sap_oe(SapOeArgs<typename LaneOf<R>::T> a) {
   using T = typename LaneOf<R>::T;
   constexpr bool BLOCKED = S != ST_NATIVE;  // operator in block order
+  constexpr bool E_OWN = MT > 128;          // e_e in the thread's own storage
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SapGeom& sg = a.sg;
   const Lat& g = sg.g;
@@ -599,7 +610,8 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
   cx<R>* ev = reinterpret_cast<cx<R>*>(smem_raw);  // [12][HB] even-site values (rho, then e_e)
   cx<R>* od = ev + 12 * HB;                         // [12][HB] odd-site values
   cx<R>* ee = od + 12 * HB;                         // [12][HB] e_e
-  R* red = reinterpret_cast<R*>(ee + 12 * HB);      // 3 per warp
+  R* red = reinterpret_cast<R*>(E_OWN ? ee : ee + 12 * HB);  // 3 per warp
+  cx<R> e_own[E_OWN ? 12 : 1];
   const int groups = a.nrhs / LaneOf<R>::n;  // right-hand sides fastest over the CTAs (operator reuse in L2)
   const long fs = (long)NR_SPINOR * g.V;
   const long r0 = (long)(blockIdx.x % groups) * LaneOf<R>::n * fs;
@@ -832,7 +844,10 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
 #pragma unroll
           for (int i = 0; i < 12; ++i) {
             rho[i] = cx<R>{lfma(hf, acc[i].r, rho[i].r), lfma(hf, acc[i].i, rho[i].i)};
-            st_shared(ee + i * HB + j, czero<R>());
+            if constexpr (E_OWN)
+              e_own[i] = czero<R>();
+            else
+              st_shared(ee + i * HB + j, czero<R>());
             st_shared(ev + i * HB + j, store_e ? czero<R>() : rho[i]);
           }
         }
@@ -859,10 +874,17 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
           const R nr = bcast<R>(T(0)) - ar, ni = bcast<R>(T(0)) - ai;
 #pragma unroll
           for (int i = 0; i < 12; ++i) {
-            cx<R> e = ld_shared(ee + i * HB + j);
+            cx<R> e;
+            if constexpr (E_OWN)
+              e = e_own[i];
+            else
+              e = ld_shared(ee + i * HB + j);
             e.r = lfma(ni, rho[i].i, lfma(ar, rho[i].r, e.r));
             e.i = lfma(ai, rho[i].r, lfma(ar, rho[i].i, e.i));
-            if (!store_e) st_shared(ee + i * HB + j, e);
+            if constexpr (E_OWN)
+              e_own[i] = e;
+            else if (!store_e)
+              st_shared(ee + i * HB + j, e);
             cx<R> q = rho[i];  // rho - alpha q
             q.r = lfma(ai, acc[i].i, lfma(nr, acc[i].r, q.r));
             q.i = lfma(ni, acc[i].r, lfma(nr, acc[i].i, q.i));
@@ -874,17 +896,24 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 2)
   }
 }
 
-template <class R, int S>
-void sap_oe_s(SapOeArgs<typename LaneOf<R>::T> a, int nblocks, cudaStream_t st) {
+template <class R, int S, int MT>
+void sap_oe_t(const SapOeArgs<typename LaneOf<R>::T>& a, int nblocks, cudaStream_t st) {
   const int HB = a.sg.bsites / 2;
   const int threads = (HB + 31) / 32 * 32;
-  const size_t smem = 36 * (size_t)HB * sizeof(cx<R>) + (threads / 32) * 3 * sizeof(R);
+  const size_t smem = (MT > 128 ? 24 : 36) * (size_t)HB * sizeof(cx<R>) + (threads / 32) * 3 * sizeof(R);
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_sap_oe<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_sap_oe<R, S, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
-  k_sap_oe<R, S><<<dim3(nblocks * (a.nrhs / LaneOf<R>::n)), threads, smem, st>>>(a);
+  k_sap_oe<R, S, MT><<<dim3(nblocks * (a.nrhs / LaneOf<R>::n)), threads, smem, st>>>(a);
+}
+template <class R, int S>
+void sap_oe_s(const SapOeArgs<typename LaneOf<R>::T>& a, int nblocks, cudaStream_t st) {
+  if constexpr (LaneOf<R>::n == 1) {
+    if (a.sg.bsites > 256) return sap_oe_t<R, S, 512>(a, nblocks, st);
+  }
+  sap_oe_t<R, S, 128>(a, nblocks, st);
 }
 
 // ===========================================================================
@@ -1321,7 +1350,8 @@ extern "C" int tmamg_sap_oe_paired(const int* nb, const int* blk, int nrhs, int 
     const long in_flight = std::min(blocks, 12 * kSms / wpb) * bsites * (s16 == ST_NATIVE ? 768 : 384);
     paired += wave_time(w, alone) * (in_flight > 64e6 ? 2 : 1) + 0.4;
   }
-  return nrhs < 2 || wave_time(w * nrhs, alone) <= paired ? 0 : nrhs & ~1;
+  // blocks of more than 256 sites have no form for pairs
+  return nrhs < 2 || bsites > 256 || wave_time(w * nrhs, alone) <= paired ? 0 : nrhs & ~1;
 }
 
 template <typename T>

@@ -83,3 +83,22 @@ def test_full_block_sap_batch(prec, tol):
         got = g.unpack(0, prec, fx, x0.shape, nrhs)
         for r in range(nrhs):
             assert rel(got[r], sap.smooth(np.zeros_like(b[r]) if bb is None else b[r], x0[r], 2)) <= tol
+
+
+@pytest.mark.parametrize("L,blk,oe,prec,store,tol", [
+    ((8, 8, 8, 16), (4, 4, 4, 8), 0, tm.TM_F32, tm.TM_F32, 1e-4), ((8, 8, 8, 16), (4, 4, 4, 8), 1, tm.TM_F32, tm.TM_F32, 1e-4),
+    ((8, 8, 16, 16), (4, 4, 8, 8), 0, tm.TM_F64, tm.TM_F32, 1e-10), ((8, 8, 16, 16), (4, 4, 8, 8), 1, tm.TM_F64, tm.TM_F32, 1e-10),
+    ((8, 8, 16, 16), (4, 4, 8, 8), 1, tm.TM_F32, tm.TM_F16, 5e-3), ((6, 6, 12, 12), (3, 3, 6, 6), 0, tm.TM_F32, tm.TM_F32, 1e-4)])
+def test_blocks_of_more_than_256_sites(L, blk, oe, prec, store, tol):
+    # up to the 1024 sites that tm_create takes; two right-hand sides, the second with b = 0
+    U = inputs.gauge_field(L, 0.5, 23)
+    g = GPU(U, m0=-0.3, c_sw=1.3, mu=0.05, nv=2, agg=(L[0] // 2, L[1] // 2, 2, 2), sap_block=blk, cycle_prec=prec,
+            max_rhs=2, block_oe=oe, sap_prec=store)
+    sap = SAP(Operator(U, -0.3, 1.3, 0.05), blk, n_mr=4, block_oe=bool(oe))
+    b, x0 = inputs.gaussian_spinor(L, 1, 2), inputs.gaussian_spinor(L, 2, 2)
+    b[1] = 0
+    fx = g.pack(0, prec, x0, 2)
+    tm.tm_sap(g.h, prec, g.pack(0, prec, b, 2), fx, 1, 2)
+    got = g.unpack(0, prec, fx, x0.shape, 2)
+    for r in range(2):
+        assert rel(got[r], sap.smooth(b[r], x0[r], 1)) <= tol
