@@ -46,8 +46,9 @@ __device__ __forceinline__ int coarse_of(const AggGeom& ag, const int c[4]) {
 // orthonormalisation: per (aggregate, chirality) classical Gram-Schmidt
 // applied twice, giving the Q of the thin QR with a real positive R diagonal
 // ===========================================================================
-template <typename T>
-__global__ void k_orthonormalise(T* P, AggGeom ag, int* err) {
+// MT: most threads, one per site (FP64 uses 80 registers, 64 beyond 672 sites)
+template <typename T, int MT>
+__global__ void __launch_bounds__(MT, 1) k_orthonormalise(T* P, AggGeom ag, int* err) {
   __shared__ T red[32 * 16];
   const int a = blockIdx.x, chi = blockIdx.y, nv = ag.nv;
   const int l = threadIdx.x;
@@ -279,7 +280,13 @@ void launch_orthonormalise(T* P, const AggGeom& ag, int* err, cudaStream_t st) {
     return;
   }
   dim3 grid(ag.gc.V, 2);
-  k_orthonormalise<T><<<grid, threads, 0, st>>>(P, ag, err);
+  if constexpr (sizeof(T) == 8) {
+    if (threads <= 672) {
+      k_orthonormalise<T, 672><<<grid, threads, 0, st>>>(P, ag, err);
+      return;
+    }
+  }
+  k_orthonormalise<T, 1024><<<grid, threads, 0, st>>>(P, ag, err);
 }
 
 // ===========================================================================
@@ -294,9 +301,10 @@ __device__ __forceinline__ void ld_pcol(const void* __restrict__ P, int i, long 
     ld_cx16<T, S, 12>(static_cast<const unsigned short*>(P) + (long)i * NR_SPINOR * V, V, s, p);
 }
 
-// one right-hand side, FP64 and narrow aggregates (k_restrict_l takes other FP32 batches)
-template <typename T, int S>
-__global__ void k_restrict(const void* __restrict__ P, const T* __restrict__ fine, T* __restrict__ coarse,
+// one right-hand side, FP64 and narrow aggregates (k_restrict_l takes other FP32 batches);
+// MT: most threads, one per site (FP64 uses 128 registers, 64 beyond 512 sites)
+template <typename T, int S, int MT>
+__global__ void __launch_bounds__(MT, 1) k_restrict(const void* __restrict__ P, const T* __restrict__ fine, T* __restrict__ coarse,
                            AggGeom ag, int nrhs) {
   __shared__ T red[32 * 16];
   __shared__ T fin[16];
@@ -611,7 +619,14 @@ void restrict_any(const void* P, const T* fine, T* coarse, const AggGeom& ag, in
     if (nrhs > 1 && ag.agg[3] >= 4) return restrict_l<S>(P, fine, coarse, ag, nrhs, st);
   }
   const int threads = (ag.asites + 31) / 32 * 32;
-  k_restrict<T, S><<<(unsigned)ag.gc.V * (unsigned)nrhs, threads, 0, st>>>(P, fine, coarse, ag, nrhs);
+  const unsigned grid = (unsigned)ag.gc.V * (unsigned)nrhs;
+  if constexpr (sizeof(T) == 8) {
+    if (threads <= 512) {
+      k_restrict<T, S, 512><<<grid, threads, 0, st>>>(P, fine, coarse, ag, nrhs);
+      return;
+    }
+  }
+  k_restrict<T, S, 1024><<<grid, threads, 0, st>>>(P, fine, coarse, ag, nrhs);
 }
 
 template <typename T>

@@ -45,3 +45,23 @@ def test_transfer_batches(L, agg, nv, nrhs, prec, tol):
         want = P.prolong(c[r])
         assert rel(new[r], want) <= tol
         assert rel(acc[r], psi[r] + want) <= tol
+
+
+@pytest.mark.parametrize("nrhs", [1, 2])
+def test_fp64_transfers_of_the_largest_aggregates(nrhs):
+    # 1024 sites, one thread each: orthonormalisation and restriction have 64 registers there
+    L, agg, nv = (8, 8, 16, 16), (4, 4, 8, 8), 3
+    g = GPU(inputs.gauge_field(L, 0.3, 3), m0=0.1, c_sw=1.0, mu=0.1, nv=nv, agg=agg, sap_block=(2, 2, 2, 2),
+            cycle_prec=tm.TM_F64, max_rhs=nrhs)
+    tv = inputs.random_test_vectors(L, nv, 4)
+    tm.tm_setup_from_vectors(g.h, tv)
+    P = Interpolation(tv, agg)
+    psi, c = inputs.gaussian_spinor(L, 5, nrhs), inputs.random_coarse_vectors(g.Lc, 2 * nv, nrhs, 6)
+    psi, c = psi.reshape((nrhs,) + L + (4, 3)), c.reshape(g.coarse_shape(nrhs))
+    fc, ff = g.field(1, tm.TM_F64, nrhs), g.field(0, tm.TM_F64, nrhs)
+    tm.tm_restrict(g.h, tm.TM_F64, g.pack(0, tm.TM_F64, psi, nrhs), fc, nrhs)
+    tm.tm_prolong(g.h, tm.TM_F64, g.pack(1, tm.TM_F64, c, nrhs), ff, nrhs, 0)
+    got, up = g.unpack(1, tm.TM_F64, fc, c.shape, nrhs), g.unpack(0, tm.TM_F64, ff, psi.shape, nrhs)
+    for r in range(nrhs):
+        assert rel(got[r], P.restrict(psi[r])) <= 1e-12
+        assert rel(up[r], P.prolong(c[r])) <= 1e-12
