@@ -43,7 +43,6 @@ namespace cg = cooperative_groups;
 
 constexpr int kCl = 8;            // CTAs per cluster
 constexpr int kClThreads = 512;
-constexpr int kClMaxRestart = 48;  // Hessenberg matrix in shared memory
 // bytes read per step up to which eight SMs are faster than the chip with its dearer barriers
 constexpr long kClMaxBytes = 6L << 20;
 constexpr size_t kClSmem = 200 * 1024;
@@ -623,7 +622,7 @@ bool stream_sms(cudaStream_t st, int* sms, int* together) {
 
 bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes, cudaStream_t st) {
   const int q = (oe.nhalf + kCl - 1) / kCl;
-  if (restart > kClMaxRestart || step_bytes(oe, real_bytes) > kClMaxBytes || nrhs * kCl > 152 ||
+  if (restart > kCoarseOneLaunchSteps || step_bytes(oe, real_bytes) > kClMaxBytes || nrhs * kCl > 152 ||
       cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total > kClSmem)
     return false;
   int sms = 0, together = 0;
@@ -634,7 +633,7 @@ bool coarse_grid_fits(const OEGeom& oe, int restart, size_t real_bytes, cudaStre
   int sms = 0, together = 0;
   if (!stream_sms(st, &sms, &together) || sms < kGridCtas) return false;  // all CTAs have to be resident
   const int q = (oe.nhalf + kGridCtas - 1) / kGridCtas;
-  return restart <= kClMaxRestart && cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total <= kClSmem;
+  return restart <= kCoarseOneLaunchSteps && cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total <= kClSmem;
 }
 long coarse_grid_scratch_doubles(int restart) { return 3L * kGridCtas * 2 * (restart + 1) + 1; }
 

@@ -2059,6 +2059,9 @@ MemPlan memory_plan(const tm_params* p, int nrhs) {
     P += nh * 17 * kp * mp * 4 * (p->coarse_mma == 3 ? 2 : 1) + nh * 17 * 4;
   }
   P += (double)kScratchBlocks * kMaxDots * 2 * 8 + kSmall * 8;
+  // partial sums of the whole-chip coarse solve of one right-hand side
+  for (int m1 : {p->coarse_restart, p->coarsest_steps})
+    if (m1 >= 1 && m1 <= kCoarseOneLaunchSteps) P += coarse_grid_scratch_doubles(m1) * 8.0;
   // work of one K-cycle over r right-hand sides
   auto kcycle_work = [&](double r) {
     double w = (p->pre_smooth > 0 ? fr * r * cs : 0) + 2 * (2 * Vc * n) * r * cs;  // k_r, k_rc, k_ec

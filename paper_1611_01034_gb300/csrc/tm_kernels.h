@@ -225,6 +225,7 @@ void launch_tc_schur(const TcGeom& tg, const OEGeom& oe, const float* ve, float*
                      cudaStream_t st, unsigned spin = 0);
 
 // ---- one-launch coarse solve (coarse_cluster.cu) --------------------------------
+constexpr int kCoarseOneLaunchSteps = 48;  // longest cycle: the Hessenberg matrix is in shared memory
 // whether the odd-even system is small enough for a cluster per right-hand side, on this stream's SMs
 bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes, cudaStream_t st);
 // GMRES(restart) on the odd-even Schur complement, from zero, to tol or maxit steps, and x_o from

@@ -145,5 +145,8 @@ def test_workspace_bytes_plan(lib):
     # a 16-bit copy of P: nv fine fields of 4 bytes per complex number
     b16 = tm.tm_workspace_bytes(tm.params(**dict(kw, transfer_prec=tm.TM_BF16)), 4)
     assert b16 - b4 == 24 * 96 * 48 ** 3 * 12 * 4
+    # cycles of up to 48 coarse steps keep the partial sums of the whole-chip solve (152 CTAs, three sums)
+    p48, p49, p50 = (tm.tm_workspace_bytes(tm.params(**dict(kw, coarse_restart=m)), 4) for m in (48, 49, 50))
+    assert (p50 - p49) - (p49 - p48) == (3 * 152 * 2 * 49 + 1) * 8
     assert tm.tm_workspace_bytes(tm.params(**dict(kw, nv=40)), 1) == 0
     assert tm.tm_workspace_bytes(p, 0) == 0
