@@ -18,7 +18,7 @@ __global__ void k_convert(const Ti* __restrict__ in, To* __restrict__ out, long 
 
 static inline int grid_for(long n, int threads = 256) {
   long b = (n + threads - 1) / threads;
-  if (b > 152L * 16) b = 152L * 16;
+  if (b > 16L * kSms) b = 16L * kSms;
   if (b < 1) b = 1;
   return (int)b;
 }

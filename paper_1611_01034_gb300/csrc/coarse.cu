@@ -416,9 +416,6 @@ __device__ __forceinline__ void ld_phalf(const void* __restrict__ P, int i, int 
 }
 
 constexpr int kTrSites = 128;    // sites per CTA of the prolongation
-#ifndef TRC
-#define TRC 4
-#endif
 constexpr int kTrThreads = 256;  // of the restriction
 constexpr int kTrPairs = 12;     // pairs per CTA of the restriction
 
@@ -686,7 +683,7 @@ __global__ void k_to16(const float2* __restrict__ in, unsigned* __restrict__ out
 
 void launch_to16(const float* in, void* out, long n_cx, int kind, cudaStream_t st) {
   long b = (n_cx + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
+  if (b > 16 * kSms) b = 16 * kSms;
   if (kind == ST_F16)
     k_to16<ST_F16><<<(int)b, 256, 0, st>>>(reinterpret_cast<const float2*>(in), static_cast<unsigned*>(out), n_cx);
   else
@@ -1060,7 +1057,7 @@ __global__ void k_count_mismatch(const unsigned* __restrict__ a, const unsigned*
 
 void launch_count_mismatch(const void* a, const void* b, long words, unsigned long long* count, cudaStream_t st) {
   long blocks = (words + 255) / 256;
-  if (blocks > 152L * 8) blocks = 152L * 8;
+  if (blocks > 8L * kSms) blocks = 8L * kSms;
   if (blocks < 1) blocks = 1;
   k_count_mismatch<<<(unsigned)blocks, 256, 0, st>>>(static_cast<const unsigned*>(a), static_cast<const unsigned*>(b),
                                                      words, count);

@@ -24,7 +24,8 @@
 // kept as one matrix instead of applied one after another, the norm from the second
 // projection's sums by Pythagoras) and put beside other work: the Hessenberg column is
 // turned while one warp takes the norm, the next rotation is made while the others write
-// the basis vector.  FP32, 24 steps from zero, us per step (MB read per step):
+// the basis vector.  FP32, 24 steps from zero, us per step of the whole call with its launch,
+// reduced right-hand side, odd sites and wait (at 0.3 MB 11.5 of the 13.6 are the step itself):
 //
 //   MB            0.3   2.4   5.3   7.2   7.4   29    59    85   118   231   340
 //   host-driven    54    57    63    63    63    69    69    75   120   150   215
@@ -46,7 +47,7 @@ constexpr int kClThreads = 512;
 // bytes read per step up to which eight SMs are faster than the chip with its dearer barriers
 constexpr long kClMaxBytes = 6L << 20;
 constexpr size_t kClSmem = 200 * 1024;
-constexpr int kGridCtas = 152;          // of the whole-chip form, one per SM
+constexpr int kGridCtas = kSms;         // of the whole-chip form, one per SM
 constexpr unsigned kGridPolls = 1u << 22;   // of one barrier before a CTA gives up, unless the caller sets it
 
 struct ClLayout {  // shared memory, in bytes from its start
@@ -622,7 +623,7 @@ bool stream_sms(cudaStream_t st, int* sms, int* together) {
 
 bool coarse_cluster_fits(const OEGeom& oe, int restart, int nrhs, size_t real_bytes, cudaStream_t st) {
   const int q = (oe.nhalf + kCl - 1) / kCl;
-  if (restart > kCoarseOneLaunchSteps || step_bytes(oe, real_bytes) > kClMaxBytes || nrhs * kCl > 152 ||
+  if (restart > kCoarseOneLaunchSteps || step_bytes(oe, real_bytes) > kClMaxBytes || nrhs * kCl > kSms ||
       cl_layout(restart, q, 2 * oe.nv, 2 * real_bytes).total > kClSmem)
     return false;
   int sms = 0, together = 0;

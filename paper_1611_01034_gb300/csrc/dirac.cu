@@ -91,7 +91,7 @@ void launch_zero_parity_nat(double* nat, const Lat& g, int parity, int nrhs, cud
 
 void launch_gamma5_nat(const double* in, double* out, long nsites, cudaStream_t st) {
   long blocks = (nsites * 24 + 255) / 256;
-  if (blocks > 152L * 16) blocks = 152L * 16;
+  if (blocks > 16L * kSms) blocks = 16L * kSms;
   k_gamma5_nat<<<(int)blocks, 256, 0, st>>>(in, out, nsites);
 }
 
@@ -395,7 +395,7 @@ void launch_dslash(const T* gauge, const T* clover, const T* in, T* out, const T
     // two right-hand sides per thread where that still fills the chip with four CTAs per SM: 309 against
     // 340 us at 48 x 24^3 and 11.1 against 12.3 us at 16^3 x 8, six right-hand sides, but 8.3 against
     // 6.3 us for two there; an odd count in one launch (three at 48 x 24^3: 183 us; two and one: 202 us)
-    if (nrhs % 2 == 0 && (long)((g.V + 127) / 128) * (nrhs / 2) >= 4 * 152)
+    if (nrhs % 2 == 0 && (long)((g.V + 127) / 128) * (nrhs / 2) >= 4 * kSms)
       dslash_r<T, 2, 4>(a, st);
     else
       dslash_r<T, 1, 4>(a, st);

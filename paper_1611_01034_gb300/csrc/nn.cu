@@ -373,7 +373,7 @@ __global__ void k_wgrad_reduce(const double2* __restrict__ partial, int ncta, do
   if (threadIdx.x == 0) out[e] = make_double2(red[0], red[128]);
 }
 
-constexpr int kGCtas = 2 * 152;
+constexpr int kGCtas = 2 * kSms;
 
 template <bool FIRST>
 void run_wgrad(const float* hid, const float* one, const float* gauge, const Lat& g, double bc, int nrhs,

@@ -188,7 +188,7 @@ __global__ void k_acc_f32(const float* __restrict__ e, double* __restrict__ x, l
 
 int stream_grid(long n) {
   long b = (n + 255) / 256;
-  if (b > 152L * 8) b = 152L * 8;
+  if (b > 8L * kSms) b = 8L * kSms;
   return (int)(b < 1 ? 1 : b);
 }
 

@@ -223,7 +223,7 @@ __device__ __forceinline__ f2 mr_ratio(f2 n, f2 d) {
 // chip: the block's links in shared memory (48 KB), the site's clover blocks and e,
 // which only their own thread reads, in tensor memory (96 columns per warp), r in
 // shared memory.  The general kernel reads links and clover from L1 and L2 in every
-// step and waits for them: four sweeps, one right-hand side, 32 x 16^3, 335 -> 285
+// step and waits for them: four sweeps, one right-hand side, 32 x 16^3, 342 -> 291
 // us; 8^4 218 -> 169 us; three sweeps of 7 at 24^2 x 16^2 1.63 -> 1.37 ms.  Measured
 // and left out: two right-hand sides per thread as packed lanes, as in the odd-even
 // form (4 right-hand sides 878 -> 900 us: eight warps per SM wait longer); e alone
@@ -1392,8 +1392,8 @@ template void launch_sap_oe_colour<double>(const void*, const void*, const void*
 template void launch_sap_oe_colour<float>(const void*, const void*, const void*, const float*, float*,
                                           const SapGeom&, double, double, int, int, int, cudaStream_t, double, int);
 
-// 16-bit copy in block order of a chunked FP32 field: `planes` chunk planes of n
-// sites, all V of them (PAR = 0) or the V / 2 odd ones by their index s >> 1
+// 16-bit copy in block order of a chunked FP32 field, a chunk plane of n sites per
+// blockIdx.y: all V sites, or the V / 2 odd ones by their index s >> 1
 template <int KIND>
 __global__ void k_to16_blocks(const float4* __restrict__ in, uint2* __restrict__ out, SapGeom sg, int n) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
