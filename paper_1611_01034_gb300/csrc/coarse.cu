@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(MT, 1) k_orthonormalise(T* P, AggGeom ag, int*
 // columns (each twice per pass) and by the shuffles of the reductions; a panel
 // shares both: 16 inner products per four columns loaded, one reduce-scatter of 32
 // sums, the update from the registers just used (N_v 20, FP32, 32 x 16^3, 4^4
-// aggregates: 1.11 -> 0.44 ms).
+// aggregates: 1.11 -> 0.44 ms).  take_off and one
+// scaling, at the end, keep few roundings at the size of a column.
 constexpr int kPanel = 4;
 
 // NC complex numbers of a field that the kernel writes as well (ordinary loads)
@@ -127,9 +128,11 @@ __device__ __forceinline__ void ld_cx_rw(const T* base, long V, long s, cx<T> (&
   ld_lanes_rw<T, NC, T>(base, base, V, s, z);
 }
 
-// sums over the CTA of 32 values per thread; fin[k] = sum k for every thread after the call
+// sums over the CTA of 32 values per thread; fin[k] = sum k for every thread after the call.  They are
+// the projections of a panel's columns, (re, im) of column p at 8 i + 2 p; *few: all are small against
+// the columns, whose squared norms are n0
 template <typename T>
-__device__ __forceinline__ void cta_sum32(T (&v)[32], T* red, T* fin) {
+__device__ __forceinline__ void cta_sum32(T (&v)[32], T* red, T* fin, const T* n0, bool* few) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -143,10 +146,16 @@ __device__ __forceinline__ void cta_sum32(T (&v)[32], T* red, T* fin) {
     T sum = 0;
     for (int w = 0; w < nw; ++w) sum += red[w * 32 + threadIdx.x];
     fin[threadIdx.x] = sum;
+    T size = sum * sum;
+    size += __shfl_xor_sync(0xffffffffu, size, 1);
+    size += __shfl_xor_sync(0xffffffffu, size, 8);
+    size += __shfl_xor_sync(0xffffffffu, size, 16);
+    const bool all = __all_sync(0xffffffffu, 16 * size <= n0[(threadIdx.x >> 1) & 3]);
+    if (threadIdx.x == 0) *few = all;
   }
   __syncthreads();
 }
-// the same for N <= 8 values, every thread left with the sums
+// sums as above of N <= 8 values, every thread left with the sums
 template <typename T, int N>
 __device__ __forceinline__ void cta_sum(T (&v)[N], T* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -166,10 +175,33 @@ __device__ __forceinline__ void cta_sum(T (&v)[N], T* red) {
   __syncthreads();
 }
 
+// v -= sum of N columns q times m.  Small against v the sum is formed first and rounds once at the size of v;
+// a large one is taken off term by term, so that no product is rounded and all but the first rounding are at the
+// size of what is left.
+template <typename T, int N>
+__device__ __forceinline__ void take_off(cx<T> (&v)[6], const cx<T> (&m)[kPanel], const cx<T> (&q)[kPanel][6], bool few) {
+  if (few) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      cx<T> sum = m[0] * q[0][k];
+#pragma unroll
+      for (int i = 1; i < N; ++i) cfma(sum, m[i], q[i][k]);
+      v[k] = v[k] - sum;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) cfma(v[k], -m[i], q[i][k]);
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_orthonormalise_p(T* P, AggGeom ag, int* err) {
   __shared__ T red[8 * 32];
   __shared__ T fin[32];
+  __shared__ bool few;
+  __shared__ T n0[kPanel], inv[kPanel];  // squared norms of the given columns; one over the norms of v
   const int a = blockIdx.x >> 1, chi = blockIdx.x & 1, nv = ag.nv;
   const int l = threadIdx.x;
   const bool act = l < ag.asites;
@@ -181,7 +213,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_orthonormalise_
   const T rank_tol = sizeof(T) == 8 ? T(1e-24) : T(1e-10);
   for (int j0 = 0; j0 < nv; j0 += kPanel) {
     cx<T> v[kPanel][6];
-    T n0[kPanel];
+    T sq[kPanel];
 #pragma unroll
     for (int p = 0; p < kPanel; ++p) {
       if (act && j0 + p < nv) {
@@ -190,11 +222,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_orthonormalise_
 #pragma unroll
         for (int k = 0; k < 6; ++k) v[p][k] = cx<T>{0, 0};
       }
-      n0[p] = 0;
+      sq[p] = 0;
 #pragma unroll
-      for (int k = 0; k < 6; ++k) n0[p] += norm2(v[p][k]);
+      for (int k = 0; k < 6; ++k) sq[p] += norm2(v[p][k]);
     }
-    cta_sum<T, kPanel>(n0, red);
+    cta_sum<T, kPanel>(sq, red);
+    if (l == 0) {  // read after the barriers of the next sums
+#pragma unroll
+      for (int p = 0; p < kPanel; ++p) n0[p] = sq[p];
+    }
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
       // against the finished columns, four at a time
@@ -219,15 +255,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_orthonormalise_
             d[8 * ii + 2 * p + 1] = acc.i;
           }
         }
-        cta_sum32(d, red, fin);
+        cta_sum32(d, red, fin, n0, &few);
 #pragma unroll
-        for (int ii = 0; ii < kPanel; ++ii)
+        for (int p = 0; p < kPanel; ++p) {
+          cx<T> m[kPanel];
 #pragma unroll
-          for (int p = 0; p < kPanel; ++p) {
-            const cx<T> m{-fin[8 * ii + 2 * p], -fin[8 * ii + 2 * p + 1]};
-#pragma unroll
-            for (int k = 0; k < 6; ++k) cfma(v[p][k], m, q[ii][k]);
-          }
+          for (int ii = 0; ii < kPanel; ++ii) m[ii] = cx<T>{fin[8 * ii + 2 * p], fin[8 * ii + 2 * p + 1]};
+          take_off<T, kPanel>(v[p], m, q, few);
+        }
       }
       // within the panel
 #pragma unroll
@@ -245,30 +280,37 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_orthonormalise_
             d[2 * pp + 1] = acc.i;
           }
           cta_sum<T, 2 * kPanel>(d, red);
+          cx<T> m[kPanel];
+          T size = 0;
 #pragma unroll
           for (int pp = 0; pp < p; ++pp) {
-            const cx<T> m{-d[2 * pp], -d[2 * pp + 1]};
-#pragma unroll
-            for (int k = 0; k < 6; ++k) cfma(v[p][k], m, v[pp][k]);
+            m[pp] = cx<T>{d[2 * pp] * inv[pp], d[2 * pp + 1] * inv[pp]};
+            size += norm2(m[pp]);
+            m[pp] = inv[pp] * m[pp];
           }
+          if (p == 1) take_off<T, 1>(v[p], m, v, 16 * size <= n0[p]);
+          if (p == 2) take_off<T, 2>(v[p], m, v, 16 * size <= n0[p]);
+          if (p == 3) take_off<T, 3>(v[p], m, v, 16 * size <= n0[p]);
         }
         T nn[1] = {0};
 #pragma unroll
         for (int k = 0; k < 6; ++k) nn[0] += norm2(v[p][k]);
         cta_sum<T, 1>(nn, red);
-        const T least = pass == 0 ? rank_tol * n0[p] : T(0);  // what the first pass left of the column
-        if (j0 + p < nv && (!(nn[0] > least) || !(nn[0] > T(0)))) {
+        if (pass == 1 && j0 + p < nv && (!(nn[0] > rank_tol * n0[p]) || !(nn[0] > T(0)))) {
           if (l == 0) atomicOr(err, ERRF_RANK);
           nn[0] = T(1);
         }
-        const T inv = j0 + p < nv ? T(1) / sqrt(nn[0]) : T(0);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[p][k] = inv * v[p][k];
+        if (l == 0) inv[p] = nn[0] > T(0) ? T(1) / sqrt(nn[0]) : T(0);
       }
     }
+    __syncthreads();
 #pragma unroll
     for (int p = 0; p < kPanel; ++p)
-      if (act && j0 + p < nv) st_cx<T, 6>(Pc + (j0 + p) * fstride, V, s, v[p]);
+      if (act && j0 + p < nv) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[p][k] = inv[p] * v[p][k];
+        st_cx<T, 6>(Pc + (j0 + p) * fstride, V, s, v[p]);
+      }
   }
 }
 

@@ -3,6 +3,7 @@
 Every right-hand side against the oracle's P: one alone, whole pairs, an odd one out, and more pairs than
 one CTA takes; aggregates below a warp, of one CTA and beyond one CTA; N_v that leaves columns over.
 FP32 sums of at most 6144 terms: 1e-5; a 16-bit P rounds every entry by 2^-11 (FP16) or 2^-8 (BF16).
+And the FP32 error of P itself.
 """
 import numpy as np
 import pytest
@@ -65,3 +66,21 @@ def test_fp64_transfers_of_the_largest_aggregates(nrhs):
     for r in range(nrhs):
         assert rel(got[r], P.restrict(psi[r])) <= 1e-12
         assert rel(up[r], P.prolong(c[r])) <= 1e-12
+
+
+@pytest.mark.parametrize("agg", [(4, 4, 4, 4), (2, 2, 2, 2)])
+@pytest.mark.parametrize("nv", [11, 24])
+@pytest.mark.parametrize("common", [0, 10])
+def test_fp32_error_of_the_orthonormalisation(agg, nv, common):
+    # Gram-Schmidt rounds a column once per finished column and pass (nv on average) and once when it is scaled, each
+    # time by 2.5e-8 of its size (the root mean square of FP32); a common part of the vectors ten times the rest
+    # leaves roundings of ten times that size.  The vectors are exact in FP32.
+    L = (8, 8, 8, 8)
+    U, tv = inputs.gauge_field(L, 0.3, 3), inputs.random_test_vectors(L, nv, 4)
+    tv = (tv + common * inputs.random_test_vectors(L, 1, 5)).astype(np.complex64).astype(np.complex128)
+    P = []
+    for prec in (tm.TM_F32, tm.TM_F64):
+        g = GPU(U, m0=0.1, c_sw=1.0, mu=0.1, nv=nv, agg=agg, sap_block=(2, 2, 2, 2), cycle_prec=prec)
+        tm.tm_setup_from_vectors(g.h, tv)
+        P.append(g.P_columns())
+    assert rel(P[0], P[1]) <= 2.5e-8 * (10 if common else (1 + nv) ** 0.5)
