@@ -458,11 +458,11 @@ __device__ __forceinline__ void ld_phalf(const void* __restrict__ P, int i, int 
 }
 
 constexpr int kTrSites = 128;    // sites per CTA of the prolongation
-constexpr int kTrThreads = 256;  // of the restriction
-constexpr int kTrPairs = 12;     // pairs per CTA of the restriction
+constexpr int kTrThreads = 512;  // of the restriction
+constexpr int kTrWarpPairs = 96; // warps times pairs of one of its CTAs (sums in shared memory)
 
-// Restriction: CTA = one aggregate, one chirality and up to kTrPairs pairs;
-// thread = site.  Four columns at a time, pair after pair: 16 sums per thread, reduced over the warp by a reduce-scatter
+// Restriction: CTA = one aggregate, one chirality and ppc pairs; thread = site
+// (two of them beyond 512).  Four columns at a time, pair after pair: 16 sums per thread, reduced over the warp by a reduce-scatter
 // that leaves each lane one of them; the warps' sums meet in shared memory at the
 // end.  Bound by the latency of the P loads (from L1 and L2 for all pairs but the
 // first), so the batch of columns is what 64 registers (32 warps per SM) hold: 6
@@ -470,14 +470,14 @@ constexpr int kTrPairs = 12;     // pairs per CTA of the restriction
 // registers 574 us, 128 registers 650 us; the fine vectors staged in shared memory
 // and P read once for three pairs, 168 registers, 570 us.
 template <int S>
-__global__ void __launch_bounds__(kTrThreads, 4) k_restrict_l(const void* __restrict__ P, const float* __restrict__ fine,
+__global__ void __launch_bounds__(kTrThreads, 2) k_restrict_l(const void* __restrict__ P, const float* __restrict__ fine,
                                                              float* __restrict__ coarse, AggGeom ag, int nrhs,
-                                                             int ngrp) {
+                                                             int ngrp, int ppc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* red = reinterpret_cast<float*>(smem_raw);  // [ceil(nv / C)][pairs][warps][16]
   const int h = blockIdx.x & 1, a = (blockIdx.x >> 1) / ngrp;
   constexpr int C = 4;  // columns at a time
-  const int p0 = ((blockIdx.x >> 1) % ngrp) * kTrPairs, pairs = min(kTrPairs, (nrhs + 1) / 2 - p0);
+  const int p0 = ((blockIdx.x >> 1) % ngrp) * ppc, pairs = min(ppc, (nrhs + 1) / 2 - p0);
   const int nv = ag.nv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const long V = ag.g.V, fs = (long)NR_SPINOR * V;
   int lc[4], c[4];
@@ -613,12 +613,40 @@ static int transfer_pairs(int nrhs, int* ngrp) {
   return (pairs + *ngrp - 1) / *ngrp;
 }
 
+static int restrict_threads(int asites) { return std::min(kTrThreads, (asites + 31) / 32 * 32); }
+
+// Pairs per CTA of an FP32 restriction, 0 where one right-hand side per CTA is faster.  Pairs win by reading a P that
+// comes from DRAM once, and by sharing its conversion; they lose a lane to an odd count, and with a P that stays in L2
+// that costs more.  So pairs from 75 MB of P on (100 MB beyond 256 sites, where a CTA takes half the SM), from 48 MB
+// for five and more, below that for even counts.  Us, one per CTA against pairs, N_v 24, 4^4 aggregates: 75 MB (16^4,
+// FP16) 2 right-hand sides 30 27, 3 56 47, 6 86 70; 151 MB (16^4, FP32) 43 32, 74 49, 104 68; 28 MB (24 x 16 x 24 x 8,
+// N_v 8, FP16) 12.4 12.5, 3 16.5 18.7, 6 26.6 26.5; 5 MB (8^4, FP16) 6 14.6 14.6.  Over 1296 such pairs of times
+// (aggregates of 32 to 1024 sites, N_v 8 to 24, 2 to 12 right-hand sides) pairs, where they are taken, are at most 1.11
+// times slower.  Aggregates of two sites in X (half-empty warps) and one right-hand side keep the other form.
+// Then the fewest CTAs per aggregate that give every SM 24 warps: one for all pairs reads P once, but leaves a small
+// lattice's SMs idle (8 right-hand sides, N_v 24, FP32 P: 8^4 49 -> 14.5 us, 16 x 8^2 x 16 49 -> 25 us).
+extern "C" int tmamg_restrict_pairs(const int* L, const int* agg, int nv, int nrhs, int real_bytes) {
+  const long V = (long)L[0] * L[1] * L[2] * L[3], asites = (long)agg[0] * agg[1] * agg[2] * agg[3];
+  const double mb = 1e-6 * nv * V * NR_SPINOR * real_bytes;
+  const bool small = asites <= 256;
+  if (nrhs < 2 || agg[3] < 4 || !(mb >= (small ? 75 : 100) || (small && (nrhs % 2 == 0 || (nrhs >= 5 && mb >= 48)))))
+    return 0;
+  const int pairs = (nrhs + 1) / 2, warps = restrict_threads((int)asites) / 32;
+  int ppc = pairs, ngrp = 1;
+  while (ppc > 1 && (ppc * warps > kTrWarpPairs || V / asites * 2 * ngrp * warps < 24 * kSms)) {
+    --ppc;
+    ngrp = (pairs + ppc - 1) / ppc;
+    ppc = (pairs + ngrp - 1) / ngrp;
+  }
+  return ppc;
+}
+
 template <int S>
-void restrict_l(const void* P, const float* fine, float* coarse, const AggGeom& ag, int nrhs, cudaStream_t st) {
-  const int pairs = (nrhs + 1) / 2, ngrp = (pairs + kTrPairs - 1) / kTrPairs;
-  const int threads = std::min(kTrThreads, (ag.asites + 31) / 32 * 32);
-  const size_t smem = (size_t)((ag.nv + 3) / 4) * std::min(pairs, kTrPairs) * (threads / 32) * 16 * sizeof(float);
-  k_restrict_l<S><<<(unsigned)ag.gc.V * (unsigned)ngrp * 2u, threads, smem, st>>>(P, fine, coarse, ag, nrhs, ngrp);
+void restrict_l(const void* P, const float* fine, float* coarse, const AggGeom& ag, int nrhs, int ppc,
+                cudaStream_t st) {
+  const int threads = restrict_threads(ag.asites), ngrp = ((nrhs + 1) / 2 + ppc - 1) / ppc;
+  const size_t smem = (size_t)((ag.nv + 3) / 4) * ppc * (threads / 32) * 16 * sizeof(float);
+  k_restrict_l<S><<<(unsigned)ag.gc.V * (unsigned)ngrp * 2u, threads, smem, st>>>(P, fine, coarse, ag, nrhs, ngrp, ppc);
 }
 
 template <int S, int PR>
@@ -652,10 +680,8 @@ void prolong_s(const void* P, const float* coarse, float* fine, const AggGeom& a
 template <typename T, int S>
 void restrict_any(const void* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value) {
-    // pairs beat one right-hand side per CTA from two on (6: 540 against 716 us); one
-    // alone is 1 to 9 % faster in the form that keeps both chiralities in a thread,
-    // as are half-empty warps (2^4 aggregates, 3 right-hand sides: 146 and 150 us)
-    if (nrhs > 1 && ag.agg[3] >= 4) return restrict_l<S>(P, fine, coarse, ag, nrhs, st);
+    const int ppc = tmamg_restrict_pairs(ag.g.L, ag.agg, ag.nv, nrhs, S == ST_NATIVE ? 4 : 2);
+    if (ppc > 0) return restrict_l<S>(P, fine, coarse, ag, nrhs, ppc, st);
   }
   const int threads = (ag.asites + 31) / 32 * 32;
   const unsigned grid = (unsigned)ag.gc.V * (unsigned)nrhs;

@@ -96,6 +96,8 @@ struct AggGeom {
 // P <- per (aggregate, chirality) CGS2 orthonormalisation of the Nv fields in P (in place)
 template <typename T>
 void launch_orthonormalise(T* P, const AggGeom& ag, int* err, cudaStream_t st);
+// pairs of right-hand sides per CTA of an FP32 restriction (P of real_bytes per real), 0: none
+extern "C" int tmamg_restrict_pairs(const int* L, const int* agg, int nv, int nrhs, int real_bytes);
 // coarse[rhs][Vc][2Nv] = P^dagger fine
 template <typename T>
 void launch_restrict(const T* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st,

@@ -1,4 +1,4 @@
-"""FP32 restriction and prolongation of batches (pairs of right-hand sides share a thread).
+"""FP32 restriction and prolongation of batches (on many sizes pairs of right-hand sides share a thread).
 
 Every right-hand side against the oracle's P: one alone, whole pairs, an odd one out, and more pairs than
 one CTA takes; aggregates below a warp, of one CTA and beyond one CTA; N_v that leaves columns over.
@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 from tests.gpu_helpers import GPU, rel  # noqa: E402
+from tests.test_transfer_pairs import restrict_pairs  # noqa: E402
 
 F32 = tm.TM_F32
 
@@ -46,6 +47,26 @@ def test_transfer_batches(L, agg, nv, nrhs, prec, tol):
         want = P.prolong(c[r])
         assert rel(new[r], want) <= tol
         assert rel(acc[r], psi[r] + want) <= tol
+
+
+# restriction in pairs: one CTA for all of them or several, an odd one out, aggregates below a warp's CTA and beyond
+# one CTA, and enough pairs to be split by shared memory
+@pytest.mark.parametrize("L,agg,nv,nrhs,prec,pairs", [
+    ((8, 8, 8, 8), (4, 4, 4, 4), 9, 6, tm.TM_BF16, 1), ((16, 16, 16, 16), (4, 4, 4, 4), 8, 5, tm.TM_F32, 3),
+    ((16, 16, 16, 16), (4, 4, 4, 4), 25, 3, tm.TM_F16, 2), ((16, 16, 16, 16), (4, 4, 4, 4), 6, 26, tm.TM_F32, 7),
+    ((4, 4, 8, 32), (2, 2, 2, 4), 7, 4, tm.TM_F32, 1), ((16, 16, 16, 32), (4, 4, 8, 8), 9, 4, tm.TM_F32, 2)])
+def test_restriction_of_pairs(L, agg, nv, nrhs, prec, pairs):
+    assert restrict_pairs(L, agg, nv, nrhs, prec) == pairs
+    g = GPU(inputs.gauge_field(L, 0.3, 3), m0=0.1, c_sw=1.0, mu=0.1, nv=nv, agg=agg, sap_block=(2, 2, 2, 2),
+            cycle_prec=F32, max_rhs=nrhs, transfer_prec=prec)
+    tm.tm_setup_from_vectors(g.h, inputs.random_test_vectors(L, nv, 4))
+    psi = inputs.gaussian_spinor(L, 5, nrhs)
+    fc, f1 = g.field(1, F32, nrhs), g.field(1, F32, 1)
+    tm.tm_restrict(g.h, F32, g.pack(0, F32, psi, nrhs), fc, nrhs)
+    got = g.unpack(1, F32, fc, g.coarse_shape(nrhs), nrhs)
+    for r in range(nrhs):  # FP32 sums of at most 12288 terms in another order
+        tm.tm_restrict(g.h, F32, g.pack(0, F32, psi[r]), f1, 1)
+        assert rel(got[r], g.unpack(1, F32, f1, got[r].shape)) <= 1e-6
 
 
 @pytest.mark.parametrize("nrhs", [1, 2])
