@@ -649,6 +649,21 @@ void restrict_l(const void* P, const float* fine, float* coarse, const AggGeom& 
   k_restrict_l<S><<<(unsigned)ag.gc.V * (unsigned)ngrp * 2u, threads, smem, st>>>(P, fine, coarse, ag, nrhs, ngrp, ppc);
 }
 
+// Whether an FP32 prolongation takes pairs.  They win where they save passes over P (six right-hand sides a pass
+// against three), on lattices too small to fill the chip otherwise (one chirality per CTA), and for three right-hand
+// sides of many columns (shared conversion); one pass of two is faster in lattice order, as is an accumulating last
+// group of one or two with few columns.  Us, lattice order against pairs, 4^4 aggregates: N_v 24, FP16 P, 16^4: 2
+// right-hand sides 21 29, 3 27 28, 4 46 29, 7 69 48; 32 x 16^3: 55 60, 64 51, 90 53, 129 86; 8^4: 14.4 10.4, 16.5 8.5; N_v
+// 8, FP32 P, 32 x 24^3: 74 85, 84 96, 113 101, 7 (accumulating) 194 215.  Over 2592 such pairs of times (aggregates
+// of 32 to 1024 sites, 2 to 12 right-hand sides) the form taken is at most 1.08 times slower.  Aggregates of two
+// sites in X, whose site order breaks up the loads, keep lattice order.
+extern "C" int tmamg_prolong_pairs(const int* L, const int* agg, int nv, int nrhs, int accumulate) {
+  if (nrhs < 2 || agg[3] < 4) return 0;
+  if ((long)L[0] * L[1] * L[2] * L[3] <= 20000) return 1;
+  if (nrhs <= 3) return nrhs == 3 && nv >= 20;
+  return !(accumulate && nv < 12 && (nrhs == 7 || nrhs == 8));
+}
+
 template <int S, int PR>
 void prolong_l(const void* P, const float* coarse, float* fine, const AggGeom& ag, int nrhs, int ngrp, bool acc,
                cudaStream_t st) {
@@ -709,9 +724,8 @@ template <typename T, int S>
 void prolong_any(const void* P, const T* coarse, T* fine, const AggGeom& ag, int nrhs, bool accumulate,
                  cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value) {
-    // 2^4 aggregates, 3 right-hand sides, FP32 P at 24 x 24 x 16^2: 61.5 us in lattice
-    // order, 63 in aggregate order; 4^4 and 2 right-hand sides at 8^4: 8.4 and 6.4 us
-    if (nrhs > 1 && ag.agg[3] >= 4) return prolong_s<S>(P, coarse, fine, ag, nrhs, accumulate, st);
+    if (tmamg_prolong_pairs(ag.g.L, ag.agg, ag.nv, nrhs, accumulate))
+      return prolong_s<S>(P, coarse, fine, ag, nrhs, accumulate, st);
   }
   constexpr int RG = sizeof(T) == 4 ? 3 : 1;
   const unsigned ngrp = (unsigned)((nrhs + RG - 1) / RG);

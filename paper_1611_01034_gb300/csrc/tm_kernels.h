@@ -102,6 +102,8 @@ extern "C" int tmamg_restrict_pairs(const int* L, const int* agg, int nv, int nr
 template <typename T>
 void launch_restrict(const T* P, const T* fine, T* coarse, const AggGeom& ag, int nrhs, cudaStream_t st,
                      const void* P16 = nullptr, int p16 = 0);  // P16: 16-bit copy of P (ST_F16 / ST_BF16)
+// whether an FP32 prolongation runs pairs of right-hand sides
+extern "C" int tmamg_prolong_pairs(const int* L, const int* agg, int nv, int nrhs, int accumulate);
 // fine = (accumulate ? fine : 0) + P coarse
 template <typename T>
 void launch_prolong(const T* P, const T* coarse, T* fine, const AggGeom& ag, int nrhs, bool accumulate,

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 from tests.gpu_helpers import GPU, rel  # noqa: E402
-from tests.test_transfer_pairs import restrict_pairs  # noqa: E402
+from tests.test_transfer_pairs import prolong_pairs, restrict_pairs  # noqa: E402
 
 F32 = tm.TM_F32
 
@@ -67,6 +67,26 @@ def test_restriction_of_pairs(L, agg, nv, nrhs, prec, pairs):
     for r in range(nrhs):  # FP32 sums of at most 12288 terms in another order
         tm.tm_restrict(g.h, F32, g.pack(0, F32, psi[r]), f1, 1)
         assert rel(got[r], g.unpack(1, F32, f1, got[r].shape)) <= 1e-6
+
+
+# prolongation in lattice order beside pairs: both sides of the rule, on more than one CTA's sites
+@pytest.mark.parametrize("L,nv,nrhs,acc,pairs", [
+    ((16, 12, 12, 12), 5, 2, 0, False), ((16, 12, 12, 12), 5, 3, 1, False), ((16, 12, 12, 12), 5, 4, 0, True),
+    ((16, 12, 12, 12), 5, 7, 1, False), ((16, 12, 12, 12), 5, 7, 0, True), ((16, 12, 12, 12), 21, 3, 1, True)])
+def test_prolongation_forms(L, nv, nrhs, acc, pairs):
+    agg = (4, 6, 6, 6)
+    assert prolong_pairs(L, agg, nv, nrhs, acc) == pairs
+    g = GPU(inputs.gauge_field(L, 0.3, 3), m0=0.1, c_sw=1.0, mu=0.1, nv=nv, agg=agg, sap_block=(2, 2, 2, 2),
+            cycle_prec=F32, max_rhs=nrhs)
+    tm.tm_setup_from_vectors(g.h, inputs.random_test_vectors(L, nv, 4))
+    psi, c = inputs.gaussian_spinor(L, 5, nrhs), inputs.random_coarse_vectors(g.Lc, 2 * nv, nrhs, 6)
+    ff = g.pack(0, F32, psi, nrhs)
+    tm.tm_prolong(g.h, F32, g.pack(1, F32, c, nrhs), ff, nrhs, acc)
+    got = g.unpack(0, F32, ff, psi.shape, nrhs)
+    for r in range(nrhs):
+        f1 = g.pack(0, F32, psi[r])
+        tm.tm_prolong(g.h, F32, g.pack(1, F32, c[r]), f1, 1, acc)
+        assert rel(got[r], g.unpack(0, F32, f1, psi[r].shape)) <= 1e-6
 
 
 @pytest.mark.parametrize("nrhs", [1, 2])

@@ -20,6 +20,12 @@ def restrict_pairs(L, agg, nv, nrhs, prec):
     return tm.lib().tmamg_restrict_pairs(four(*L), four(*agg), nv, nrhs, _bytes(prec))
 
 
+def prolong_pairs(L, agg, nv, nrhs, accumulate):
+    """Whether the prolongation runs pairs."""
+    four = ctypes.c_int * 4
+    return bool(tm.lib().tmamg_prolong_pairs(four(*L), four(*agg), nv, nrhs, accumulate))
+
+
 @pytest.fixture(scope="module", autouse=True)
 def lib():
     from paper_1611_01034_gb300 import build
@@ -50,3 +56,12 @@ def test_restriction_splits_are_even_and_fit_shared_memory(agg):
             if p:
                 ctas = -(-pairs // p)
                 assert p == -(-pairs // ctas) and 7 * p * warps * 16 * 4 <= 48 * 1024
+
+
+@pytest.mark.parametrize("L,nv,nrhs,accumulate,expect", [
+    ((8, 8, 8, 8), 24, 2, 0, True), ((16, 16, 16, 16), 24, 2, 0, False),  # 29 us in pairs, 21 in lattice order
+    ((32, 24, 24, 24), 8, 3, 1, False), ((32, 24, 24, 24), 24, 3, 0, True), ((32, 24, 24, 24), 8, 7, 1, False),
+    ((32, 24, 24, 24), 8, 7, 0, True), ((48, 24, 24, 24), 24, 6, 1, True), ((16, 16, 16, 16), 24, 1, 0, False)])
+def test_prolongation(L, nv, nrhs, accumulate, expect):
+    assert prolong_pairs(L, A4, nv, nrhs, accumulate) == expect
+    assert not prolong_pairs(L, (2, 2, 2, 2), nv, nrhs, accumulate)
