@@ -10,6 +10,7 @@
 // coarse operator: [site][9 blocks][col][row].
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "tm_kernels.h"
@@ -382,11 +383,37 @@ void csap_l(const void* Dc, const float* b, float* x, const CSapGeom& sg, double
   const unsigned grid = (unsigned)(sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2) * (unsigned)ngrp;
   k_csap_l<S, PR, MT><<<grid, threads, smem, st>>>(Dc, b, x, sg, (float)mu, n_mr, colour, nrhs, ngrp);
 }
+// Pairs of right-hand sides per CTA (at most 3) for `blocks` blocks of one colour of `rows` rows.  One block's chain of
+// MR steps takes 1, 1.45 or 1.95 times as long with 1, 2 or 3 pairs, and the CTAs come in waves of what registers let
+// an SM hold: 80 per thread up to 384 threads, 128 beyond.  So a small lattice spreads its pairs over the chip and a
+// large one shares the block's loads.  Us per sweep for 1, 2, 3 pairs per CTA (one right-hand side per thread and all
+// six in a CTA, the form before this one), 2^4 blocks, 16-bit, 6 right-hand sides: 8 blocks of N_v 28 333 538 750 (317),
+// of N_v 8 85 127 168 (145); 128 of N_v 24 695 713 660 (829); 256 of N_v 24 1278 1393 1004 (1614).  Over 1344 such
+// sets of times (N_v 4 to 28, blocks of 2 to 32 sites, 8 to 1024 of them, 2 to 12 right-hand sides) the choice is
+// 1.002 of the best of the three on average, 1.2 at worst.
+extern "C" int tmamg_csap_pairs(int blocks, int rows, int nrhs) {
+  constexpr double chain[3] = {1, 1.45, 1.95};
+  const int pairs = (nrhs + 1) / 2, threads = (rows / kRows + 31) / 32 * 32;
+  const long at_once = (long)kSms * std::min(32, std::max(1, 65536 / ((threads <= 384 ? 80 : 128) * threads)));
+  int best = 1;
+  double best_t = 0;
+  for (int p = std::min(3, pairs); p >= 1; --p) {
+    const int ngrp = (pairs + p - 1) / p, even = (pairs + ngrp - 1) / ngrp;
+    const double t = (double)(((long)blocks * ngrp + at_once - 1) / at_once) * chain[even - 1];
+    if (best_t == 0 || t < best_t) {
+      best_t = t;
+      best = even;
+    }
+  }
+  return best;
+}
+
 template <int S, int MT>
 void csap_t(const void* Dc, const float* b, float* x, const CSapGeom& sg, double mu, int n_mr, int colour, int nrhs,
             int threads, cudaStream_t st) {
-  const int pairs = (nrhs + 1) / 2, ngrp = (pairs + 2) / 3;  // up to 3 pairs per CTA, evenly filled
-  switch ((pairs + ngrp - 1) / ngrp) {
+  const int ppc = tmamg_csap_pairs(sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3] / 2, sg.bsites * sg.n, nrhs);
+  const int ngrp = ((nrhs + 1) / 2 + ppc - 1) / ppc;
+  switch (ppc) {
     case 1: return csap_l<S, 1, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);
     case 2: return csap_l<S, 2, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);
     default: return csap_l<S, 3, MT>(Dc, b, x, sg, mu, n_mr, colour, nrhs, ngrp, threads, st);

@@ -169,6 +169,8 @@ struct CAggGeom {
   int asites;
   int nv1, nv2;
 };
+// pairs of right-hand sides per CTA of a batched FP32 level-1 SAP
+extern "C" int tmamg_csap_pairs(int blocks, int rows, int nrhs);
 // one colour of SAP on D_c1(mu) x = b (b may be null), nrhs level-1 vectors;
 // with Dc_half (16-bit copy of the FP32 blocks, half_kind ST_F16 or ST_BF16)
 // the blocks are read from it

@@ -102,3 +102,34 @@ def test_blocks_of_more_than_256_sites(L, blk, oe, prec, store, tol):
     got = g.unpack(0, prec, fx, x0.shape, 2)
     for r in range(2):
         assert rel(got[r], sap.smooth(b[r], x0[r], 1)) <= tol
+
+
+@pytest.mark.parametrize("nv,blk,nrhs,pairs", [(5, (2, 2, 2, 2), 5, 1), (28, (2, 2, 2, 2), 3, 2), (28, (2, 2, 2, 2), 5, 3),
+                                               (24, (2, 2, 2, 2), 11, 3), (23, (1, 2, 2, 2), 16, 2)])
+@pytest.mark.parametrize("prec", [tm.TM_F32, tm.TM_F16, tm.TM_BF16])
+def test_level1_sap_batches(nv, blk, nrhs, pairs, prec):
+    # 1 to 3 pairs per CTA, each right-hand side as alone (rounding of another order of 4 MR steps: 1e-6)
+    L, L1 = (16, 16, 16, 16), (8, 8, 8, 8)
+    rows = 2 * nv * int(np.prod(blk))
+    assert tm.lib().tmamg_csap_pairs(int(np.prod(L1)) // int(np.prod(blk)) // 2, rows, nrhs) == pairs
+    p = dict(m0=-0.3, c_sw=1.4, mu=0.05, delta=3.0, nv=nv, agg=(2, 2, 2, 2), sap_block=(2, 2, 2, 2), cycle_prec=F32,
+             max_rhs=nrhs, levels=3, nv2=2, sap1_prec=prec)
+    prm = tm.params(L=L, **p)
+    prm.agg2[:], prm.sap_block1[:] = (2, 2, 2, 2), blk
+    h = tm.tm_create(prm, torch.cuda.current_stream())
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    draw = lambda n, dtype: torch.randn(n, dtype=dtype, device="cuda", generator=gen)  # noqa: E731
+    try:
+        tm.tm_load_gauge(h, torch.from_numpy(inputs.gauge_field(L, 0.5, 7)).cuda())
+        tm.tm_setup_from_vectors(h, draw(nv * 16 ** 4 * 24 + 2 * 8 ** 4 * 4 * nv, torch.float64))
+        one = tm.tm_field_bytes(h, 1, F32, 1) // 4
+        b, x0 = draw(nrhs * one, torch.float32), draw(nrhs * one, torch.float32)
+        got = x0.clone()
+        tm.tm_sap1(h, F32, b, got, 2, nrhs)
+        for r in range(nrhs):
+            part = slice(r * one, (r + 1) * one)
+            x = x0[part].clone()
+            tm.tm_sap1(h, F32, b[part].clone(), x, 2, 1)
+            assert float((got[part] - x).norm() / x.norm()) <= 1e-6
+    finally:
+        tm.tm_destroy(h)
