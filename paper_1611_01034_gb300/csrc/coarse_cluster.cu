@@ -612,8 +612,12 @@ bool stream_sms(cudaStream_t st, int* sms, int* together) {
   CUcontext ctx = nullptr;
   CUgreenCtx green = nullptr;
   CUdevResource r{};
-  if (!get_ctx || !ctx_res || !green_res || get_ctx(st, &ctx, &green) != CUDA_SUCCESS ||
-      (green ? green_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) : ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM)) != CUDA_SUCCESS)
+  if (!get_ctx || !ctx_res || !green_res) return false;
+  // in a thread's first call with the default stream no context is current yet: cudaFree(0) makes it so
+  if (get_ctx(st, &ctx, &green) != CUDA_SUCCESS &&
+      (cudaFree(nullptr) != cudaSuccess || get_ctx(st, &ctx, &green) != CUDA_SUCCESS))
+    return false;
+  if ((green ? green_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) : ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM)) != CUDA_SUCCESS)
     return false;
   *sms = (int)r.sm.smCount;
   *together = (int)r.sm.smCoscheduledAlignment;

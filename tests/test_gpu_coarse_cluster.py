@@ -7,6 +7,7 @@ alone (FP64).  Short cycles, with the true residual between them, are held again
 exported D_c, and K-cycles of a batch too large for the clusters against those of one right-hand side alone.
 """
 import ctypes
+import threading
 
 import numpy as np
 import pytest
@@ -191,3 +192,14 @@ def test_stream_on_part_of_the_chip(L, nv, sms, flags):
     for (i0, x0), (i1, x1) in zip(whole, got):
         assert i0 == i1
         assert rel(x1, x0) <= 1e-9
+
+
+def test_first_call_of_a_thread_takes_one_launch():
+    # on the default stream, before anything has made the device's context current in that thread
+    g = _gpu((8, 8, 8, 8), (4, 4, 4, 4), 8, tm.TM_F32)
+    fb, fx = g.pack(1, tm.TM_F32, np.ones(g.coarse_shape())), g.field(1, tm.TM_F32)
+    tm.tm_profile(g.h, True)
+    t = threading.Thread(target=tm.tm_coarse_solve, args=(g.h, tm.TM_F32, fb, fx, 0.0, 7))
+    t.start()
+    t.join()
+    assert tm.tm_profile_read(g.h)["coarse_oe"]["launches"] == 1
