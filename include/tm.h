@@ -180,7 +180,8 @@ typedef struct {
      complement to coarse_tol / coarsest_tol with the host deciding each step;
      k in 1..64 = exactly k GMRES steps (a right-hand side whose residual
      estimate reaches the tolerance stops updating), all bookkeeping on the
-     device: for one right-hand side a single launch, else captured once as a
+     device: for one right-hand side and up to 48 steps a single launch (if its
+     vectors fit and the stream has the whole chip), else captured once as a
      CUDA graph and replayed for every later coarsest solve with the same
      buffers and twisted mass. */
   int coarsest_steps;

@@ -24,6 +24,12 @@
 //   dot            184 218 260 299 -> 100 113 124 143
 //   update + dot   290 334 391 449 -> 155 181 213 242
 //   update + norm  197 236 274 310 -> 140 163 184 208
+// From 5 vectors on the 8-wide kernels, with the loads of one element only in flight (k_pdot_partial_b<8> spills 52
+// bytes), and from 9 on updates without a reduction fused in; for k = 5, 8, 9, 16, 17, 25:
+//   dot            514 669 880 1288 1505 2145 -> 247 312 454 610 745 1040
+//   update + dot   798 1062 - - - -           -> 558 692 - - - -
+//   update         - - 354 579 614 869        -> - - 375 571 625 874
+//   update + norm  346 449 483 725 761 1041   -> 268 345 406 621 681 958
 #include "tm_kernels.h"
 #include "tm_pair.cuh"
 
